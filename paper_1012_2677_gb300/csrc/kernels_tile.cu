@@ -1059,11 +1059,14 @@ __device__ __forceinline__ double gsum(double v) {
 
 // Shared memory of the force kernel: `nbuf` tile buffers (with two, the next tile's copies are in
 // flight while the current one is computed); one for the whole-box case.
+static size_t dp_force_smem_bytes(const TileArgs& ta, int half);
+static bool dp_fits(const TileArgs& ta);
 size_t force_buffer_bytes(const TileArgs& ta, int precision, int half) {
   const bool mixed = precision == LJ_MIXED;
   return align16(tile_layout(ta, mixed, true, !mixed && (half || ta.whole)).total);
 }
 size_t force_smem_bytes(const TileArgs& ta, int precision, int nbuf, int half) {
+  if (precision != LJ_MIXED && !ta.whole) return dp_fits(ta) ? dp_force_smem_bytes(ta, half) : force_buffer_bytes(ta, precision, half);
   return (ta.whole ? 1 : (nbuf == 2 ? 2 : 1)) * force_buffer_bytes(ta, precision, half);
 }
 
@@ -1415,22 +1418,11 @@ __device__ __forceinline__ bool tile_interior(const TileInfo& ti, const TileArgs
   return ti.cx >= 1 && ti.cx <= ta.n - 2 && ti.cy >= 1 && ti.cy <= ta.n - 2 && ti.z0 >= 1 && ti.z0 + ti.Tp <= ta.n - 1;
 }
 
-// FP64 half list, by the producer warp: the sorted indices of a staged tile (the consumers put the
-// periodic images in place, as for the mixed form).
-__device__ __forceinline__ void stage_gid_warp(const TileShared& S, unsigned char* smem, const TileLayout& L,
-                                               int lane) {
-  for (int q = 0; q < S.ncell; ++q) {
-    const int a = S.offq[q], b = S.offq[q + 1], gq = S.g0[q];
-    for (int e = a + lane; e < b; e += 32) ((int*)(smem + L.gid))[e] = gq + (e - a);
-  }
-}
-
 // Image shifts of a staged tile's periodic cells by the consumer warps (warp per cell, lanes over
 // its particles): integer adds of round(L / u) to the fixed-point records.  Every writer orders its
 // writes before later bulk copies into the same bytes; the caller then waits for all consumer
 // warps (a bounded mbarrier wait, not bar.sync, so that a warp that left on a timeout cannot hold
 // the others forever).
-template <bool MIXED>
 __device__ __forceinline__ void stage_shift_consumers(const TileInfo& ti, const TileArgs& ta, const Geom& g,
                                                       const TileShared& S, unsigned char* smem, const TileLayout& L,
                                                       int consumers) {
@@ -1440,17 +1432,10 @@ __device__ __forceinline__ void stage_shift_consumers(const TileInfo& ti, const 
     cell_of_q(ti, ta.n, S.ncol, q, sx, sy, sz);
     if ((sx | sy | sz) == 0) continue;
     for (int e = S.offq[q] + lane; e < S.offq[q + 1]; e += 32) {
-      if (MIXED) {
-        uint4* r = (uint4*)(smem + L.pos) + e;
-        r->x = shift_q(r->x, sx, g);
-        r->y = shift_q(r->y, sy, g);
-        r->z = shift_q(r->z, sz, g);
-      } else {  // FP64: s L added, one rounding per staged coordinate instead of a shift per pair
-        dvec4* p = (dvec4*)(smem + L.pos) + e;
-        p->x += (double)sx * g.L;
-        p->y += (double)sy * g.L;
-        p->z += (double)sz * g.L;
-      }
+      uint4* r = (uint4*)(smem + L.pos) + e;
+      r->x = shift_q(r->x, sx, g);
+      r->y = shift_q(r->y, sy, g);
+      r->z = shift_q(r->z, sz, g);
     }
   }
   fence_proxy_async_smem();
@@ -1460,24 +1445,21 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// CW consumer warps: 8 for tiles of up to 4 cells, 12 for larger tiles (more keys per tile).
-// Forms: the mixed form with the full list and the FP64 form with the half list (the producer writes
-// the sorted indices; the consumers scatter the partners' forces with atomics).  The consumers put
-// the periodic images of a boundary tile in place before computing it.
-template <bool MIXED, bool HALF, int LANES, bool ENERGY, bool LONGLIST, int CW>
-__global__ void __launch_bounds__(pipe_threads(CW), (MIXED && CW <= 8) ? 3 : 2)
+// CW consumer warps: 8 for tiles of up to 4 cells, 12 for larger tiles (more keys per tile).  The
+// consumers put the periodic images of a boundary tile in place before computing it.
+template <int LANES, bool ENERGY, bool LONGLIST, int CW>
+__global__ void __launch_bounds__(pipe_threads(CW), CW <= 8 ? 3 : 2)
     k_force_pipe(const void* __restrict__ pos, const uint32_t* __restrict__ cs, Geom g, TileArgs ta, LJConst c,
                  const uint2* __restrict__ rows, const uint2* __restrict__ tile_list,
                  const uint16_t* __restrict__ ent, void* __restrict__ fout, double* __restrict__ part,
                  int32_t* __restrict__ status, const int* __restrict__ skip) {
-  static_assert(MIXED != HALF, "pipelined forms: mixed with the full list, FP64 with the half list");
   if (skip && *skip) return;  // a device-decided run stopped before this step
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ TileShared SS[kPipeSlots];
   __shared__ TileInfo s_ti[kPipeSlots];
   __shared__ int s_valid[kPipeSlots];  // 1: interior tile, 2: periodic tile (shifts), 0: skip, -1: abort
   __shared__ __align__(8) uint64_t full[2], ready[2], empty[2], shifted[2];
-  const TileLayout L = tile_layout(ta, MIXED, true, !MIXED && HALF);
+  const TileLayout L = tile_layout(ta, true, true, false);
   const size_t buf_bytes = align16(L.total);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -1531,7 +1513,7 @@ __global__ void __launch_bounds__(pipe_threads(CW), (MIXED && CW <= 8) ? 3 : 2)
         staged = false;
       }
       if (!staged && lane == 0 && !ok_next) atomicOr(status, LJ_ST_CELL_RANGE);
-      if (staged) stage_issue<MIXED, true>(ti, ta, pos, rows, ent, S, buf, L, &full[b], warp);
+      if (staged) stage_issue<true, true>(ti, ta, pos, rows, ent, S, buf, L, &full[b], warp);
       // bookkeeping of this producer's next tile (its slot was released with tile k - 2), then
       // the loads for the one after it
       const int64_t tn = t + 2 * stride;
@@ -1552,11 +1534,6 @@ __global__ void __launch_bounds__(pipe_threads(CW), (MIXED && CW <= 8) ? 3 : 2)
             mbar_arrive(&ready[b]);
           }
           break;
-        }
-        if (!MIXED) {  // sorted indices by this warp; they precede later bulk copies
-          stage_gid_warp(S, buf, L, lane);
-          fence_proxy_async_smem();
-          __syncwarp();
         }
       }
       if (lane == 0) {
@@ -1581,7 +1558,7 @@ __global__ void __launch_bounds__(pipe_threads(CW), (MIXED && CW <= 8) ? 3 : 2)
       if (v < 0) break;
       unsigned char* buf = smem + b * buf_bytes;
       if (v == 2) {  // periodic tile: shifts by all consumer warps, then wait for all of them
-        stage_shift_consumers<MIXED>(s_ti[slot], ta, g, SS[slot], buf, L, CW);
+        stage_shift_consumers(s_ti[slot], ta, g, SS[slot], buf, L, CW);
         __syncwarp();
         if (lane == 0) mbar_arrive(&shifted[b]);
         ok = __all_sync(0xffffffffu, mbar_wait(&shifted[b], (shpar >> b) & 1u, wait_budget())) != 0;
@@ -1592,7 +1569,7 @@ __global__ void __launch_bounds__(pipe_threads(CW), (MIXED && CW <= 8) ? 3 : 2)
         }
       }
       if (v > 0)
-        force_tile_compute<MIXED, LANES, HALF, ENERGY, false, LONGLIST, 32 * CW>(SS[slot], buf, L, rows, ent, c, g,
+        force_tile_compute<true, LANES, false, ENERGY, false, LONGLIST, 32 * CW>(SS[slot], buf, L, rows, ent, c, g,
                                                                                     fout, status, eacc, ta.list_cap);
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[b]);
@@ -1605,6 +1582,334 @@ __global__ void __launch_bounds__(pipe_threads(CW), (MIXED && CW <= 8) ? 3 : 2)
     const double tp = block_sum(eacc.pe, sh);
     __syncthreads();
     const double tv = block_sum(eacc.vir, sh);
+    if (threadIdx.x == 0) {
+      part[2 * (size_t)blockIdx.x] = tp;
+      part[2 * (size_t)blockIdx.x + 1] = tv;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// FP64 pair work on staged tiles.  The FP64 pipe takes 2 lanes per clock per SM on this part (1/64 of
+// the FP32 rate), whatever the number of active lanes, so it is given the pairs inside r_c alone and
+// full warps of them.  A warp takes a run of consecutive keys.  It first filters their rows in FP32
+// (differences of fixed-point copies, r_c^2 widened by a relative 4e-6 against the 3e-7 that the
+// quantisation and FP32 rounding can err) and queues the kept (key, partner) pairs in shared memory;
+// then each lane evaluates a contiguous share of the queue, so that at most the last pair of a lane
+// idles and a key's sum needs no shuffles.  A lane stores the partial sum of a key that began in an earlier
+// lane in its head slot, every other one in the key's slot; the key's own lane adds slot and heads in
+// lane order, so the sums do not depend on timing.  The exact r^2 < r_c^2 test is still the FP64 one.
+constexpr int kDpThreads = 128;
+constexpr int kDpWarps = kDpThreads / 32;
+constexpr int kDpQueue = 288;  // queued pairs per warp: nine a lane (the smallest that keeps four CTAs per SM)
+
+template <int NACC, bool DIRECT>
+struct DpWarp {
+  double seg[32][NACC];   // per key: the partial sum of the lane in which its run begins
+  double head[32][NACC];  // per lane: the partial sum of a run begun in an earlier lane
+  uint32_t q[kDpQueue];   // key of the warp's run << 16 | staged partner
+};
+template <int NACC>
+struct DpWarp<NACC, true> {
+  uint32_t q[kDpQueue];
+};
+
+// Shared memory of an FP64 tile: FP64 positions, fixed-point records (sorted index in w), own rows,
+// list segment, the warps' queues.
+struct DpLayout {
+  size_t xq, warp, total;
+  TileLayout L;  // pos, rows, ent as the staging helpers take them
+};
+template <int NACC, bool DIRECT>
+__host__ __device__ __forceinline__ DpLayout dp_layout(const TileArgs& ta) {
+  DpLayout D;
+  const size_t ms = (size_t)ta.max_staged;
+  D.L.pos = 0;
+  size_t o = align16(ms * 32);
+  D.xq = D.L.gid = o;
+  o += ms * 16;
+  D.L.rows = o;
+  o += align16(8 * ((size_t)ta.max_own + 2));
+  D.L.ent = D.L.cnt = o;
+  o += align16(2 * (size_t)ta.list_cap);
+  D.warp = o;
+  o += sizeof(DpWarp<NACC, DIRECT>) * kDpWarps;
+  D.total = D.L.total = align16(o);
+  return D;
+}
+
+// Wait (bounded, all threads) for a staged FP64 tile, put the periodic images in place and write the
+// fixed-point records of the staged positions (integer operations on the FP64 bits: reading the
+// records from HBM would cost 16 B per staged particle and a second array).  False on timeout.
+__device__ __forceinline__ bool dp_stage_finish(const TileInfo& ti, const TileArgs& ta, const Geom& g, TileShared& S,
+                                                unsigned char* smem, const DpLayout& D, uint64_t* bar, uint32_t& phase,
+                                                int32_t* status) {
+  bool ok = true;
+  if (threadIdx.x == 0) ok = mbar_wait(bar, phase, wait_budget());
+  ok = __syncthreads_and(ok) != 0;
+  if (!ok) {
+    if (threadIdx.x == 0) {
+      atomicOr(status, LJ_ST_TIMEOUT);
+      mbar_wait(bar, phase, kWaitBudget);  // let copies in flight land before the CTA leaves
+    }
+    __syncthreads();
+    return false;
+  }
+  phase ^= 1u;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ncol = S.ncol;
+  // a column's cells are contiguous in the sorted arrays except where z wraps: up to three runs of
+  // one image each (as stage_issue copies them)
+  const int cut0 = ti.z0 == 0 ? 1 : 0, cut1 = ti.z0 + ti.Tp == ta.n ? ncol - 1 : ncol;
+  for (int k = warp; k < 9; k += (int)(blockDim.x >> 5)) {
+    int sx, sy;
+    wrap_cell(ti.cx + k / 3 - 1, ta.n, sx);
+    wrap_cell(ti.cy + k % 3 - 1, ta.n, sy);
+#pragma unroll 1
+    for (int r = 0; r < 3; ++r) {
+      const int m0 = r == 0 ? 0 : (r == 1 ? cut0 : cut1), m1 = r == 0 ? cut0 : (r == 1 ? cut1 : ncol);
+      if (m1 <= m0) continue;
+      const int sz = r == 0 ? -1 : (r == 2 ? 1 : 0);
+      const int a = S.offq[k * ncol + m0], b = S.offq[k * ncol + m1], gq = S.g0[k * ncol + m0];
+      for (int s = a + lane; s < b; s += 32) {
+        dvec4* w = (dvec4*)(smem + D.L.pos) + s;
+        dvec4 p = *w;
+        if ((sx | sy | sz) != 0) {  // the image itself: one rounding per staged coordinate, none per pair
+          if (sx != 0) p.x += sx > 0 ? g.L : -g.L;
+          if (sy != 0) p.y += sy > 0 ? g.L : -g.L;
+          if (sz != 0) p.z += sz > 0 ? g.L : -g.L;
+          *w = p;
+        }
+        ((uint4*)(smem + D.xq))[s] =
+            make_uint4(fixq(p.x, g.qk), fixq(p.y, g.qk), fixq(p.z, g.qk), (uint32_t)(gq + (s - a)));
+      }
+    }
+  }
+  // these generic writes precede later bulk copies into the same bytes
+  fence_proxy_async_smem();
+  __syncthreads();
+  return true;
+}
+
+// The listed pairs of a staged tile's keys inside r_c (or within the filter's margin of it).
+// pair(key slot, qi, partner slot, acc) adds one pair to the key's NACC sums; done(o, acc) receives
+// the sums of own key o.  ent: the tile's segment (staged, or in HBM if it is longer).
+// DIRECT: done(o, acc) is called by the lanes themselves with each partial sum (it must add atomically).
+template <int NACC, bool DIRECT, class Pair, class Done>
+__device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigned char* smem, const DpLayout& D,
+                                              const uint16_t* ent, float cut2, int32_t* status, Pair&& pair,
+                                              Done&& done) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const uint4* sq = (const uint4*)(smem + D.xq);
+  const dvec4* sp = (const dvec4*)(smem + D.L.pos);
+  const uint2* s_rows = (const uint2*)(smem + D.L.rows) + S.row_off;
+  auto& W = ((DpWarp<NACC, DIRECT>*)(smem + D.warp))[warp];
+  const int n_own = S.own1 - S.own0;
+  const int per = min(32, (n_own + kDpWarps - 1) / kDpWarps);  // keys per warp and turn
+  for (int b0 = warp * per; b0 < n_own; b0 += kDpWarps * per) {
+    const int nk = min(per, n_own - b0);
+    double tot[NACC];  // lane k: the sums of key b0 + k
+#pragma unroll
+    for (int q = 0; q < NACC; ++q) tot[q] = 0.0;
+    int ka = 0, kb = 0, cnt = 0;  // lane k: the key's range of the queue; queued pairs
+    auto drain = [&]() {
+      __syncwarp();
+      const int c = (cnt + 31) >> 5, lo = lane * c, hi = min(lo + c, cnt);
+      double acc[NACC];
+      int kc = -1;
+      bool head = lo > 0 && lo < cnt && (W.q[lo - 1] >> 16) == (W.q[lo] >> 16);
+      dvec4 qi = make_dvec4(0.0, 0.0, 0.0, 0.0);
+      auto put = [&]() {
+        if constexpr (DIRECT) {
+          done(b0 + kc, acc);
+        } else {
+          double* dst = head ? W.head[lane] : W.seg[kc];
+#pragma unroll
+          for (int q = 0; q < NACC; ++q) dst[q] = acc[q];
+          head = false;
+        }
+      };
+      for (int t = lo; t < hi; ++t) {
+        const uint32_t w = W.q[t];
+        const int k = (int)(w >> 16);
+        if (k != kc) {
+          if (kc >= 0) put();
+          kc = k;
+          qi = sp[S.own0 + b0 + k];
+#pragma unroll
+          for (int q = 0; q < NACC; ++q) acc[q] = 0.0;
+        }
+        pair(b0 + k, qi, (int)(w & 0xffffu), acc);
+      }
+      if (kc >= 0) put();
+      __syncwarp();
+      if constexpr (!DIRECT) {
+        if (kb > ka) {
+          const int l0 = ka / c, l1 = (kb - 1) / c;
+#pragma unroll
+          for (int q = 0; q < NACC; ++q) tot[q] += W.seg[lane][q];
+          for (int l = l0 + 1; l <= l1; ++l) {
+#pragma unroll
+            for (int q = 0; q < NACC; ++q) tot[q] += W.head[l][q];
+          }
+        }
+        __syncwarp();
+      }
+      ka = kb = cnt = 0;
+    };
+    uint2 row = make_uint2(0u, 0u);
+    if (lane < nk) {
+      row = s_rows[b0 + lane];
+      row.x -= S.list_base;
+      if (row.x + row.y > S.list_len) {  // inconsistent row: record and skip
+        atomicOr(status, LJ_ST_LIST_OVERFLOW);
+        row.y = 0;
+      }
+    }
+    for (int k = 0; k < nk; ++k) {
+      const int start = (int)__shfl_sync(0xffffffffu, row.x, k), len = (int)__shfl_sync(0xffffffffu, row.y, k);
+      const uint4 qi = sq[S.own0 + b0 + k];
+      if (lane == k) ka = cnt;
+      for (int e0 = 0; e0 < len; e0 += 32) {
+        if (cnt > kDpQueue - 32) {
+          if (lane == k) kb = cnt;
+          drain();
+        }
+        const int e = e0 + lane;
+        uint32_t j = 0;
+        bool in = false;
+        if (e < len) {
+          j = ent[start + e];
+          const uint4 qj = sq[j];
+          const float dx = qdiff(qj.x, qi.x), dy = qdiff(qj.y, qi.y), dz = qdiff(qj.z, qi.z);
+          in = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < cut2;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) W.q[cnt + __popc(m & lt)] = ((uint32_t)k << 16) | j;
+        cnt += __popc(m);
+      }
+      if (lane == k) kb = cnt;
+    }
+    if (cnt > 0) drain();
+    if constexpr (!DIRECT) {
+      if (lane < nk) done(b0 + lane, tot);
+    }
+  }
+}
+
+// The FP64 comparison r^2 < r_c^2 of two non-negative values by their bit patterns (the order is the
+// same; a NaN compares as not inside), which takes no slot of the FP64 pipe.
+__device__ __forceinline__ bool inside_rc(double r2, double rc2) {
+  return __double_as_longlong(r2) < __double_as_longlong(rc2);
+}
+
+// 1/x in FP64 from the hardware approximation (rcp.approx.ftz.f64) refined by one third-order step
+// r' = r + r (e + e^2), e = 1 - x r, whose error is e^3: three FP64 operations where two Newton
+// steps take four.
+__device__ __forceinline__ double rcp_cubic64(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Force over the list in the FP64 form, tile by tile (single buffer: the copies of a tile overlap the
+// arithmetic of the SM's other three CTAs).  Bound by the FP64 pipe (77 % busy): 23 operations per pair
+// inside r_c with energies, where every listed pair (1.7 times as many) took 29 in partly idle
+// warps before.  The energies come from three sums over pairs (r^-6, r^-12, r^2) and their number.
+// 1,048,576 particles, rho 0.5, half list, energies: 2.75 -> 1.03 ms per launch (T = 4 cells per tile;
+// 3, 5 and 6 give 1.07, 1.14 and 1.05 ms); 4,000 particles 42 -> 24 us.
+template <bool HALF, bool ENERGY>
+__global__ void __launch_bounds__(kDpThreads, 4)
+    k_force_dp(const dvec4* __restrict__ pos, const uint32_t* __restrict__ cs, Geom g, TileArgs ta, LJConst c,
+               const uint2* __restrict__ rows, const uint2* __restrict__ tile_list, const uint16_t* __restrict__ ent,
+               dvec4* __restrict__ fout, double* __restrict__ part, int32_t* __restrict__ status,
+               const int* __restrict__ skip) {
+  if (skip && *skip) return;  // a device-decided run stopped before this step
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ TileShared S;
+  __shared__ __align__(8) uint64_t bar;
+  const DpLayout D = dp_layout<3, HALF>(ta);
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    fence_proxy_async_smem();
+  }
+  __syncthreads();
+  const double rc2 = c.rc2, f8c2 = 8.0 * c.eps * c.c2s, sig6 = c.sig2 * c.sig2 * c.sig2;
+  const double f24s = 24.0 * c.eps * sig6, f48s = 48.0 * c.eps * sig6 * sig6;
+  const float cut2 = c.rc2q * 1.000004f;
+  double s6 = 0.0, s12 = 0.0, s2 = 0.0;
+  int np = 0;
+  double npairs = 0.0;
+  uint32_t ph = 0;
+  const dvec4* sp = (const dvec4*)(smem + D.L.pos);
+  const uint4* sq = (const uint4*)(smem + D.xq);
+  for (int64_t t = blockIdx.x; t < ta.ntiles; t += gridDim.x) {
+    const TileInfo ti = tile_info(t, ta);
+    if (force_tile_prepare(ti, t, ta, cs, tile_list, S, status)) {
+      stage_issue<false, true>(ti, ta, pos, rows, ent, S, smem, D.L, &bar);
+      if (!dp_stage_finish(ti, ta, g, S, smem, D, &bar, ph, status)) return;
+      auto pair = [&](int, const dvec4& qi, int j, double* acc) {
+        const dvec4 qj = sp[j];
+        // the half list takes d = x_i - x_j, so that ff d is the force on the partner
+        const double dx = HALF ? qi.x - qj.x : qj.x - qi.x, dy = HALF ? qi.y - qj.y : qj.y - qi.y,
+                     dz = HALF ? qi.z - qj.z : qj.z - qi.z;
+        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+        if (inside_rc(r2, rc2)) {
+          const double ri2 = rcp_cubic64(r2);
+          const double ri4 = ri2 * ri2, ri6 = ri4 * ri2;
+          const double ff = fma(ri4 * ri4, fma(-f48s, ri6, f24s), f8c2);
+          if (HALF) {
+            dvec4* F = fout + sq[j].w;
+            const double fx = ff * dx, fy = ff * dy, fz = ff * dz;
+            acc[0] -= fx;
+            acc[1] -= fy;
+            acc[2] -= fz;
+            atomicAdd(&F->x, fx);
+            atomicAdd(&F->y, fy);
+            atomicAdd(&F->z, fz);
+          } else {
+            acc[0] = fma(ff, dx, acc[0]);
+            acc[1] = fma(ff, dy, acc[1]);
+            acc[2] = fma(ff, dz, acc[2]);
+          }
+          if (ENERGY) {
+            s6 += ri6;
+            s12 = fma(ri6, ri6, s12);
+            s2 += r2;
+            ++np;
+          }
+        }
+      };
+      auto done = [&](int o, const double* acc) {
+        dvec4* F = fout + S.gown0 + o;
+        if (HALF) {
+          atomicAdd(&F->x, acc[0]);
+          atomicAdd(&F->y, acc[1]);
+          atomicAdd(&F->z, acc[2]);
+        } else {
+          *F = make_dvec4(acc[0], acc[1], acc[2], 0.0);
+        }
+      };
+      if (S.list_len <= (unsigned)ta.list_cap)
+        dp_tile_pairs<3, HALF>(S, smem, D, (const uint16_t*)(smem + D.L.ent), cut2, status, pair, done);
+      else
+        dp_tile_pairs<3, HALF>(S, smem, D, ent + S.list_base, cut2, status, pair, done);  // a long segment stays in HBM
+      if (ENERGY) {
+        npairs += (double)np;
+        np = 0;
+      }
+    }
+    __syncthreads();
+  }
+  if (ENERGY) {
+    __shared__ double sh[32];
+    const double sig12 = sig6 * sig6;
+    const double pe = 4.0 * c.eps * fma(sig12, s12, fma(-sig6, s6, fma(c.c2s, s2, c.c0 * npairs)));
+    const double vir = fma(f48s, s12, fma(-f24s, s6, -f8c2 * s2));
+    const double tp = block_sum(pe, sh);
+    __syncthreads();
+    const double tv = block_sum(vir, sh);
     if (threadIdx.x == 0) {
       part[2 * (size_t)blockIdx.x] = tp;
       part[2 * (size_t)blockIdx.x + 1] = tv;
@@ -2057,6 +2362,44 @@ void launch_list_tile(int precision, int half, const void* pos, const float4* hi
 #undef LJ_LIST_LAUNCH
 }
 
+static size_t dp_force_smem_bytes(const TileArgs& ta, int half) {
+  return half ? dp_layout<3, true>(ta).total : dp_layout<3, false>(ta).total;
+}
+// Whether a CTA can stage the largest tile with its fixed-point records and queues (48 B per staged
+// particle and 11 KB; about 4,600 particles).  Larger tiles (36 B per particle) take k_force_tile.
+static bool dp_fits(const TileArgs& ta) {
+  int dev = 0, smem_max = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  TileArgs tz = ta;
+  tz.list_cap = 0;
+  return dp_layout<3, false>(tz).total + 2048 <= (size_t)smem_max;  // 2 KB: static shared memory
+}
+
+// The FP64 form on tiles; returns the grid launched.
+static int launch_force_dp(int half, int energy, const void* pos, const uint32_t* cs, Geom g, TileArgs ta, LJConst c,
+                           const uint2* rows, const uint2* tl, const uint16_t* ent, void* f, double* part,
+                           int32_t* status, int per_sm, cudaStream_t s, const int* skip) {
+  const size_t sm = dp_force_smem_bytes(ta, half);
+  int grid = 1;
+#define LJ_DP(H, E)                                                                                              \
+  do {                                                                                                           \
+    set_smem(k_force_dp<H, E>, sm);                                                                              \
+    grid = tile_grid(ta, per_sm > 0 ? per_sm : resident_per_sm(k_force_dp<H, E>, kDpThreads, sm));               \
+    k_force_dp<H, E><<<grid, kDpThreads, sm, s>>>((const dvec4*)pos, cs, g, ta, c, rows, tl, ent, (dvec4*)f, part, \
+                                                  status, skip);                                                 \
+  } while (0)
+  if (half) {
+    if (energy) LJ_DP(true, true);
+    else LJ_DP(true, false);
+  } else {
+    if (energy) LJ_DP(false, true);
+    else LJ_DP(false, false);
+  }
+#undef LJ_DP
+  return grid;
+}
+
 // Returns the grid launched (the number of energy partials written).
 template <bool MIXED, int LANES, bool HALF, bool ENERGY>
 static int force_w(const void* pos, const uint32_t* cs, int64_t N, Geom g, TileArgs ta, LJConst c, const uint2* rows,
@@ -2069,15 +2412,15 @@ static int force_w(const void* pos, const uint32_t* cs, int64_t N, Geom g, TileA
                                                                                     tl, ent, f, part, status, nbuf,  \
                                                                                     skip);                          \
   } while (0)
-  if constexpr (MIXED != HALF) {  // the pipelined forms: mixed + full list, FP64 + half list
+  if constexpr (MIXED && !HALF) {  // the pipelined form: mixed + full list
     if (!ta.whole && nbuf == 2) {  // producer warps + consumer warps over two buffers
 #define LJ_FP(LONG, CW)                                                                                          \
   do {                                                                                                           \
-    set_smem(k_force_pipe<MIXED, HALF, LANES, ENERGY, LONG, CW>, sm);                                            \
+    set_smem(k_force_pipe<LANES, ENERGY, LONG, CW>, sm);                                            \
     const int64_t want = (int64_t)sm_count() *                                                                   \
-                         resident_per_sm(k_force_pipe<MIXED, HALF, LANES, ENERGY, LONG, CW>, pipe_threads(CW), sm); \
+                         resident_per_sm(k_force_pipe<LANES, ENERGY, LONG, CW>, pipe_threads(CW), sm); \
     grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(want, ta.ntiles), (int64_t)kMaxRedBlocks)); \
-    k_force_pipe<MIXED, HALF, LANES, ENERGY, LONG, CW><<<grid, pipe_threads(CW), sm, s>>>(pos, cs, g, ta, c, rows, \
+    k_force_pipe<LANES, ENERGY, LONG, CW><<<grid, pipe_threads(CW), sm, s>>>(pos, cs, g, ta, c, rows, \
                                                                                        tl, ent, f, part, status,      \
                                                                                        skip);                         \
   } while (0)
@@ -2093,9 +2436,14 @@ static int force_w(const void* pos, const uint32_t* cs, int64_t N, Geom g, TileA
       return grid;
     }
   }
-  if (ta.whole) LJ_FW(true, false);
-  else if (ta.list_cap < ta.max_list) LJ_FW(false, true);  // some segments longer than the staged capacity
-  else LJ_FW(false, false);
+  if constexpr (MIXED) {
+    if (ta.whole) LJ_FW(true, false);
+    else if (ta.list_cap < ta.max_list) LJ_FW(false, true);  // some segments longer than the staged capacity
+    else LJ_FW(false, false);
+  } else {
+    if (ta.whole) LJ_FW(true, false);
+    else if constexpr (LANES == 8) LJ_FW(false, true);  // FP64 tiles beyond k_force_dp's capacity
+  }
 #undef LJ_FW
   return grid;
 }
@@ -2130,6 +2478,13 @@ int launch_force_tile(int precision, int half, int lanes, int energy, const void
                       Geom g, TileArgs ta, LJConst c, const uint2* rows, const uint2* tile_list, const uint16_t* ent,
                       void* f, double* part, int32_t* status, int per_sm, int nbuf, cudaStream_t s, const int* skip) {
   const size_t sm = force_smem_bytes(ta, precision, nbuf, half);
+  if (precision != LJ_MIXED && !ta.whole) {
+    if (!dp_fits(ta)) {
+      lanes = 8;
+      nbuf = 1;
+    } else
+      return launch_force_dp(half, energy, pos, cs, g, ta, c, rows, tile_list, ent, f, part, status, per_sm, s, skip);
+  }
   if (per_sm <= 0) per_sm = per_sm_for(sm);
   const int grid = tile_grid(ta, per_sm);
   if (precision == LJ_MIXED)

@@ -454,9 +454,9 @@ static int ensure_tile_list(ljmd_sys* s) {
 
 // Tile geometry for the staged list/force kernels: T cells along z per tile, shared-memory
 // capacities from the actual largest tile of the current cell occupancy.
-// Tile buffers per force CTA: the requested number, else two for the forms with a pipelined
+// Tile buffers per force CTA: the requested number, else two for the form with a pipelined
 // kernel (producer warps stage the next tile while consumer warps compute): the mixed form with
-// the full list and the FP64 form with the half list; one otherwise.
+// the full list; one otherwise.
 // Multiprocessors of a device (152 if the attribute cannot be read).
 static int sm_count_of(int dev) {
   int sms = 0;
@@ -470,9 +470,9 @@ static int sm_count_of(int dev) {
 static int force_buffers(const ljmd_sys* s) {
   if (s->force_nbuf) return s->force_nbuf;
   // fewer tiles than two per SM: the single-buffer kernel (the pipelined one holds one CTA per SM
-  // with two producer warps; 4,000 particles, FP64 form: 40 against 44 us per force launch)
+  // with two producer warps)
   if (s->ta.ntiles > 0 && s->ta.ntiles < 2 * (int64_t)sm_count_of(s->device)) return 1;
-  return ((s->precision == LJ_MIXED) != s->list_half) ? 2 : 1;
+  return s->precision == LJ_MIXED && !s->list_half ? 2 : 1;
 }
 
 // Default cells per tile along z.  The mixed form with the full list (the pipelined force kernel):
@@ -481,11 +481,11 @@ static int force_buffers(const ljmd_sys* s) {
 // (13.8 particles per cell), T = 4, 8, 10, 12 give force launches of 2.41, 2.09, 1.96, 1.88 ms and
 // list constructions of 11.7, 14.0, 13.2, 13.2 ms, and T = 12 the shortest step.  The half-list
 // forms keep 4 cells: at rho 0.8 (mixed, half list) T = 3, 4, 6 give force 3.76, 3.56, 4.06 ms and
-// construction 19.0, 19.8, 33.7 ms; the FP64 form at rho 0.5 gives force 45.5 ms at T = 4 and
-// 49.4 ms at T = 10 with 2 lanes.
+// construction 19.0, 19.8, 33.7 ms; the FP64 form at 1M particles, rho 0.5, gives force 1.07, 1.03,
+// 1.14, 1.05 ms at T = 3, 4, 5, 6.
 // Small boxes: the tile length is lowered until there are at least two tiles per SM, so that the
 // force launch spreads over the GPU (4,000 particles, 6 cells per side, FP64 form: T = 4, 2, 1 give
-// 72, 108, 216 tiles and force launches of 69, 40, 39 us).
+// 72, 108, 216 tiles and force launches of 40, 29, 24 us).
 static int default_tile_cells(const ljmd_sys* s) {
   int T = 4;
   if (s->precision == LJ_MIXED && !s->list_half) {
@@ -636,11 +636,14 @@ static int rebuild(ljmd_sys* s) {
     // the force kernel stages a tile's list segment if it fits; longer segments are read from HBM
     TileArgs tz = s->ta;
     tz.list_cap = 0;
-    const size_t base_bytes = std::max(force_smem_bytes(tz, s->precision, force_buffers(s), 1),
+    const size_t base_bytes = std::max(force_smem_bytes(tz, s->precision, force_buffers(s), half),
                                        adjoint_smem_bytes(tz, s->precision));
     const int nbuf = s->ta.whole ? 1 : force_buffers(s);
-    if (base_bytes <= (size_t)smem_max) {
-      int64_t room = ((int64_t)smem_max - (int64_t)base_bytes) / (2 * nbuf) - 16;
+    // static shared memory (bookkeeping of two staged tiles, 1.2 KB each, or of four in the pipelined
+    // kernel) comes out of the same limit
+    const int64_t smem_dyn = (int64_t)smem_max - (nbuf == 2 ? 5376 : 2816);
+    if ((int64_t)base_bytes <= smem_dyn) {
+      int64_t room = (smem_dyn - (int64_t)base_bytes) / (2 * nbuf) - 16;
       // The pipelined kernel of the mixed form with the full list runs 3 CTAs per SM with 8
       // consumer warps (T <= 4) and 2 with 12: the staged segments are capped so that this many
       // fit in an SM's shared memory (1 KB reserved and at most 6 KB of static shared memory per
