@@ -140,7 +140,7 @@ def source_sha(path):
 
 
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_force_pipe_fcc1m_rho0.5.md")
-FORCE_SOURCE = os.path.join(ROOT, "paper_1012_2677_gb300", "csrc", "kernels_tile.cu")
+FORCE_SOURCE = os.path.join(ROOT, "paper_1012_2677_gb300", "csrc", "kernels_force.cu")
 
 
 def recorded_traffic(kernel_name, N):

@@ -154,6 +154,28 @@ int launch_force_tile(int precision, int half, int lanes, int energy, const void
                       Geom g, TileArgs ta, LJConst c, const uint2* rows, const uint2* tile_list, const uint16_t* ent,
                       void* f, double* part, int32_t* status, int per_sm, int nbuf, cudaStream_t s,
                       const int* skip = nullptr);
+// What launch_force_tile hands to the translation unit of a form.
+struct ForceLaunch {
+  const void* pos;
+  const uint32_t* cs;
+  int64_t N;
+  Geom g;
+  TileArgs ta;
+  LJConst c;
+  const uint2 *rows, *tile_list;
+  const uint16_t* ent;
+  void* f;
+  double* part;
+  int32_t* status;
+  const int* skip;
+  int lanes, energy, per_sm, nbuf, grid;
+  size_t smem;
+  cudaStream_t s;
+};
+void launch_force_mixed_half(const ForceLaunch& a);
+int launch_force_fp64(int half, ForceLaunch& a);  // returns the grid launched
+size_t dp_force_smem_bytes(const TileArgs& ta, int half);
+bool dp_fits(const TileArgs& ta);
 size_t adjoint_smem_bytes(const TileArgs& ta, int precision);
 // Adjoint pass (HVP, forces, parameter derivatives) over the list; w, hw, fo are dvec4 [N] in sorted
 // order (fo may be null), wf the FP32 copy of w (read by the mixed form).  Writes 5 partials per
@@ -269,6 +291,9 @@ void launch_load_batch(const double* xin, const double* vin, double* x, double* 
 // ---- list validity (kernels_tile.cu) --------------------------------------------------------
 // Budget of the bounded device waits of the tile kernels (0: default); 0 on success.
 int set_wait_budget(long long cycles);
+int set_wait_budget_force(long long cycles);
+int set_wait_budget_force_half(long long cycles);
+int set_wait_budget_force_dp(long long cycles);
 void launch_ldc_collect(const double* x, const double* xref, int64_t N, double th2, int32_t* list, unsigned int cap,
                         unsigned int* count, cudaStream_t s);
 void launch_ldc_pairs(const double* x, const double* xref, int64_t N, Geom g, const int32_t* list, int m, double rs2,
