@@ -324,7 +324,8 @@ int ljmd_get_stats(ljmd_sys* sys, ljmd_stats* out);
 /*
  * Turn per-phase timing on (enable = 1, resets the accumulators) or off (0).  While on, CUDA
  * events are recorded on the handle's stream around every force, integrate, rebuild, energy and
- * adjoint launch; the kernels themselves are unchanged.
+ * adjoint launch, and steps are taken as separate launches (ljmd_step otherwise advances a box whose
+ * tiles all fit on the chip many steps in one launch).
  */
 int ljmd_set_profiling(ljmd_sys* sys, int32_t enable);
 

@@ -25,78 +25,34 @@ __global__ void __launch_bounds__(kDpThreads, 4)
     fence_proxy_async_smem();
   }
   __syncthreads();
-  const double rc2 = c.rc2, f8c2 = 8.0 * c.eps * c.c2s, sig6 = c.sig2 * c.sig2 * c.sig2;
-  const double f24s = 24.0 * c.eps * sig6, f48s = 48.0 * c.eps * sig6 * sig6;
-  const float cut2 = c.rc2q * 1.000004f;
-  double s6 = 0.0, s12 = 0.0, s2 = 0.0;
-  int np = 0;
+  DpForce<HALF, ENERGY> body(c, smem, D, fout);
   double npairs = 0.0;
   uint32_t ph = 0;
-  const dvec4* sp = (const dvec4*)(smem + D.L.pos);
-  const uint4* sq = (const uint4*)(smem + D.xq);
   for (int64_t t = blockIdx.x; t < ta.ntiles; t += gridDim.x) {
     const TileInfo ti = tile_info(t, ta);
     if (force_tile_prepare(ti, t, ta, cs, tile_list, S, status)) {
       stage_issue<false, true>(ti, ta, pos, rows, ent, S, smem, D.L, &bar);
       if (!dp_stage_finish(ti, ta, g, S, smem, D, &bar, ph, status)) return;
-      auto pair = [&](int, const dvec4& qi, int j, double* acc) {
-        const dvec4 qj = sp[j];
-        // the half list takes d = x_i - x_j, so that ff d is the force on the partner
-        const double dx = HALF ? qi.x - qj.x : qj.x - qi.x, dy = HALF ? qi.y - qj.y : qj.y - qi.y,
-                     dz = HALF ? qi.z - qj.z : qj.z - qi.z;
-        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        if (inside_rc(r2, rc2)) {
-          const double ri2 = rcp_cubic64(r2);
-          const double ri4 = ri2 * ri2, ri6 = ri4 * ri2;
-          const double ff = fma(ri4 * ri4, fma(-f48s, ri6, f24s), f8c2);
-          if (HALF) {
-            dvec4* F = fout + sq[j].w;
-            const double fx = ff * dx, fy = ff * dy, fz = ff * dz;
-            acc[0] -= fx;
-            acc[1] -= fy;
-            acc[2] -= fz;
-            atomicAdd(&F->x, fx);
-            atomicAdd(&F->y, fy);
-            atomicAdd(&F->z, fz);
-          } else {
-            acc[0] = fma(ff, dx, acc[0]);
-            acc[1] = fma(ff, dy, acc[1]);
-            acc[2] = fma(ff, dz, acc[2]);
-          }
-          if (ENERGY) {
-            s6 += ri6;
-            s12 = fma(ri6, ri6, s12);
-            s2 += r2;
-            ++np;
-          }
-        }
-      };
+      auto pair = [&](int, const dvec4& qi, int j, double* acc) { body.pair(qi, j, acc); };
       auto done = [&](int o, const double* acc) {
-        dvec4* F = fout + S.gown0 + o;
-        if (HALF) {
-          atomicAdd(&F->x, acc[0]);
-          atomicAdd(&F->y, acc[1]);
-          atomicAdd(&F->z, acc[2]);
-        } else {
-          *F = make_dvec4(acc[0], acc[1], acc[2], 0.0);
-        }
+        if (HALF) body.add(S.gown0 + o, acc);
+        else fout[S.gown0 + o] = make_dvec4(acc[0], acc[1], acc[2], 0.0);
       };
       if (S.list_len <= (unsigned)ta.list_cap)
-        dp_tile_pairs<3, HALF>(S, smem, D, (const uint16_t*)(smem + D.L.ent), cut2, status, pair, done);
+        dp_tile_pairs<3, HALF>(S, smem, D, (const uint16_t*)(smem + D.L.ent), body.cut2, status, pair, done);
       else
-        dp_tile_pairs<3, HALF>(S, smem, D, ent + S.list_base, cut2, status, pair, done);  // a long segment stays in HBM
+        dp_tile_pairs<3, HALF>(S, smem, D, ent + S.list_base, body.cut2, status, pair, done);  // a long segment stays in HBM
       if (ENERGY) {
-        npairs += (double)np;
-        np = 0;
+        npairs += (double)body.np;
+        body.np = 0;
       }
     }
     __syncthreads();
   }
   if (ENERGY) {
     __shared__ double sh[32];
-    const double sig12 = sig6 * sig6;
-    const double pe = 4.0 * c.eps * fma(sig12, s12, fma(-sig6, s6, fma(c.c2s, s2, c.c0 * npairs)));
-    const double vir = fma(f48s, s12, fma(-f24s, s6, -f8c2 * s2));
+    double pe, vir;
+    dp_energies(c, body.s6, body.s12, body.s2, npairs, pe, vir);
     const double tp = block_sum(pe, sh);
     __syncthreads();
     const double tv = block_sum(vir, sh);

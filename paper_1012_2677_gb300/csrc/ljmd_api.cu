@@ -2,6 +2,7 @@
 // orchestration of the hot path.  Every step of the computation runs in the kernels of the
 // other translation units; this file only sizes buffers, launches and reads back scalars.
 #include <math.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -79,6 +80,15 @@ struct ljmd_sys {
   double* cap_x = nullptr;
   int64_t cap_step0 = 0;
   StepCtl* h_ctl = nullptr;     // pinned mirror
+  // resident runs (allocated on first use): threads per key (0: the tiles do not fit at once), control
+  // block and its pinned mirror, second position buffer, energy partials of a run's states
+  int res_lanes = 0;
+  TileArgs res_ta{};
+  ResidentCtl *d_res = nullptr, *h_res = nullptr;
+  void* pos_alt = nullptr;
+  int64_t pos_alt_cap = 0;
+  double *res_rec = nullptr, *part_force2 = nullptr;
+  int64_t res_rec_cap = 0;
   int64_t last_build_step = 0;  // sys->steps at the last list construction
   int64_t lifetime_est = 16;    // steps the last list lived (sizes the next device-decided run)
   unsigned long long* d_total64 = nullptr;
@@ -152,7 +162,8 @@ static void free_all(ljmd_sys* s) {
                   s->id_alt, s->img, s->img_alt, s->cell_of, s->perm, s->perm_id, s->cell_count, s->cell_start,
                   s->cell_fill, s->rows, s->tile_list, s->ent, s->scan_tmp, s->part_force, s->part_ke,
                   s->part_misc, s->d_scalars, s->d_energies, s->d_log_count, s->d_status, s->d_dmax, s->d_ctl, s->d_ticket, s->d_total64, s->d_sizes,
-                  s->adj_w, s->adj_hw, s->adj_f, s->adj_wf, s->adj_ticket, s->part_adj, s->d_adj, s->xref64, s->ldc_list, s->d_ldc};
+                  s->adj_w, s->adj_hw, s->adj_f, s->adj_wf, s->adj_ticket, s->part_adj, s->d_adj, s->xref64, s->ldc_list, s->d_ldc,
+                  s->d_res, s->pos_alt, s->res_rec, s->part_force2};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto& p : s->ev_pending) {
@@ -164,6 +175,7 @@ static void free_all(ljmd_sys* s) {
   if (s->h_f64) cudaFreeHost(s->h_f64);
   if (s->h_i32) cudaFreeHost(s->h_i32);
   if (s->h_ctl) cudaFreeHost(s->h_ctl);
+  if (s->h_res) cudaFreeHost(s->h_res);
 }
 
 enum { PH_FORCE = 0, PH_INTEGRATE = 1, PH_REBUILD = 2, PH_ENERGY = 3, PH_ADJOINT = 4 };
@@ -667,6 +679,9 @@ static int rebuild(ljmd_sys* s) {
   }
   s->list_entries = total;
   s->have_list = true;
+  s->res_ta = s->ta;
+  s->res_ta.list_cap = s->ta.max_list;  // a resident run keeps every segment in shared memory
+  s->res_lanes = resident_lanes(s->precision, half, s->res_ta, N);
   if (s->rebuilds > 0 && s->steps > s->last_build_step) s->lifetime_est = s->steps - s->last_build_step;
   s->last_build_step = s->steps;
   s->rebuilds += 1;
@@ -914,6 +929,117 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
   return LJ_OK;
 }
 
+static int ensure_resident(ljmd_sys* s) {
+  const size_t psz = s->precision == LJ_MIXED ? 16 : 32;
+  if (!s->d_res) TRY(dalloc_t(s, &s->d_res, 1));
+  if (!s->h_res && cudaMallocHost(&s->h_res, sizeof(ResidentCtl)) != cudaSuccess) {
+    s->h_res = nullptr;
+    cudaGetLastError();
+    return LJ_ENOMEM;
+  }
+  if (!s->part_force2) TRY(dalloc_t(s, &s->part_force2, 2 * kMaxRedBlocks));
+  if (s->pos_alt_cap < s->n) {
+    TRY(dalloc(s, &s->pos_alt, psz * (size_t)s->n));
+    s->pos_alt_cap = s->n;
+  }
+  const int64_t want = 3 * (int64_t)(kResidentSteps + 1) * s->ta.ntiles;
+  if (s->res_rec_cap < want) {
+    TRY(dalloc_t(s, &s->res_rec, (size_t)want));
+    s->res_rec_cap = want;
+  }
+  return LJ_OK;
+}
+
+// Up to `remaining` steps as one resident run (kernels_resident.cu), with the final half kick of the
+// call if it gets to its end (*finished).  *advanced and *stopped as device_run; *launched = false: the
+// device cannot hold the grid now and nothing was done.
+static int resident_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remaining, int64_t* advanced,
+                        bool* stopped, bool* finished, bool* launched) {
+  ljmd_sys* sys = s;
+  cudaStream_t st = s->st;
+  TRY(ensure_resident(s));
+  const int ee = s->prm.energy_every;
+  auto want_energy = [&](int64_t t) { return ee > 0 && (t % ee) == 0; };
+  const int K = (int)std::min<int64_t>(remaining, kResidentSteps);
+  ResidentCtl* hc = s->h_res;
+  const size_t head = offsetof(ResidentCtl, dmax);
+  memset(hc, 0, head + sizeof(hc->dmax[0]) * (size_t)K);
+  hc->stop_at = -1;
+  hc->dutc = s->dutc_buffer;
+  CK(cudaMemcpyAsync(s->d_res, hc, head + sizeof(hc->dmax[0]) * (size_t)K, cudaMemcpyHostToDevice, st));
+  ResidentArgs a{};
+  a.ta = s->res_ta;
+  a.g = s->g;
+  a.c = s->c;
+  a.cs = s->cell_start;
+  a.rows = s->rows;
+  a.tile_list = s->tile_list;
+  a.ent = s->ent;
+  a.x = s->x;
+  a.v = s->v;
+  a.f = s->f;
+  a.pos = force_pos(s);
+  a.pos_alt = s->pos_alt;
+  a.ref = s->ref;
+  a.id = s->id;
+  a.img = s->img;
+  a.N = s->n;
+  a.step0 = s->steps;
+  a.K = K;
+  a.first = first_of_call ? 1 : 0;
+  a.last = K == remaining ? 1 : 0;
+  a.need_force = !s->forces_current || (want_energy(s->steps) && s->pe_step != s->steps) ? 1 : 0;
+  a.dt = dt;
+  a.ee = ee;
+  a.rec0 = want_energy(s->steps) ? 1 : 0;
+  a.part_in = s->part_force;
+  a.nbf = s->nb_force;
+  a.part_out = s->part_force2;
+  a.pe_scale = s->list_half ? 1.0 : 0.5;
+  a.rec = s->res_rec;
+  a.energies = s->d_energies;
+  a.log = s->log_ptr;
+  a.log_cap = s->log_cap;
+  a.count = s->d_log_count;
+  a.ctl = s->d_res;
+  a.disp_limit = s->disp_limit;
+  a.two_dt = 2.0 * fabs(dt);
+  a.limit2_lo = s->disp_limit > 0.0 ? (float)(s->disp_limit * s->disp_limit * (1.0 - 1e-5)) : -1.0f;
+  a.dutc_rule = s->valid_mode == LJ_VALID_DUTC ? 1 : 0;
+  a.status = s->d_status;
+  a.cap_x = s->cap_x;
+  a.cap_step0 = s->cap_step0;
+  const int r = launch_resident(s->precision, s->list_half ? 1 : 0, s->res_lanes, a, st);
+  *launched = r == 0;
+  if (r > 0) {
+    cudaGetLastError();
+    return LJ_OK;
+  }
+  CKL();
+  s->launches += 1;
+  CK(cudaMemcpyAsync(hc, s->d_res, head, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  if (hc->abort) return LJ_EDEVICE;  // a wait ran out (recorded in the status word)
+  *stopped = hc->stop != 0;
+  const int64_t done = *stopped ? (int64_t)hc->stop_at + 1 : K;
+  *finished = !*stopped && a.last;
+  for (int64_t k = 0; k < done + (*finished ? 1 : 0); ++k)
+    if (want_energy(s->steps + k)) s->energy_step = s->steps + k;
+  s->steps += done;
+  *advanced = done;
+  s->last_dmax = sqrt((double)hc->last[0]);
+  if (a.dutc_rule) s->last_vmax = sqrt((double)hc->last[1]);
+  s->dutc_buffer = hc->dutc;
+  s->forces_current = !*stopped;
+  s->pe_step = -1;
+  if (!*stopped && want_energy(s->steps)) {
+    std::swap(s->part_force, s->part_force2);
+    s->nb_force = (int)s->ta.ntiles;
+    s->pe_step = s->steps;
+  }
+  return LJ_OK;
+}
+
 static int step_steps(ljmd_sys* sys, double dt, int64_t nsteps);
 
 // ----------------------------------------------------------------------------------------------
@@ -1141,13 +1267,31 @@ int ljmd_step(ljmd_sys* sys, double dt, int64_t nsteps) {
 static int step_steps(ljmd_sys* sys, double dt, int64_t nsteps) {
   const int ee = sys->prm.energy_every;
   auto want_energy = [&](int64_t t) { return ee > 0 && (t % ee) == 0; };
-  TRY(ensure_forces(sys, want_energy(sys->steps)));
   const double h = 0.5 * dt;
   cudaStream_t st = sys->st;
   // The margin/2 and DUTC rules are decided on the device (device_run); the rules with the large
   // displacement check need the host between steps.
   const bool on_device = sys->valid_mode == LJ_VALID_HALF_MARGIN || sys->valid_mode == LJ_VALID_DUTC;
+  // Boxes whose tiles all fit on the chip take their steps in resident runs (not while phases are timed,
+  // which are launches of their own).
+  if (!sys->have_list) TRY(rebuild(sys));
+  bool resident = on_device && !sys->profiling;
+  if (!resident || !sys->res_lanes) TRY(ensure_forces(sys, want_energy(sys->steps)));
   for (int64_t s = 0; s < nsteps;) {
+    if (resident && sys->res_lanes) {
+      int64_t advanced = 0;
+      bool stopped = false, finished = false, launched = false;
+      TRY(resident_run(sys, dt, s == 0, nsteps - s, &advanced, &stopped, &finished, &launched));
+      if (launched) {
+        s += advanced;
+        if (finished) return LJ_OK;
+        if (stopped) TRY(rebuild(sys));  // the drift of the last step expired the list
+        if (!sys->res_lanes) TRY(ensure_forces(sys, want_energy(sys->steps)));
+        continue;
+      }
+      resident = false;
+      TRY(ensure_forces(sys, want_energy(sys->steps)));
+    }
     if (on_device) {
       int64_t advanced = 0;
       bool stopped = false;
@@ -1184,6 +1328,7 @@ static int step_steps(ljmd_sys* sys, double dt, int64_t nsteps) {
     s += 1;
   }
   // final half-kick: v at the full step of the last state
+  TRY(ensure_forces(sys, want_energy(sys->steps)));
   const bool rec = sys->pe_step == sys->steps && want_energy(sys->steps);
   IntegrateArgs a{h, 0.0, 0.0, rec ? 1 : 0, 0};
   const int nb = integrate(sys, a);

@@ -240,6 +240,56 @@ struct StepCtl {
   float last[2];    // squared largest displacement and drift speed of the last checked step
   double dutc;      // DUTC buffer length
 };
+// ---- resident runs (kernels_resident.cu) ---------------------------------------------------
+// Control block of one run, cleared by the host before it (the header and the K slots used).
+constexpr int kResidentSteps = 256;  // steps of one run, at most
+struct ResidentCtl {
+  int stop, stop_at;      // as StepCtl
+  float last[2];
+  double dutc;
+  unsigned arrived;       // CTAs that arrived at the grid barriers so far
+  int abort;              // a CTA gave up
+  unsigned dmax[kResidentSteps][2];  // float bits: squared displacement and drift speed of each step
+};
+struct ResidentArgs {
+  TileArgs ta;
+  Geom g;
+  LJConst c;
+  const uint32_t* cs;
+  const uint2 *rows, *tile_list;
+  const uint16_t* ent;
+  double *x, *v;
+  void* f;
+  void *pos, *pos_alt;    // the force kernels' position copies and a second buffer of that size
+  const void* ref;
+  const int32_t *id, *img;
+  int64_t N, step0;       // state index before the run
+  int K, first, last;     // steps; first of the call (no half kick pending); take the final half kick
+  int need_force;         // the force of the first state is not current: compute it first
+  double dt;
+  int ee, rec0;           // energies every ee-th step; record the first state
+  const double* part_in;  // PE and virial partials of the first state [nbf] (unless need_force)
+  int nbf;
+  double* part_out;       // those of the last state, one per tile
+  double pe_scale;
+  double* rec;            // [K + 1][tiles][3]: PE, virial and KE partials
+  double *energies, *log;
+  int64_t log_cap;
+  int64_t* count;
+  ResidentCtl* ctl;
+  double disp_limit, two_dt;
+  float limit2_lo;        // squared displacements up to this are valid without the exact comparison
+  int dutc_rule;
+  int32_t* status;
+  double* cap_x;          // capture of the unwrapped states, as launch_unwrapped (or null)
+  int64_t cap_step0;
+};
+// Threads per key of a resident run of these tiles, 0 if they do not all fit on the chip at once.
+int resident_lanes(int precision, int half, const TileArgs& ta, int64_t N);
+// 0: launched; 1: the device cannot hold the grid now; -1: error.
+int launch_resident(int precision, int half, int lanes, ResidentArgs a, cudaStream_t s);
+int set_wait_budget_resident(long long cycles);
+
 // ---- pair export through a static device scratch array (no allocation) ----------------
 // Address of this device's scratch (resolved once per device): the kept-pair counter word and
 // LJ_PAIRS_STATIC_MAX_ENTRIES 64-bit key slots.

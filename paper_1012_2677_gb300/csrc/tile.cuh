@@ -1076,6 +1076,75 @@ __device__ __forceinline__ double rcp_cubic64(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
+// One pair of the FP64 form's force, its sums over pairs (r^-6, r^-12, r^2 and their number, from which
+// the energies come) and the scattered sums of the half list.
+template <bool HALF, bool ENERGY>
+struct DpForce {
+  double rc2, f8c2, f24s, f48s;
+  float cut2;
+  double s6 = 0.0, s12 = 0.0, s2 = 0.0;
+  int np = 0;
+  const dvec4* sp;
+  const uint4* sq;
+  dvec4* fout;
+  __device__ __forceinline__ DpForce(const LJConst& c, const unsigned char* smem, const DpLayout& D, dvec4* f) {
+    const double sig6 = c.sig2 * c.sig2 * c.sig2;
+    rc2 = c.rc2;
+    f8c2 = 8.0 * c.eps * c.c2s;
+    f24s = 24.0 * c.eps * sig6;
+    f48s = 48.0 * c.eps * sig6 * sig6;
+    cut2 = c.rc2q * 1.000004f;
+    sp = (const dvec4*)(smem + D.L.pos);
+    sq = (const uint4*)(smem + D.xq);
+    fout = f;
+  }
+  __device__ __forceinline__ void pair(const dvec4& qi, int j, double* acc) {
+    const dvec4 qj = sp[j];
+    // the half list takes d = x_i - x_j, so that ff d is the force on the partner
+    const double dx = HALF ? qi.x - qj.x : qj.x - qi.x, dy = HALF ? qi.y - qj.y : qj.y - qi.y,
+                 dz = HALF ? qi.z - qj.z : qj.z - qi.z;
+    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+    if (!inside_rc(r2, rc2)) return;
+    const double ri2 = rcp_cubic64(r2);
+    const double ri4 = ri2 * ri2, ri6 = ri4 * ri2;
+    const double ff = fma(ri4 * ri4, fma(-f48s, ri6, f24s), f8c2);
+    if (HALF) {
+      dvec4* F = fout + sq[j].w;
+      const double fx = ff * dx, fy = ff * dy, fz = ff * dz;
+      acc[0] -= fx;
+      acc[1] -= fy;
+      acc[2] -= fz;
+      atomicAdd(&F->x, fx);
+      atomicAdd(&F->y, fy);
+      atomicAdd(&F->z, fz);
+    } else {
+      acc[0] = fma(ff, dx, acc[0]);
+      acc[1] = fma(ff, dy, acc[1]);
+      acc[2] = fma(ff, dz, acc[2]);
+    }
+    if (ENERGY) {
+      s6 += ri6;
+      s12 = fma(ri6, ri6, s12);
+      s2 += r2;
+      ++np;
+    }
+  }
+  __device__ __forceinline__ void add(int64_t i, const double* acc) const {
+    dvec4* F = fout + i;
+    atomicAdd(&F->x, acc[0]);
+    atomicAdd(&F->y, acc[1]);
+    atomicAdd(&F->z, acc[2]);
+  }
+};
+
+// PE and virial from the sums over pairs: V = 4 eps (sigma^12 r^-12 - sigma^6 r^-6 + c2 r^2 / sigma^2 + c0).
+__device__ __forceinline__ void dp_energies(const LJConst& c, double s6, double s12, double s2, double n, double& pe,
+                                            double& vir) {
+  const double sig6 = c.sig2 * c.sig2 * c.sig2, sig12 = sig6 * sig6;
+  pe = 4.0 * c.eps * fma(sig12, s12, fma(-sig6, s6, fma(c.c2s, s2, c.c0 * n)));
+  vir = c.eps * fma(48.0 * sig12, s12, fma(-24.0 * sig6, s6, -8.0 * c.c2s * s2));
+}
+
 // ---------------------------------------------------------------------------------------------
 // Launch shapes.
 static inline int sm_count() {

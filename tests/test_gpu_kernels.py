@@ -2,6 +2,7 @@
 (tolerances of the other parity tests: FP64 forces 1e-11 of rms(F), energies 1e-12)."""
 import numpy as np
 import pytest
+import torch
 
 import oracle as O
 from paper_1012_2677_gb300 import ljmd, synth
@@ -29,3 +30,46 @@ def test_fp64_tiles(M, rho, rc, margin, list_form):
     rms = np.sqrt((F ** 2).sum(1).mean())
     assert np.sqrt(((gf - F) ** 2).sum(1)).max() / rms <= 1e-11
     assert gpe == pytest.approx(pe, rel=1e-12) and gvir == pytest.approx(vir, rel=1e-12)
+
+
+@pytest.mark.parametrize("precision,list_form", [(ljmd.LJ_MIXED, ljmd.LJ_LIST_FULL), (ljmd.LJ_MIXED, ljmd.LJ_LIST_HALF),
+                                                 (ljmd.LJ_FP64, ljmd.LJ_LIST_FULL), (ljmd.LJ_FP64, ljmd.LJ_LIST_HALF)])
+@pytest.mark.parametrize("M,rho,every,mode,steps", [
+    (5, 0.4, 1, ljmd.LJ_VALID_HALF_MARGIN, (7, 33)),   # 3 cells per side; a second call continues the first
+    (8, 0.6, 3, ljmd.LJ_VALID_HALF_MARGIN, (40,)),     # energies every third step
+    (9, 0.9, 0, ljmd.LJ_VALID_DUTC, (1, 39)),          # dense, the DUTC rule, no energies; a single step
+    (6, 0.5, 1, ljmd.LJ_VALID_HALF_MARGIN, (300,)),    # more steps than one run takes
+])
+def test_resident_run_matches_separate_launches(M, rho, every, mode, steps, precision, list_form):
+    """A box whose tiles fit on the chip takes its steps in one launch; with the phase timers on, the same
+    steps are separate launches.  Positions agree to the drift that one rounding of every force makes in 40
+    steps (dt^2 40^2 / 2 times 1e-5 of rms(F) < 50 in the mixed form, 1e-11 in the FP64 form), the energy
+    logs have the same records; after 300 steps the energies agree to the drift test's scale."""
+    out = []
+    for timed in (False, True):
+        log = torch.zeros((400, 4), dtype=torch.float64, device="cuda")
+        with ljmd.System(cutoff=2.5, margin=0.4, precision=precision, list_form=list_form, energy_every=every) as s:
+            s.init_lattice(M, rho, 1.1, 7)
+            s.set_validity(mode)
+            s.set_energy_log(log)
+            s.set_profiling(timed)
+            for k in steps:
+                s.step(0.004, k)
+            x, v, _, img = s.get_state()
+            st = s.stats()
+            out.append((x + img * s.box, v, st, log.cpu().numpy(), s.energies()))
+    (xa, va, sa, la, ea), (xb, vb, sb, lb, eb) = out
+    assert sa["steps"] == sb["steps"] == sum(steps) and sa["status_word"] == sb["status_word"] == 0
+    assert sa["kernel_launches"] < sb["kernel_launches"]
+    assert np.array_equal(la[:, 0], lb[:, 0])
+    n = np.count_nonzero(lb[:, 1])
+    if sum(steps) <= 40:
+        tol = 8e-6 if precision == ljmd.LJ_MIXED else 8e-12
+        assert np.abs(xa - xb).max() <= tol
+        assert sa["rebuilds"] == sb["rebuilds"]
+        etol = 1e-6 if precision == ljmd.LJ_MIXED else 1e-11
+        assert np.allclose(la[:n, 1:], lb[:n, 1:], rtol=etol, atol=etol * np.abs(lb[:n, 1:]).max() if n else 0)
+    else:
+        tot = lambda l: l[:n, 1] + l[:n, 2]  # noqa: E731
+        assert np.abs(tot(la) - tot(lb)).max() <= 1e-3 * np.abs(lb[:n, 1]).max()
+    assert ea[0] == pytest.approx(eb[0], rel=1e-2 if sum(steps) > 40 else 1e-5)
