@@ -295,13 +295,18 @@ constexpr long long kWaitBudget = 4000000000LL;  // ~2 s at 2 GHz: a wait that l
 
 // Wait for phase `parity` of bar to complete, giving up after `budget` clock cycles (false).  A
 // budget below the default also drops the suspend hint, so that a short budget is not outlasted
-// by one suspended try_wait.
+// by one suspended try_wait, and holds for a phase found complete too late (a cold instruction cache
+// can let the copies land before the first look).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long budget) {
-  const uint32_t hint = budget < kWaitBudget ? 0u : 1000000u;
+  const bool brief = budget < kWaitBudget;
+  const uint32_t hint = brief ? 0u : 1000000u;
   const long long t0 = clock64();
-  while (!mbar_test(bar, parity, hint))
+  for (;;) {
+    const bool done = mbar_test(bar, parity, hint);
+    if (done && !brief) return true;
     if (clock64() - t0 > budget) return false;
-  return true;
+    if (done) return true;
+  }
 }
 
 }  // namespace ljmd

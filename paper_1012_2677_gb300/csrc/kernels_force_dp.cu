@@ -38,10 +38,8 @@ __global__ void __launch_bounds__(kDpThreads, 4)
         if (HALF) body.add(S.gown0 + o, acc);
         else fout[S.gown0 + o] = make_dvec4(acc[0], acc[1], acc[2], 0.0);
       };
-      if (S.list_len <= (unsigned)ta.list_cap)
-        dp_tile_pairs<3, HALF>(S, smem, D, (const uint16_t*)(smem + D.L.ent), body.cut2, status, pair, done);
-      else
-        dp_tile_pairs<3, HALF>(S, smem, D, ent + S.list_base, body.cut2, status, pair, done);  // a long segment stays in HBM
+      dp_tile_pairs<3, HALF>(S, smem, D, (const uint16_t*)(smem + D.L.ent), ent + S.list_base, (unsigned)ta.list_cap,
+                             body.cut2, status, pair, done);
       if (ENERGY) {
         npairs += (double)body.np;
         body.np = 0;

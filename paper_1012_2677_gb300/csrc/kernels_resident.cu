@@ -147,10 +147,8 @@ __global__ void __launch_bounds__(MIXED ? kResThreads : kDpThreads, MIXED ? 3 : 
       const uint32_t code = image_code(sx, sy, sz);
       for (int s = S.offq[q] + lane; s < S.offq[q + 1]; s += 32) src[s] = (uint32_t)(S.g0[q] + (s - S.offq[q])) | code;
     }
-    if (S.list_len <= (unsigned)ta.list_cap) {  // segments are padded to 8 entries (16 bytes)
-      const uint4* e = (const uint4*)(a.ent + S.list_base);
-      for (unsigned w = tid; w < S.list_len / 8u; w += NT) ((uint4*)(smem + R.L.ent))[w] = e[w];
-    }
+    const uint4* e = (const uint4*)(a.ent + S.list_base);  // segments are padded to 8 entries (16 bytes)
+    for (unsigned w = tid; w < min(S.list_len, (unsigned)ta.list_cap) / 8u; w += NT) ((uint4*)(smem + R.L.ent))[w] = e[w];
   }
   if (tid == 0) {
     S.row_off = 0;
@@ -326,10 +324,9 @@ __global__ void __launch_bounds__(MIXED ? kResThreads : kDpThreads, MIXED ? 3 : 
       }
     } else {
       DpForce<HALF, E> body(a.c, smem, R.D, (dvec4*)a.f);
-      const uint16_t* ent =
-          S.list_len <= (unsigned)ta.list_cap ? (const uint16_t*)(smem + R.L.ent) : a.ent + S.list_base;
       dp_tile_pairs<3, HALF>(
-          S, smem, R.D, ent, body.cut2, a.status,
+          S, smem, R.D, (const uint16_t*)(smem + R.L.ent), a.ent + S.list_base, (unsigned)ta.list_cap, body.cut2,
+          a.status,
           [&](int, const dvec4& qi, int j, double* acc) { body.pair(qi, j, acc); },
           [&](int o, const double* acc) {
             if (HALF) body.add(S.gown0 + o, acc);

@@ -374,6 +374,8 @@ __global__ void __launch_bounds__(NT, kWinCtas)
         if (t + 2 * (int64_t)gridDim.x < ta_in.ntiles) prefetch(t + 2 * (int64_t)gridDim.x);
       }
     };
+    if (warp == kNW - 1)  // the pipelined force kernel's staging descriptor
+      tile_desc_write(ti, ta.n, g.Lq, S, s_ready[buf] != 0, tile_list + ta_in.ntiles + kTileDesc * t, lane);
     if (!s_ready[buf]) {  // sizing inconsistency: record and skip the tile
       if (threadIdx.x == 0) atomicOr(status, LJ_ST_CELL_RANGE);
       if (warp == 0) prepare_next();
@@ -628,7 +630,7 @@ __device__ __forceinline__ void adjoint_tile_compute(const TileShared& S, const 
       } else {
         row = s_rows[S.row_off + o];
         row.x -= S.list_base;
-        el = S.list_len <= (unsigned)list_cap ? s_ent : ent + S.list_base;  // long segments stay in HBM
+        el = row.x + row.y <= (unsigned)list_cap ? s_ent : ent + S.list_base;  // the end of a long segment stays in HBM
         if (row.x + row.y > S.list_len) {
           if (lane == 0) atomicOr(status, LJ_ST_LIST_OVERFLOW);
           row.y = 0;

@@ -55,7 +55,7 @@ struct ljmd_sys {
   uint32_t *cell_of = nullptr, *perm = nullptr, *perm_id = nullptr;  // perm_id: perm ordered by id in each cell
   uint32_t *cell_count = nullptr, *cell_start = nullptr, *cell_fill = nullptr;
   uint2* rows = nullptr;        // per particle: (start, length) of its row in ent
-  uint2* tile_list = nullptr;   // per tile: (start, length) of its segment of ent
+  uint2* tile_list = nullptr;   // per tile: (start, length) of its segment of ent; then the staging descriptors
   int64_t tile_list_cap = 0;
   uint16_t* ent = nullptr;       // SortedList: partner indices into the key's staged tile
   size_t ent_cap = 0;
@@ -458,7 +458,7 @@ static void* force_pos(ljmd_sys* s);
 
 static int ensure_tile_list(ljmd_sys* s) {
   if (s->ta.ntiles > s->tile_list_cap) {
-    TRY(dalloc_t(s, &s->tile_list, s->ta.ntiles));
+    TRY(dalloc_t(s, &s->tile_list, kTileWords * (size_t)s->ta.ntiles));
     s->tile_list_cap = s->ta.ntiles;
   }
   return LJ_OK;
@@ -488,13 +488,12 @@ static int force_buffers(const ljmd_sys* s) {
 }
 
 // Default cells per tile along z.  The mixed form with the full list (the pipelined force kernel):
-// about 165 key particles per tile, so that the staging of the 9 (T + 2) neighbour cells and the
-// per-tile bookkeeping are spread over many keys; measured on GB300 at 16.4M particles, rho 0.5
-// (13.8 particles per cell), T = 4, 8, 10, 12 give force launches of 2.41, 2.09, 1.96, 1.88 ms and
-// list constructions of 11.7, 14.0, 13.2, 13.2 ms, and T = 12 the shortest step.  The half-list
-// forms keep 4 cells: at rho 0.8 (mixed, half list) T = 3, 4, 6 give force 3.76, 3.56, 4.06 ms and
-// construction 19.0, 19.8, 33.7 ms; the FP64 form at 1M particles, rho 0.5, gives force 1.07, 1.03,
-// 1.14, 1.05 ms at T = 3, 4, 5, 6.
+// about 165 key particles per tile, so that the staging of the 9 (T + 2) neighbour cells is spread over
+// many keys and four staged tiles keep 24 warps busy; measured on GB300 at 16.4M particles, rho 0.5
+// (13.8 particles per cell), T = 8, 10, 12, 14 give force launches of 1.59, 1.39, 1.32, 1.46 ms and list
+// constructions of 9.2, 8.6, 8.4, 9.2 ms.  The half-list forms keep 4 cells: at rho 0.8 (mixed, half list)
+// T = 3, 4, 6 give force 3.76, 3.56, 4.06 ms and construction 19.0, 19.8, 33.7 ms; the FP64 form at 1M
+// particles, rho 0.5, gives force 1.07, 1.03, 1.14, 1.05 ms at T = 3, 4, 5, 6.
 // Small boxes: the tile length is lowered until there are at least two tiles per SM, so that the
 // force launch spreads over the GPU (4,000 particles, 6 cells per side, FP64 form: T = 4, 2, 1 give
 // 72, 108, 216 tiles and force launches of 40, 29, 24 us).
@@ -510,9 +509,8 @@ static int default_tile_cells(const ljmd_sys* s) {
 }
 
 // Default threads per key in the force kernel: for the mixed form with the full list, 2 for tiles
-// of about 100 keys or more (more keys than 4-lane groups otherwise), 4 below (measured as above:
-// T = 10 with 2 lanes 1.96 ms, 4 lanes 2.01 ms; T = 4 with 2 lanes 2.41 ms, 4 lanes 2.41 ms,
-// 8 lanes 2.67 ms); 4 for the half-list forms.
+// of about 100 keys or more (16.4M particles, T = 12: 1.32 ms, 4 threads 1.44 ms), 4 below; 4 for
+// the half-list forms, 8 for their small tiles.
 static int default_lanes(const ljmd_sys* s) {
   const double ppc = (double)s->n / (double)std::max<int64_t>(s->ncells, 1);
   if (s->precision != LJ_MIXED || s->list_half) return (double)s->ta.T * ppc <= 32.0 ? 8 : 4;
@@ -545,8 +543,8 @@ static int choose_tiles(ljmd_sys* s, int t_cap) {
   if (T > kMaxTileT) T = kMaxTileT;
   if (T < 1) T = 1;
   for (;; --T) {
-    ta.T = T;
     ta.ntz = (n + T - 1) / T;
+    ta.T = T = (n + ta.ntz - 1) / ta.ntz;  // the same number of tiles, of even length
     ta.ntiles = (int64_t)n * n * ta.ntz;
     CK(cudaMemsetAsync(s->d_sizes, 0, 3 * sizeof(unsigned int), s->st));
     launch_tile_sizes(s->cell_start, ta, s->d_sizes, s->st);
@@ -655,22 +653,7 @@ static int rebuild(ljmd_sys* s) {
     // kernel) comes out of the same limit
     const int64_t smem_dyn = (int64_t)smem_max - (nbuf == 2 ? 5376 : 2816);
     if ((int64_t)base_bytes <= smem_dyn) {
-      int64_t room = (smem_dyn - (int64_t)base_bytes) / (2 * nbuf) - 16;
-      // The pipelined kernel of the mixed form with the full list runs 3 CTAs per SM with 8
-      // consumer warps (T <= 4) and 2 with 12: the staged segments are capped so that this many
-      // fit in an SM's shared memory (1 KB reserved and at most 6 KB of static shared memory per
-      // CTA), when that still stages at least half of the largest segment.  Longer segments are
-      // read from HBM (on the FCC start, whose longest segment is 1.5 times the liquid's, this
-      // still beat one CTA per SM: 16.4M, 20 steps, 3.41 -> 3.35 ms per step).
-      if (s->precision == LJ_MIXED && !s->list_half && !s->ta.whole && nbuf == 2) {
-        int smem_sm = 0;
-        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        const int target = s->ta.T <= 4 ? 3 : 2;
-        const int64_t per_cta = (int64_t)smem_sm / target - 1024 - 6144;
-        const int64_t fb = (int64_t)force_smem_bytes(tz, s->precision, 2, 0);
-        const int64_t room_occ = (per_cta - fb) / (2 * nbuf) - 16;
-        if (room_occ >= (int64_t)s->ta.max_list / 2) room = std::min(room, room_occ);
-      }
+      const int64_t room = (smem_dyn - (int64_t)base_bytes) / (2 * nbuf) - 16;
       s->ta.list_cap = (int32_t)std::max<int64_t>(0, std::min<int64_t>(s->ta.max_list, room) & ~(int64_t)7);
       break;
     }

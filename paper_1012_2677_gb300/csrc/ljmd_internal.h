@@ -128,7 +128,7 @@ struct TileArgs {
   int32_t max_own;     // own particles per tile, at most
   int32_t max_chunks;  // 32-candidate chunks per own particle, at most
   int32_t max_list;    // list entries per tile (padded to 8), at most (known after construction)
-  int32_t list_cap;    // entries of a tile's segment the force kernel stages; longer ones stay in HBM
+  int32_t list_cap;    // entries of a tile's segment the force kernel stages (multiple of 8); the rest stays in HBM
 };
 // One replica of a batch: its box (offset and p are the batch's), grid, tiles and particles.
 // Global tiles, cells and particles are the replicas' ranges concatenated in replica order.
@@ -139,6 +139,7 @@ struct ReplicaGeo {
   int64_t cell_base;       // first global cell
   int64_t base, count;     // first global particle, particles
 };
+constexpr int kTileWords = 25;  // 8-byte words of tile_list per tile: its list segment and its staging descriptor
 size_t list_smem_bytes(const TileArgs& ta, int precision);
 size_t force_smem_bytes(const TileArgs& ta, int precision, int nbuf, int half);
 void launch_max_count(const uint32_t* cnt, int64_t n, unsigned int* out, cudaStream_t s);

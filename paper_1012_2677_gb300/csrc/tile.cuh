@@ -115,66 +115,57 @@ __device__ __forceinline__ bool stage_offsets(const TileInfo& ti, const TileArgs
   return S.total <= ta.max_staged;
 }
 
-// Cell bounds of a tile's staged cells held in one warp's registers (lane l: cells l, l + 32, ...),
-// loaded a tile ahead of their use so the bookkeeping never waits on memory.
-constexpr int kPfRounds = (kMaxCells + 31) / 32;
-struct TilePrefetch {
-  TileInfo ti;
-  uint2 tl;
-  uint32_t a[kPfRounds], b[kPfRounds];
-};
+// Staging descriptor of a tile, kTileDesc words of 8 bytes written by the list kernel (behind the tiles'
+// list segments: tile_list + ntiles) and read by the pipelined force kernel, one word per lane, so that
+// staging a tile takes no bookkeeping at all in the ten or so steps of a list's life:
+//   0..17  run 2 k + r of column k: first sorted index; staged slot << 16 | particles (a column is one
+//          run, or two where z wraps)
+//   18     staged particles (kTileInvalid: the tile exceeded the capacities); own slot | own particles << 16
+//   19     sorted index of the first own particle; 1 if the tile has periodic images
+//   20     cx | cy << 16; z0 | cells << 16
+//   21     cells per side; image shift round(L / u)
+constexpr int kTileDesc = kTileWords - 1;
+constexpr int kTileDescWords = 22;
+constexpr uint32_t kTileInvalid = 0xffffffffu;
 
-__device__ __forceinline__ void tile_prefetch(int64_t t, const TileArgs& ta, const uint32_t* __restrict__ cs,
-                                              const uint2* __restrict__ tile_list, TilePrefetch& pf, int lane) {
-  pf.ti = tile_info(t, ta);
-  const int ncol = pf.ti.Tp + 2, ncell = 9 * ncol;
-  pf.tl = tile_list ? tile_list[t] : make_uint2(0u, 0u);
-#pragma unroll
-  for (int r = 0; r < kPfRounds; ++r) {
-    const int q = 32 * r + lane;
-    pf.a[r] = pf.b[r] = 0u;
-    if (q < ncell) {
-      int sx, sy, sz;
-      const uint32_t c = cell_of_q(pf.ti, ta.n, ncol, q, sx, sy, sz);
-      pf.a[r] = cs[c];
-      pf.b[r] = cs[c + 1];
-    }
-  }
+__device__ __forceinline__ bool tile_interior(const TileInfo& ti, int n) {
+  return ti.cx >= 1 && ti.cx <= n - 2 && ti.cy >= 1 && ti.cy <= n - 2 && ti.z0 >= 1 && ti.z0 + ti.Tp <= n - 1;
 }
 
-// The bookkeeping of stage_offsets done by one warp from prefetched bounds (no CTA barrier, the
-// other warps keep computing); also the tile's list segment.
-__device__ __forceinline__ bool tile_prepare_pf(const TilePrefetch& pf, const TileArgs& ta, TileShared& S, int lane) {
-  const int ncol = pf.ti.Tp + 2, ncell = 9 * ncol;
-  int run = 0;
-#pragma unroll
-  for (int r = 0; r < kPfRounds; ++r) {
-    if (32 * r >= ncell) break;
-    const int q = 32 * r + lane;
-    int inc = q < ncell ? (int)(pf.b[r] - pf.a[r]) : 0;
-    if (q < ncell) S.g0[q] = (int)pf.a[r];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
+// The first cell of run r = 1 of a tile's columns (ncol: there is none).
+__device__ __forceinline__ int tile_run_cut(int z0, int Tp, int n) {
+  return z0 == 0 ? 1 : (z0 + Tp == n ? Tp + 1 : Tp + 2);
+}
+
+// Image shifts of run l of a tile.
+__device__ __forceinline__ void tile_run_shift(const TileInfo& ti, int n, int l, int& sx, int& sy, int& sz) {
+  const int k = l >> 1, r = l & 1;
+  wrap_cell(ti.cx + k / 3 - 1, n, sx);
+  wrap_cell(ti.cy + k % 3 - 1, n, sy);
+  sz = ti.z0 == 0 && r == 0 ? -1 : (ti.z0 + ti.Tp == n && r == 1 ? 1 : 0);
+}
+
+// One warp writes the descriptor of a tile from its bookkeeping.
+__device__ __forceinline__ void tile_desc_write(const TileInfo& ti, int n, uint32_t Lq, const TileShared& S, bool valid,
+                                                uint2* __restrict__ desc, int lane) {
+  uint2 d = make_uint2(0u, 0u);
+  if (lane < 18) {
+    const int k = lane >> 1, r = lane & 1, ncol = S.ncol, cut = tile_run_cut(ti.z0, ti.Tp, n);
+    const int m0 = r ? cut : 0, m1 = r ? ncol : cut;
+    if (valid && m1 > m0) {
+      const int a = S.offq[k * ncol + m0], b = S.offq[k * ncol + m1];
+      d = make_uint2((uint32_t)S.g0[k * ncol + m0], (uint32_t)a << 16 | (uint32_t)(b - a));
     }
-    if (q < ncell) S.offq[q + 1] = run + inc;
-    run += __shfl_sync(0xffffffffu, inc, 31);
+  } else if (lane == 18) {
+    d = make_uint2(valid ? (uint32_t)S.total : kTileInvalid, (uint32_t)S.own0 | (uint32_t)(S.own1 - S.own0) << 16);
+  } else if (lane == 19) {
+    d = make_uint2((uint32_t)S.gown0, tile_interior(ti, n) ? 0u : 1u);
+  } else if (lane == 20) {
+    d = make_uint2((uint32_t)(ti.cx | ti.cy << 16), (uint32_t)(ti.z0 | ti.Tp << 16));
+  } else if (lane == 21) {
+    d = make_uint2((uint32_t)n, Lq);
   }
-  __syncwarp();
-  if (lane == 0) {
-    S.offq[0] = 0;
-    S.ncol = ncol;
-    S.ncell = ncell;
-    S.total = run;
-    S.own0 = S.offq[4 * ncol + 1];
-    S.own1 = S.offq[4 * ncol + pf.ti.Tp + 1];
-    S.gown0 = S.g0[4 * ncol + 1];
-    S.list_base = pf.tl.x;
-    S.list_len = pf.tl.y;
-  }
-  __syncwarp();
-  return run <= ta.max_staged;
+  if (lane < kTileDescWords) desc[lane] = d;
 }
 
 // Cell bounds of a tile's staged cells copied asynchronously into shared memory (one warp; lane m
@@ -299,7 +290,7 @@ __device__ __forceinline__ void stage_issue(const TileInfo& ti, const TileArgs& 
     r0 = S.gown0 & ~1;
     r1 = (S.gown0 + n_own + 1) & ~1;
     if (n_own > 0) bytes += 8u * (unsigned)(r1 - r0);
-    if (S.list_len <= (unsigned)ta.list_cap) bytes += 2u * S.list_len;
+    bytes += 2u * min(S.list_len, (unsigned)ta.list_cap);
   }
   if (lane == 0) {
     fence_proxy_async_smem();
@@ -332,8 +323,8 @@ __device__ __forceinline__ void stage_issue(const TileInfo& ti, const TileArgs& 
     }
   } else if (FORCE && lane == 9) {
     if (n_own > 0) bulk_g2s(smem + L.rows, rows + r0, 8u * (unsigned)(r1 - r0), bar);
-    if (S.list_len > 0 && S.list_len <= (unsigned)ta.list_cap)
-      bulk_g2s(smem + L.ent, ent + S.list_base, 2u * S.list_len, bar);
+    const unsigned n_ent = min(S.list_len, (unsigned)ta.list_cap);  // rows beyond the capacity stay in HBM
+    if (n_ent > 0) bulk_g2s(smem + L.ent, ent + S.list_base, 2u * n_ent, bar);
     S.row_off = S.gown0 - r0;
   }
 }
@@ -542,8 +533,9 @@ __device__ __forceinline__ double rcp_nr64(double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
+// A key's sums over the two pairs a lane takes side by side (x: even, y: odd entries of the lane).
 struct AccF {
-  float fx, fy, fz, pe, vir;
+  float2 fx, fy, fz, pe, vir;
 };
 
 // Per-thread energy and virial sums over the keys a thread finishes: FP32 partials of at most
@@ -578,53 +570,81 @@ __device__ __forceinline__ float qd(uint32_t a, uint32_t b, const Geom& g) {
   return __int2float_rn(d);
 }
 
-// One listed pair in the mixed form (Alg. 6 in eps/sigma form) on differences in units of u:
+// Two listed pairs of one key in the mixed form (Alg. 6 in eps/sigma form) on differences in units of u:
 //   f = ri2 s3i (24 eps - 48 eps s3i) + 8 eps c2 / sigma^2, zero for r^2 >= r_c^2 (select)
 //   V = 4 eps [s3i (s3i - 1) + c2 r^2 / sigma^2 + c0],  W += -f r^2
 // with the constants scaled by powers of u (LJConst::*q), so f d and V come out in sigma units and
-// W in units of 1/u.  HALF: Newton-3 scatter to the partner's sorted index, carried in qj.w.
+// W in units of 1/u.  The FP32 arithmetic is packed two by two (the kernels are bound by issue: one
+// packed instruction in the place of two): the reciprocal is taken of -r^2, which keeps every sign out of
+// the packed instructions (they have no negation), and the factor 4 eps of V is left to the caller;
+// a.vir sums +f r^2.  HALF: d is x_i - x_j, so that f d is the force on the partner, added to its sorted
+// index (carried in q.w); a then holds minus the key's sums.  two: the second pair exists (else it
+// repeats the first and counts nothing).
 template <bool HALF, bool ENERGY, bool WHOLE>
-__device__ __forceinline__ void pair_q(const uint4& qi, const uint4& qj, const LJConst& c, const Geom& g, AccF& a,
-                                       float4* fout) {
-  const float dx = qd<WHOLE>(qj.x, qi.x, g), dy = qd<WHOLE>(qj.y, qi.y, g), dz = qd<WHOLE>(qj.z, qi.z, g);
-  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float ri2 = rcp_nr(r2);
-  const float si = c.sig2q * ri2;
-  const float s3i = si * si * si;
-  const bool in = r2 < c.rc2q;
-  float ff = fmaf(ri2 * s3i, fmaf(-c.f48q, s3i, c.f24q), c.f8c2q);
-  ff = in ? ff : 0.0f;
-  a.fx = fmaf(ff, dx, a.fx);
-  a.fy = fmaf(ff, dy, a.fy);
-  a.fz = fmaf(ff, dz, a.fz);
-  if (HALF) atomicAdd(&fout[qj.w], make_float4(-ff * dx, -ff * dy, -ff * dz, 0.0f));
+__device__ __forceinline__ void pair2_q(const uint4& qi, const uint4& q0, const uint4& q1, bool two, const LJConst& c,
+                                        const Geom& g, AccF& a, float4* fout) {
+  float2 dx, dy, dz;
+  if (HALF) {
+    dx = make_float2(qd<WHOLE>(qi.x, q0.x, g), qd<WHOLE>(qi.x, q1.x, g));
+    dy = make_float2(qd<WHOLE>(qi.y, q0.y, g), qd<WHOLE>(qi.y, q1.y, g));
+    dz = make_float2(qd<WHOLE>(qi.z, q0.z, g), qd<WHOLE>(qi.z, q1.z, g));
+  } else {
+    dx = make_float2(qd<WHOLE>(q0.x, qi.x, g), qd<WHOLE>(q1.x, qi.x, g));
+    dy = make_float2(qd<WHOLE>(q0.y, qi.y, g), qd<WHOLE>(q1.y, qi.y, g));
+    dz = make_float2(qd<WHOLE>(q0.z, qi.z, g), qd<WHOLE>(q1.z, qi.z, g));
+  }
+  const float2 one = make_float2(1.0f, 1.0f);
+  const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+  // -1/r^2: the hardware approximation of it, refined by one Newton-Raphson step (as rcp_nr)
+  float2 nr;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(nr.x) : "f"(-r2.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(nr.y) : "f"(-r2.y));
+  nr = __ffma2_rn(nr, __ffma2_rn(r2, nr, one), nr);
+  const float2 ns = __fmul2_rn(make_float2(c.sig2q, c.sig2q), nr);
+  const float2 ns3 = __fmul2_rn(__fmul2_rn(ns, ns), ns);  // -s3i
+  float2 ff = __ffma2_rn(__fmul2_rn(nr, ns3), __ffma2_rn(make_float2(c.f48q, c.f48q), ns3, make_float2(c.f24q, c.f24q)),
+                         make_float2(c.f8c2q, c.f8c2q));
+  const bool in0 = r2.x < c.rc2q, in1 = two && r2.y < c.rc2q;
+  ff.x = in0 ? ff.x : 0.0f;
+  ff.y = in1 ? ff.y : 0.0f;
+  a.fx = __ffma2_rn(ff, dx, a.fx);
+  a.fy = __ffma2_rn(ff, dy, a.fy);
+  a.fz = __ffma2_rn(ff, dz, a.fz);
+  if (HALF) {
+    const float2 fx = __fmul2_rn(ff, dx), fy = __fmul2_rn(ff, dy), fz = __fmul2_rn(ff, dz);
+    atomicAdd(&fout[q0.w], make_float4(fx.x, fy.x, fz.x, 0.0f));
+    if (two) atomicAdd(&fout[q1.w], make_float4(fx.y, fy.y, fz.y, 0.0f));
+  }
   if (ENERGY) {
-    const float v = c.e4 * fmaf(s3i, s3i - 1.0f, fmaf(c.c2q, r2, c.c0f));
-    a.pe += in ? v : 0.0f;
-    a.vir = fmaf(-ff, r2, a.vir);
+    float2 v = __ffma2_rn(ns3, __fadd2_rn(ns3, one),
+                          __ffma2_rn(make_float2(c.c2q, c.c2q), r2, make_float2(c.c0f, c.c0f)));
+    v.x = in0 ? v.x : 0.0f;
+    v.y = in1 ? v.y : 0.0f;
+    a.pe = __fadd2_rn(a.pe, v);
+    a.vir = __ffma2_rn(ff, r2, a.vir);
   }
 }
 
-// Forces of the own particles of one staged tile (buffer `buf`); group `grp` of LANES threads per
-// key particle, lanes striding over its row.
-template <bool MIXED, int LANES, bool HALF, bool ENERGY, bool WHOLE, bool LONGLIST, int NTH = kTileThreads>
-__device__ __forceinline__ void force_tile_compute(const TileShared& S, const unsigned char* buf, const TileLayout& L,
+// Forces of the own particles of one staged tile (buffer `buf`); LANES threads per key particle, striding
+// over its row; a thread's group starts at key grp and steps by the number of groups.
+template <bool MIXED, int LANES, bool HALF, bool ENERGY, bool WHOLE, bool LONGLIST, int NTH = kTileThreads, class TS>
+__device__ __forceinline__ void force_tile_compute(const TS& S, const unsigned char* buf, const TileLayout& L,
                                                    const uint2* __restrict__ rows, const uint16_t* __restrict__ ent,
                                                    const LJConst& c, const Geom& g, void* __restrict__ fout,
-                                                   int32_t* __restrict__ status, EAcc& eacc, int list_cap) {
+                                                   int32_t* __restrict__ status, EAcc& eacc, int list_cap,
+                                                   int grp = threadIdx.x / LANES) {
   const void* sh_pos = buf + L.pos;
   const int* sh_gid = (const int*)(buf + L.gid);
   const uint2* s_rows = (const uint2*)(buf + L.rows);
   const uint16_t* s_ent = (const uint16_t*)(buf + L.ent);
   const int lane = threadIdx.x & (LANES - 1);
-  const int grp = threadIdx.x / LANES;
   constexpr int kGroups = NTH / LANES;  // groups of the computing threads
   const double f24d = 24.0 * c.eps, f48d = 48.0 * c.eps, f8c2d = 8.0 * c.eps * c.c2 / c.sig2;
   const double e4d = 4.0 * c.eps, c2sd = c.c2 / c.sig2;
   const int n_own = S.own1 - S.own0;
   for (int o = grp; __any_sync(0xffffffffu, o < n_own); o += kGroups) {
     const bool valid = o < n_own;
-    AccF a0{0.f, 0.f, 0.f, 0.f, 0.f}, a1{0.f, 0.f, 0.f, 0.f, 0.f};
+    AccF a = {};
     double dfx = 0.0, dfy = 0.0, dfz = 0.0, dpe = 0.0, dvir = 0.0;
     int gi = 0;
     if (valid) {
@@ -648,27 +668,22 @@ __device__ __forceinline__ void force_tile_compute(const TileShared& S, const un
         const uint32_t a_pos = smem_addr(sh_pos);
         const uint4 qi = lds_u4(a_pos + 16u * l);
         float4* F = (float4*)fout;
-        auto pair_at = [&](uint32_t j, AccF& acc) {
-          pair_q<HALF, ENERGY, WHOLE>(qi, lds_u4(a_pos + (j << 4)), c, g, acc, F);
+        auto pairs_at = [&](uint32_t j0, uint32_t j1, bool two) {
+          pair2_q<HALF, ENERGY, WHOLE>(qi, lds_u4(a_pos + (j0 << 4)), lds_u4(a_pos + (j1 << 4)), two, c, g, a, F);
         };
         if (in_smem) {
-          // list segment staged: entries by 32-bit shared address, two independent per iteration
+          // list segment staged: entries by 32-bit shared address, two per iteration
           uint32_t p = smem_addr(s_ent) + 2u * (row.x + lane);
           const uint32_t pend = smem_addr(s_ent) + 2u * (row.x + row.y);
-          for (; p + 2u * LANES < pend; p += 4u * LANES) {
-            const uint32_t j0 = lds_u16(p), j1 = lds_u16(p + 2u * LANES);
-            pair_at(j0, a0);
-            pair_at(j1, a1);
+          for (; p + 2u * LANES < pend; p += 4u * LANES) pairs_at(lds_u16(p), lds_u16(p + 2u * LANES), true);
+          if (p < pend) {
+            const uint32_t j = lds_u16(p);
+            pairs_at(j, j, false);
           }
-          if (p < pend) pair_at(lds_u16(p), a0);
         } else {
           unsigned e = lane;
-          for (; e + LANES < row.y; e += 2 * LANES) {
-            const uint32_t j0 = el[row.x + e], j1 = el[row.x + e + LANES];
-            pair_at(j0, a0);
-            pair_at(j1, a1);
-          }
-          if (e < row.y) pair_at(el[row.x + e], a0);
+          for (; e + LANES < row.y; e += 2 * LANES) pairs_at(el[row.x + e], el[row.x + e + LANES], true);
+          if (e < row.y) pairs_at(el[row.x + e], el[row.x + e], false);
         }
       } else {
         const dvec4 qi = ((const dvec4*)sh_pos)[l];
@@ -707,19 +722,19 @@ __device__ __forceinline__ void force_tile_compute(const TileShared& S, const un
       }
       };
       if (WHOLE) row_pairs(ent, false);
-      else if (!LONGLIST || S.list_len <= (unsigned)list_cap) row_pairs(s_ent, true);
-      else row_pairs(ent + S.list_base, false);  // a long segment stays in HBM
+      else if (!LONGLIST || row.x + row.y <= (unsigned)list_cap) row_pairs(s_ent, true);
+      else row_pairs(ent + S.list_base, false);  // the end of a long segment stays in HBM
     }
     if (MIXED) {
-      float fx = gsum<LANES>(a0.fx + a1.fx);
-      float fy = gsum<LANES>(a0.fy + a1.fy);
-      float fz = gsum<LANES>(a0.fz + a1.fz);
+      float fx = gsum<LANES>(a.fx.x + a.fx.y);
+      float fy = gsum<LANES>(a.fy.x + a.fy.y);
+      float fz = gsum<LANES>(a.fz.x + a.fz.y);
       if (valid && lane == 0) {
-        if (HALF) atomicAdd(&((float4*)fout)[gi], make_float4(fx, fy, fz, 0.0f));
+        if (HALF) atomicAdd(&((float4*)fout)[gi], make_float4(-fx, -fy, -fz, 0.0f));
         else ((float4*)fout)[gi] = make_float4(fx, fy, fz, 0.0f);
       }
       if (ENERGY) {  // the group's lanes reduce in FP32, one lane accumulates
-        const float pe = gsum<LANES>(a0.pe + a1.pe), vir = gsum<LANES>(a0.vir + a1.vir);
+        const float pe = c.e4 * gsum<LANES>(a.pe.x + a.pe.y), vir = -gsum<LANES>(a.vir.x + a.vir.y);
         if (lane == 0) eacc.add32(pe, vir);
       }
     } else {
@@ -955,12 +970,13 @@ __device__ __forceinline__ bool dp_stage_finish(const TileInfo& ti, const TileAr
 
 // The listed pairs of a staged tile's keys inside r_c (or within the filter's margin of it).
 // pair(key slot, qi, partner slot, acc) adds one pair to the key's NACC sums; done(o, acc) receives
-// the sums of own key o.  ent: the tile's segment (staged, or in HBM if it is longer).
+// the sums of own key o.
+// ent_s: the staged part of the tile's segment, its first cap entries; rows beyond it are read from ent_g.
 // DIRECT: done(o, acc) is called by the lanes themselves with each partial sum (it must add atomically).
 template <int NACC, bool DIRECT, class Pair, class Done>
 __device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigned char* smem, const DpLayout& D,
-                                              const uint16_t* ent, float cut2, int32_t* status, Pair&& pair,
-                                              Done&& done) {
+                                              const uint16_t* ent_s, const uint16_t* ent_g, unsigned cap, float cut2,
+                                              int32_t* status, Pair&& pair, Done&& done) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const uint4* sq = (const uint4*)(smem + D.xq);
@@ -1031,6 +1047,7 @@ __device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigne
     }
     for (int k = 0; k < nk; ++k) {
       const int start = (int)__shfl_sync(0xffffffffu, row.x, k), len = (int)__shfl_sync(0xffffffffu, row.y, k);
+      const uint16_t* ent = (unsigned)(start + len) <= cap ? ent_s : ent_g;
       const uint4 qi = sq[S.own0 + b0 + k];
       if (lane == k) ka = cnt;
       for (int e0 = 0; e0 < len; e0 += 32) {
