@@ -334,14 +334,15 @@ int ljmd_get_profile(ljmd_sys* sys, ljmd_profile* out);
 
 /*
  * Kernel shape of the list and force kernels (the autotuner's knobs); 0 keeps the default.
- * tile_cells: cells per shared-memory tile along z (1..14; default: for the mixed form with the
- * full list about 165 particles per tile, at most 12 cells, else 4); lanes: threads per key
+ * tile_cells: cells per shared-memory tile along z (1..14; default: for the mixed form about 165
+ * particles per tile with the full list and 216 with the half list, at most 12 cells; 4 in the FP64
+ * form); lanes: threads per key
  * particle in the force kernel (1, 2, 4, 8, 16, 32; default: for the mixed form with the full list
  * 2 for tiles of 96 or more particles, else 4; the FP64 form shares a warp among a run of keys
  * whatever the value); force_ctas_per_sm: resident force CTAs per SM
  * (1..4; the pipelined kernel runs one); force_buffers: tile buffers per force CTA
  * (1: tiles staged one after the other; 2: the next tile's copies overlap the current tile's
- * arithmetic; for the mixed form with the full list this is the pipelined kernel, in which producer
+ * arithmetic; for the mixed form this is the pipelined kernel, in which producer
  * warps stage tiles into two to four buffers and consumer warps compute, and it is the default there;
  * 1 is the default otherwise, and the FP64 form always uses one).  A new tile_cells or force_buffers
  * takes effect at the next list construction (forced at the next force evaluation).  Results

@@ -467,8 +467,8 @@ static int ensure_tile_list(ljmd_sys* s) {
 // Tile geometry for the staged list/force kernels: T cells along z per tile, shared-memory
 // capacities from the actual largest tile of the current cell occupancy.
 // Tile buffers per force CTA: the requested number, else two for the form with a pipelined
-// kernel (producer warps stage the next tile while consumer warps compute): the mixed form with
-// the full list; one otherwise.
+// kernel (producer warps stage the next tiles while consumer warps compute): the mixed form; one
+// otherwise.
 // Multiprocessors of a device (152 if the attribute cannot be read).
 static int sm_count_of(int dev) {
   int sms = 0;
@@ -484,24 +484,25 @@ static int force_buffers(const ljmd_sys* s) {
   // fewer tiles than two per SM: the single-buffer kernel (the pipelined one holds one CTA per SM
   // with two producer warps)
   if (s->ta.ntiles > 0 && s->ta.ntiles < 2 * (int64_t)sm_count_of(s->device)) return 1;
-  return s->precision == LJ_MIXED && !s->list_half ? 2 : 1;
+  return s->precision == LJ_MIXED ? 2 : 1;
 }
 
 // Default cells per tile along z.  The mixed form with the full list (the pipelined force kernel):
 // about 165 key particles per tile, so that the staging of the 9 (T + 2) neighbour cells is spread over
 // many keys and four staged tiles keep 24 warps busy; measured on GB300 at 16.4M particles, rho 0.5
 // (13.8 particles per cell), T = 8, 10, 12, 14 give force launches of 1.59, 1.39, 1.32, 1.46 ms and list
-// constructions of 9.2, 8.6, 8.4, 9.2 ms.  The half-list forms keep 4 cells: at rho 0.8 (mixed, half list)
-// T = 3, 4, 6 give force 3.76, 3.56, 4.06 ms and construction 19.0, 19.8, 33.7 ms; the FP64 form at 1M
-// particles, rho 0.5, gives force 1.07, 1.03, 1.14, 1.05 ms at T = 3, 4, 5, 6.
+// constructions of 9.2, 8.6, 8.4, 9.2 ms.  With the half list (mixed form) about 216: at rho 0.8, 2M
+// particles, T = 4, 6, 8, 10, 12 give force launches of 341, 309, 291, 276, 335 us and constructions of
+// 1.37, 1.23, 1.16, 1.03, 1.27 ms.  The FP64 form keeps 4 cells: at 1M particles, rho 0.5, its force takes
+// 1.07, 1.03, 1.14, 1.05 ms at T = 3, 4, 5, 6.
 // Small boxes: the tile length is lowered until there are at least two tiles per SM, so that the
 // force launch spreads over the GPU (4,000 particles, 6 cells per side, FP64 form: T = 4, 2, 1 give
 // 72, 108, 216 tiles and force launches of 40, 29, 24 us).
 static int default_tile_cells(const ljmd_sys* s) {
   int T = 4;
-  if (s->precision == LJ_MIXED && !s->list_half) {
+  if (s->precision == LJ_MIXED) {
     const double ppc = (double)s->n / (double)std::max<int64_t>(s->ncells, 1);
-    T = std::max(1, std::min((int)lround(165.0 / std::max(ppc, 1.0)), 12));
+    T = std::max(1, std::min((int)lround((s->list_half ? 216.0 : 165.0) / std::max(ppc, 1.0)), 12));
   }
   const int64_t n = s->g.n, want = 2 * (int64_t)sm_count_of(s->device);
   while (T > 1 && n * n * ((n + T - 1) / T) < want) --T;

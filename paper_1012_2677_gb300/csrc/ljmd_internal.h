@@ -174,6 +174,8 @@ struct ForceLaunch {
   cudaStream_t s;
 };
 void launch_force_mixed_half(const ForceLaunch& a);
+int launch_force_pipe_half(const ForceLaunch& a);
+int pipe_plan(TileArgs& ta);
 int launch_force_fp64(int half, ForceLaunch& a);  // returns the grid launched
 size_t dp_force_smem_bytes(const TileArgs& ta, int half);
 bool dp_fits(const TileArgs& ta);

@@ -612,8 +612,8 @@ __device__ __forceinline__ void pair2_q(const uint4& qi, const uint4& q0, const 
   a.fz = __ffma2_rn(ff, dz, a.fz);
   if (HALF) {
     const float2 fx = __fmul2_rn(ff, dx), fy = __fmul2_rn(ff, dy), fz = __fmul2_rn(ff, dz);
-    atomicAdd(&fout[q0.w], make_float4(fx.x, fy.x, fz.x, 0.0f));
-    if (two) atomicAdd(&fout[q1.w], make_float4(fx.y, fy.y, fz.y, 0.0f));
+    if (in0) atomicAdd(&fout[q0.w], make_float4(fx.x, fy.x, fz.x, 0.0f));
+    if (in1) atomicAdd(&fout[q1.w], make_float4(fx.y, fy.y, fz.y, 0.0f));
   }
   if (ENERGY) {
     float2 v = __ffma2_rn(ns3, __fadd2_rn(ns3, one),
