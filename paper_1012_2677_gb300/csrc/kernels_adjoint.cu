@@ -77,32 +77,35 @@ void launch_accum_q(const double* q, double a0, double a1, double a3, double a4,
   k_accum_q<<<1, 1, 0, s>>>(q, a0, a1, a3, a4, gth);
 }
 
-// y += a x (n doubles)
-// The reverse step's update of the position adjoint from one adjoint pass (sorted order):
-// lx[3 id[s] + k] -= c hw[s].k + a f[s].k (f may be null when a = 0).
-__global__ void k_adjoint_update(const dvec4* __restrict__ hw, const dvec4* __restrict__ f,
-                                 const int32_t* __restrict__ id, int64_t N, double c, double a,
-                                 double* __restrict__ lx) {
+// The reverse step's preparation (see launch_adjoint_prepare): what separate launches of k_axpy, k_to_sorted,
+// k_load_unwrapped and the integrator's copy pass did, one pass over the particles.
+__global__ void k_adjoint_prepare(const double* __restrict__ u, double* __restrict__ lv, const double* __restrict__ lx,
+                                  double dt, const int32_t* __restrict__ img, const int32_t* __restrict__ id, int64_t N,
+                                  double offset, double L, int qk, double* __restrict__ x, uint4* __restrict__ xq,
+                                  dvec4* __restrict__ pos64, dvec4* __restrict__ w, float4* __restrict__ wf) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) {
     const int64_t p = id[s];
-    const dvec4 h = hw[s];
-    double dx = c * h.x, dy = c * h.y, dz = c * h.z;
-    if (f) {
-      const dvec4 g = f[s];
-      dx = fma(a, g.x, dx);
-      dy = fma(a, g.y, dy);
-      dz = fma(a, g.z, dz);
+    double v[3], xs[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      v[k] = fma(dt, lx[3 * p + k], lv[3 * p + k]);
+      lv[3 * p + k] = v[k];
+      xs[k] = offset + (u[3 * p + k] - (double)img[k * N + s] * L);
+      x[k * N + s] = xs[k];
     }
-    lx[3 * p] -= dx;
-    lx[3 * p + 1] -= dy;
-    lx[3 * p + 2] -= dz;
+    w[s] = make_dvec4(v[0], v[1], v[2], 0.0);
+    wf[s] = make_float4((float)v[0], (float)v[1], (float)v[2], 0.0f);
+    if (xq) xq[s] = make_uint4(fixq(xs[0], qk), fixq(xs[1], qk), fixq(xs[2], qk), (uint32_t)s);
+    else pos64[s] = make_dvec4(xs[0], xs[1], xs[2], 0.0);
   }
 }
-void launch_adjoint_update(const dvec4* hw, const dvec4* f, const int32_t* id, int64_t N, double c, double a,
-                           double* lx, cudaStream_t s) {
-  k_adjoint_update<<<grid_of(N), 256, 0, s>>>(hw, f, id, N, c, a, lx);
+void launch_adjoint_prepare(const double* u, double* lv, const double* lx, double dt, const int32_t* img,
+                            const int32_t* id, int64_t N, double offset, double L, int qk, double* x, uint4* xq,
+                            dvec4* pos64, dvec4* w, float4* wf, cudaStream_t s) {
+  k_adjoint_prepare<<<grid_of(N), 256, 0, s>>>(u, lv, lx, dt, img, id, N, offset, L, qk, x, xq, pos64, w, wf);
 }
 
+// y += a x (n doubles)
 __global__ void k_axpy(double* __restrict__ y, double a, const double* __restrict__ x, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = fma(a, x[i], y[i]);

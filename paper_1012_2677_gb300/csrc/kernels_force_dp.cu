@@ -33,13 +33,12 @@ __global__ void __launch_bounds__(kDpThreads, 4)
     if (force_tile_prepare(ti, t, ta, cs, tile_list, S, status)) {
       stage_issue<false, true>(ti, ta, pos, rows, ent, S, smem, D.L, &bar);
       if (!dp_stage_finish(ti, ta, g, S, smem, D, &bar, ph, status)) return;
-      auto pair = [&](int, const dvec4& qi, int j, double* acc) { body.pair(qi, j, acc); };
+      auto pair = [&](const dvec4& qi, int j, double* acc) { body.pair(qi, j, acc); };
       auto done = [&](int o, const double* acc) {
         if (HALF) body.add(S.gown0 + o, acc);
         else fout[S.gown0 + o] = make_dvec4(acc[0], acc[1], acc[2], 0.0);
       };
-      dp_tile_pairs<3, HALF>(S, smem, D, (const uint16_t*)(smem + D.L.ent), ent + S.list_base, (unsigned)ta.list_cap,
-                             body.cut2, status, pair, done);
+      dp_tile_pairs<3, HALF>(S, smem, D, ent + S.list_base, (unsigned)ta.list_cap, body.cut2, status, pair, done);
       if (ENERGY) {
         npairs += (double)body.np;
         body.np = 0;

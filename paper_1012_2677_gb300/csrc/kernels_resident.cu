@@ -325,9 +325,8 @@ __global__ void __launch_bounds__(MIXED ? kResThreads : kDpThreads, MIXED ? 3 : 
     } else {
       DpForce<HALF, E> body(a.c, smem, R.D, (dvec4*)a.f);
       dp_tile_pairs<3, HALF>(
-          S, smem, R.D, (const uint16_t*)(smem + R.L.ent), a.ent + S.list_base, (unsigned)ta.list_cap, body.cut2,
-          a.status,
-          [&](int, const dvec4& qi, int j, double* acc) { body.pair(qi, j, acc); },
+          S, smem, R.D, a.ent + S.list_base, (unsigned)ta.list_cap, body.cut2, a.status,
+          [&](const dvec4& qi, int j, double* acc) { body.pair(qi, j, acc); },
           [&](int o, const double* acc) {
             if (HALF) body.add(S.gown0 + o, acc);
             else ((dvec4*)s_f)[o] = make_dvec4(acc[0], acc[1], acc[2], 0.0);

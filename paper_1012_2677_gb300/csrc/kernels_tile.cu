@@ -582,229 +582,6 @@ __global__ void k_tile_sizes_batch(const uint32_t* __restrict__ cs_in, TileArgs 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Adjoint pass over the list (the derivatives the reverse-time recurrences need), for the pair
-// energy u(s) of Eq. 2 as a function of s = r^2 (a = sigma^2 / s):
-//   u   = 4 eps (a^6 - a^3 + c2 s / sigma^2 + c0)
-//   u'  = du/ds   = 4 eps ((3 a^3 - 6 a^6) / s + c2 / sigma^2)
-//   u'' = d2u/ds2 = 4 eps (42 a^6 - 12 a^3) / s^2
-//   du/dsigma  = (4 eps / sigma) (12 a^6 - 6 a^3 - 2 c2 s / sigma^2)
-//   du'/dsigma = (4 eps / sigma) ((18 a^3 - 72 a^6) / s - 2 c2 / sigma^2)
-// (c2, c0 fixed: r_c scales with sigma).  Per key i, with d = x_j - x_i and dw = w_i - w_j:
-//   (H w)_i += 2 u' dw + 4 u'' d (d . dw)        (Hessian of the potential energy times w)
-//   F_i     += 2 u' d                              (force, = -dPE/dx_i)
-//   w . dF/dsigma += w_i . (2 du'/dsigma d),  w . dF/deps += w_i . (2 u' d) / eps
-//   PE += u / 2,  dPE/deps += u / (2 eps),  dPE/dsigma += (du/dsigma) / 2   (full list: each pair twice)
-// all zero for s >= r_c^2.  Block partials: [w.dF/deps, w.dF/dsigma, dPE/deps, dPE/dsigma, PE].
-constexpr int kAdjLanes = 4;
-constexpr int kAdjParts = 5;
-
-template <bool MIXED, bool WHOLE>
-__device__ __forceinline__ void adjoint_tile_compute(const TileShared& S, const unsigned char* buf, const TileLayout& L,
-                                                     const uint2* __restrict__ rows, const uint16_t* __restrict__ ent,
-                                                     const LJConst& c, const Geom& g, const dvec4* __restrict__ w,
-                                                     const float4* __restrict__ wf, dvec4* __restrict__ hw,
-                                                     dvec4* __restrict__ fo, int32_t* __restrict__ status, double* acc,
-                                                     int list_cap) {
-  const void* sh_pos = buf + L.pos;
-  const int* sh_gid = (const int*)(buf + L.gid);
-  const uint2* s_rows = (const uint2*)(buf + L.rows);
-  const uint16_t* s_ent = (const uint16_t*)(buf + L.ent);
-  const int lane = threadIdx.x & (kAdjLanes - 1);
-  const int grp = threadIdx.x / kAdjLanes;
-  constexpr int kGroups = kTileThreads / kAdjLanes;
-  const double e4 = 4.0 * c.eps, inv_sig = c.inv_sigma, c2s = c.c2s;
-  const int n_own = S.own1 - S.own0;
-  for (int o = grp; __any_sync(0xffffffffu, o < n_own); o += kGroups) {
-    const bool valid = o < n_own;
-    double h[3] = {0.0, 0.0, 0.0}, f[3] = {0.0, 0.0, 0.0}, q[kAdjParts] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    float ah[3] = {0.f, 0.f, 0.f}, af[3] = {0.f, 0.f, 0.f}, aq[kAdjParts] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    int gi = 0;
-    if (valid) {
-      const int l = S.own0 + o;
-      gi = S.gown0 + o;
-      uint2 row;
-      const uint16_t* el;
-      if (WHOLE) {
-        row = rows[gi];
-        el = ent;
-      } else {
-        row = s_rows[S.row_off + o];
-        row.x -= S.list_base;
-        el = row.x + row.y <= (unsigned)list_cap ? s_ent : ent + S.list_base;  // the end of a long segment stays in HBM
-        if (row.x + row.y > S.list_len) {
-          if (lane == 0) atomicOr(status, LJ_ST_LIST_OVERFLOW);
-          row.y = 0;
-        }
-      }
-      if (MIXED) {
-        const uint4 qi = ((const uint4*)sh_pos)[l];
-        const float e4f = c.e4, sig2f = c.sig2f, c2sf = c.c2sf, rc2f = c.rc2f, c0f = c.c0f, isgf = c.inv_sigmaf;
-        const float4 wif = wf[gi];  // the FP32 copy of w (no conversions per pair)
-        const float wx = wif.x, wy = wif.y, wz = wif.z;
-        for (unsigned e = lane; e < row.y; e += kAdjLanes) {
-          const int j = el[row.x + e];
-          const uint4 qj = ((const uint4*)sh_pos)[j];
-          // differences in sigma units: the integer difference in units of u, converted once and
-          // scaled by u (a power of two: exact)
-          const float dx = qd<WHOLE>(qj.x, qi.x, g) * g.qu, dy = qd<WHOLE>(qj.y, qi.y, g) * g.qu,
-                      dz = qd<WHOLE>(qj.z, qi.z, g) * g.qu;
-          const float s2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          if (!(s2 < rc2f)) continue;
-          const float4 wj = wf[qj.w];
-          const float is = rcp_nr(s2);
-          const float a = sig2f * is, a3 = a * a * a, a6 = a3 * a3;
-          const float u = e4f * (a6 - a3 + c2sf * s2 + c0f);
-          const float u1 = e4f * (is * (3.0f * a3 - 6.0f * a6) + c2sf);
-          const float u2 = e4f * is * is * (42.0f * a6 - 12.0f * a3);
-          const float dus = e4f * isgf * (12.0f * a6 - 6.0f * a3 - 2.0f * c2sf * s2);
-          const float du1s = e4f * isgf * (is * (18.0f * a3 - 72.0f * a6) - 2.0f * c2sf);
-          const float dwx = wx - wj.x, dwy = wy - wj.y, dwz = wz - wj.z;
-          const float ddw = dx * dwx + dy * dwy + dz * dwz;
-          const float t1 = 2.0f * u1, t2 = 4.0f * u2 * ddw;
-          ah[0] += t1 * dwx + t2 * dx;
-          ah[1] += t1 * dwy + t2 * dy;
-          ah[2] += t1 * dwz + t2 * dz;
-          af[0] += t1 * dx;
-          af[1] += t1 * dy;
-          af[2] += t1 * dz;
-          const float wd = wx * dx + wy * dy + wz * dz;
-          aq[0] += t1 * wd;
-          aq[1] += 2.0f * du1s * wd;
-          aq[2] += 0.5f * u;
-          aq[3] += 0.5f * dus;
-          aq[4] += 0.5f * u;
-        }
-      } else {
-        const dvec4 wi = w[gi];
-        const dvec4 qi = ((const dvec4*)sh_pos)[l];
-        for (unsigned e = lane; e < row.y; e += kAdjLanes) {
-          const int j = el[row.x + e];
-          const dvec4 qj = ((const dvec4*)sh_pos)[j];  // its image already in place (tiles)
-          double dx = qj.x - qi.x, dy = qj.y - qi.y, dz = qj.z - qi.z;
-          if (WHOLE) {
-            dx = fma(-rint(dx * g.inv_L64), g.L, dx);
-            dy = fma(-rint(dy * g.inv_L64), g.L, dy);
-            dz = fma(-rint(dz * g.inv_L64), g.L, dz);
-          }
-          const double s2 = fma(dx, dx, fma(dy, dy, dz * dz));
-          if (!(s2 < c.rc2)) continue;
-          const dvec4 wj = w[sh_gid[j]];
-          const double is = rcp_nr64(s2);
-          const double a = c.sig2 * is, a3 = a * a * a, a6 = a3 * a3;
-          const double u = e4 * (a6 - a3 + c2s * s2 + c.c0);
-          const double u1 = e4 * (is * (3.0 * a3 - 6.0 * a6) + c2s);
-          const double u2 = e4 * is * is * (42.0 * a6 - 12.0 * a3);
-          const double dus = e4 * inv_sig * (12.0 * a6 - 6.0 * a3 - 2.0 * c2s * s2);
-          const double du1s = e4 * inv_sig * (is * (18.0 * a3 - 72.0 * a6) - 2.0 * c2s);
-          const double dwx = wi.x - wj.x, dwy = wi.y - wj.y, dwz = wi.z - wj.z;
-          const double ddw = dx * dwx + dy * dwy + dz * dwz;
-          const double t1 = 2.0 * u1, t2 = 4.0 * u2 * ddw;
-          h[0] += t1 * dwx + t2 * dx;
-          h[1] += t1 * dwy + t2 * dy;
-          h[2] += t1 * dwz + t2 * dz;
-          f[0] += t1 * dx;
-          f[1] += t1 * dy;
-          f[2] += t1 * dz;
-          const double wd = wi.x * dx + wi.y * dy + wi.z * dz;
-          q[0] += t1 * wd;
-          q[1] += 2.0 * du1s * wd;
-          q[2] += 0.5 * u;
-          q[3] += 0.5 * dus;
-          q[4] += 0.5 * u;
-        }
-      }
-    }
-    if (MIXED) {  // the group's lanes reduce in FP32; one lane converts and accumulates in FP64
-      for (int k = 0; k < 3; ++k) {
-        ah[k] = gsum<kAdjLanes>(ah[k]);
-        af[k] = gsum<kAdjLanes>(af[k]);
-      }
-      for (int k = 0; k < kAdjParts; ++k) aq[k] = gsum<kAdjLanes>(aq[k]);
-      if (valid && lane == 0) {
-        hw[gi] = make_dvec4(ah[0], ah[1], ah[2], 0.0);
-        if (fo) fo[gi] = make_dvec4(af[0], af[1], af[2], 0.0);
-        for (int k = 0; k < kAdjParts; ++k) acc[k] += (double)aq[k];
-      }
-    } else {
-      for (int k = 0; k < 3; ++k) {
-        h[k] = gsum<kAdjLanes>(h[k]);
-        f[k] = gsum<kAdjLanes>(f[k]);
-      }
-      if (valid && lane == 0) {
-        hw[gi] = make_dvec4(h[0], h[1], h[2], 0.0);
-        if (fo) fo[gi] = make_dvec4(f[0], f[1], f[2], 0.0);
-      }
-      for (int k = 0; k < kAdjParts; ++k) acc[k] += q[k];
-    }
-  }
-}
-
-template <bool MIXED, bool WHOLE>
-__global__ void __launch_bounds__(kTileThreads, 2)
-    k_adjoint_tile(const void* __restrict__ pos, const uint32_t* __restrict__ cs, int64_t N, Geom g, TileArgs ta,
-                   LJConst c, const uint2* __restrict__ rows,
-                   const uint2* __restrict__ tile_list, const uint16_t* __restrict__ ent,
-                   const dvec4* __restrict__ w, const float4* __restrict__ wf, dvec4* __restrict__ hw,
-                   dvec4* __restrict__ fo, double* __restrict__ part, unsigned int* __restrict__ ticket,
-                   double* __restrict__ sums, int32_t* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ TileShared S;
-  __shared__ __align__(8) uint64_t bar;
-  const TileLayout L = tile_layout(ta, MIXED, true, !MIXED);
-  double acc[kAdjParts] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (WHOLE) {
-    if (blockIdx.x == 0) {
-      stage_whole<MIXED, !MIXED>(N, pos, S, smem, L);
-      __syncthreads();
-      adjoint_tile_compute<MIXED, true>(S, smem, L, rows, ent, c, g, w, wf, hw, fo, status, acc, ta.list_cap);
-    }
-  } else {
-    if (threadIdx.x == 0) {
-      mbar_init(&bar, 1);
-      fence_proxy_async_smem();
-    }
-    __syncthreads();
-    uint32_t ph = 0;
-    for (int64_t t = blockIdx.x; t < ta.ntiles; t += gridDim.x) {
-      const bool ok = force_tile_prepare(tile_info(t, ta), t, ta, cs, tile_list, S, status);
-      if (ok) {
-        const TileInfo ti = tile_info(t, ta);
-        stage_issue<MIXED, true>(ti, ta, pos, rows, ent, S, smem, L, &bar);
-        if (!stage_finish<MIXED, true>(ti, ta, g, S, smem, L, &bar, ph, !MIXED, status)) return;
-        adjoint_tile_compute<MIXED, false>(S, smem, L, rows, ent, c, g, w, wf, hw, fo, status, acc, ta.list_cap);
-      }
-      __syncthreads();
-    }
-  }
-  __shared__ double sh[32];
-  for (int k = 0; k < kAdjParts; ++k) {
-    const double t = block_sum(acc[k], sh);
-    if (threadIdx.x == 0) part[kAdjParts * (size_t)blockIdx.x + k] = t;
-    __syncthreads();
-  }
-  // the last CTA to finish sums the partials of all CTAs in block order (thread 0 wrote this CTA's
-  // partials and orders them before its ticket)
-  __shared__ int s_last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    for (int k = 0; k < kAdjParts; ++k) {
-      double v = 0.0;
-      for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) v += __ldcg(part + kAdjParts * (size_t)b + k);
-      v = block_sum(v, sh);
-      if (threadIdx.x == 0) sums[k] = v;
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) *ticket = 0u;
-  }
-}
-
-
-// ---------------------------------------------------------------------------------------------
 // Expand the list into (key, partner) sorted-index pairs (for inspection).  The whole-box case
 // is a template parameter: no barrier sits under a runtime branch.
 template <bool WHOLE>
@@ -861,7 +638,7 @@ int set_wait_budget(long long cycles) {
   const long long v = cycles > 0 ? cycles : kWaitBudget;
   if (cudaDeviceSynchronize() != cudaSuccess) return -1;
   if (set_unit_wait_budget(v) || set_wait_budget_force(v) || set_wait_budget_force_half(v) ||
-      set_wait_budget_force_dp(v) || set_wait_budget_resident(v))
+      set_wait_budget_force_dp(v) || set_wait_budget_resident(v) || set_wait_budget_adjoint(v))
     return -1;
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : -1;
 }
@@ -969,35 +746,6 @@ void launch_max_count(const uint32_t* cnt, int64_t n, unsigned int* out, cudaStr
   if (b > 4096) b = 4096;
   k_max_count<<<(int)b, 256, 0, s>>>(cnt, n, out);
 }
-
-size_t adjoint_smem_bytes(const TileArgs& ta, int precision) {
-  return align16(tile_layout(ta, precision == LJ_MIXED, true, precision != LJ_MIXED).total);
-}
-
-int launch_adjoint_tile(int precision, const void* pos, const uint32_t* cs, int64_t N, Geom g, TileArgs ta, LJConst c,
-                        const uint2* rows, const uint2* tile_list, const uint16_t* ent, const void* w,
-                        const float4* wf, void* hw, void* fo, double* part, unsigned int* ticket, double* sums,
-                        int32_t* status, cudaStream_t s) {
-  const size_t sm = adjoint_smem_bytes(ta, precision);
-  const int grid = tile_grid(ta, min(per_sm_for(sm), 2));
-#define LJ_ADJ_LAUNCH(M, W)                                                                                 \
-  do {                                                                                                      \
-    set_smem(k_adjoint_tile<M, W>, sm);                                                                     \
-    k_adjoint_tile<M, W><<<grid, kTileThreads, sm, s>>>(pos, cs, N, g, ta, c, rows, tile_list, ent,         \
-                                                        (const dvec4*)w, wf, (dvec4*)hw, (dvec4*)fo, part,      \
-                                                        ticket, sums, status);                                  \
-  } while (0)
-  if (precision == LJ_MIXED) {
-    if (ta.whole) LJ_ADJ_LAUNCH(true, true);
-    else LJ_ADJ_LAUNCH(true, false);
-  } else {
-    if (ta.whole) LJ_ADJ_LAUNCH(false, true);
-    else LJ_ADJ_LAUNCH(false, false);
-  }
-#undef LJ_ADJ_LAUNCH
-  return grid;
-}
-
 
 // ---- batched replicas -----------------------------------------------------------------------
 size_t batch_list_smem_bytes(const TileArgs& caps) { return win_layout(caps).total; }

@@ -1583,25 +1583,30 @@ static int ensure_adjoint(ljmd_sys* s) {
   return LJ_OK;
 }
 
+// One adjoint launch at the current position copies with s->adj_w.
+static void adjoint_launch(ljmd_sys* s, const AdjointOut& out) {
+  PhaseTimer timer(s, PH_ADJOINT);
+  launch_adjoint_tile(s->precision, force_pos(s), s->cell_start, s->n, s->g, s->ta, s->c, s->rows, s->tile_list, s->ent,
+                      s->adj_w, s->adj_wf, out, s->part_adj, s->adj_ticket, s->d_adj, s->d_status, s->st);
+  s->launches += 1;
+}
+
 // One adjoint pass at the current positions with the vector w (device, id order; null = 0):
 // hw = H w and f = F (device, id order; either may be null), q = [w.F, w.dF/dsigma, PE,
 // dPE/dsigma, PE] (w.dF/deps = w.F / eps, dPE/deps = PE / eps).  With q non-null the sums are read
 // to the host (synchronises); with q null they stay in the device scalars s->d_adj[0..4].
-static int adjoint_pass(ljmd_sys* s, const double* w_id, double* hw_id, double* f_id, double* q,
-                        bool f_sorted = false) {
+static int adjoint_pass(ljmd_sys* s, const double* w_id, double* hw_id, double* f_id, double* q) {
   ljmd_sys* sys = s;
   if (!s->have_list) TRY(rebuild(s));
   TRY(ensure_adjoint(s));
   const int64_t N = s->n;
   cudaStream_t st = s->st;
   launch_to_sorted(w_id, s->id, N, s->adj_w, s->adj_wf, st);
-  {
-    PhaseTimer timer(s, PH_ADJOINT);
-    launch_adjoint_tile(s->precision, force_pos(s), s->cell_start, N, s->g, s->ta, s->c, s->rows, s->tile_list,
-                        s->ent, s->adj_w, s->adj_wf, s->adj_hw, (f_id || f_sorted) ? s->adj_f : nullptr, s->part_adj,
-                        s->adj_ticket, s->d_adj, s->d_status, st);
-  }
-  s->launches += 2;
+  s->launches += 1;
+  AdjointOut out{};
+  out.hw = s->adj_hw;
+  out.fo = f_id ? s->adj_f : nullptr;
+  adjoint_launch(s, out);
   if (hw_id) {
     launch_scatter_back_f64x4_to_f64x3(s->adj_hw, hw_id, s->id, N, st);
     s->launches += 1;
@@ -1638,9 +1643,7 @@ struct DevBuf {  // device scratch owned by one call
 // current order and image counts are kept, the force kernels' copies are rewritten, and the list
 // stays if no particle moved more than margin/2 from where it was built (else it is rebuilt).
 // Velocities are left as they are.  Synchronises once (the displacement maximum).
-// known_valid: the state was reached by a step that the validity rule accepted for the current list
-// (no rebuild since), so its displacement need not be read back.
-static int load_keeping_list(ljmd_sys* s, const double* u, bool known_valid = false) {
+static int load_keeping_list(ljmd_sys* s, const double* u) {
   ljmd_sys* sys = s;
   if (!s->have_list) {  // nothing to keep: the general path
     return ljmd_set_state(s, s->n, s->L, u, nullptr, 1);
@@ -1648,14 +1651,13 @@ static int load_keeping_list(ljmd_sys* s, const double* u, bool known_valid = fa
   launch_load_unwrapped(u, s->img, s->id, s->n, s->g.offset, s->L, s->x, s->st);
   s->launches += 1;
   CKL();
-  if (!known_valid) CK(cudaMemsetAsync(s->d_dmax, 0, 8, s->st));  // (a run clears it before its use)
+  CK(cudaMemsetAsync(s->d_dmax, 0, 8, s->st));
   IntegrateArgs a{0.0, 0.0, 0.0, 0, 1};  // no kick, no drift: copies and displacement only
   integrate(s, a);
   CKL();
   s->forces_current = false;
   s->pe_step = -1;
   s->energy_step = -1;
-  if (known_valid) return LJ_OK;
   TRY(read_dmax(s, &s->last_dmax));
   if (s->last_dmax > s->disp_limit) TRY(rebuild(s));
   return LJ_OK;
@@ -1846,22 +1848,45 @@ int ljmd_traj_loss_grad(ljmd_sys* sys, int64_t n, double box, const double* x0, 
     const int64_t valid_from = sys->last_build_step;
     const int64_t builds = sys->rebuilds;
     for (int64_t t = t1 - 1; t >= t0; --t) {
-      launch_axpy(lv.p, dt, lx.p, (int64_t)n3, st);  // x_{t+1} = x_t + dt v'
-      // state t in the particle order of the recomputation: its list is kept while it is valid
-      TRY(load_keeping_list(sys, seg_x.p + n3 * (size_t)(t - t0), t - t0 >= valid_from && sys->rebuilds == builds));
+      // x_{t+1} = x_t + dt v': lv += dt lx; state t in the particle order of the recomputation (its list is
+      // kept while it is valid) and lv in that order
+      const double* u = seg_x.p + n3 * (size_t)(t - t0);
+      TRY(ensure_adjoint(sys));
+      if (t - t0 >= valid_from && sys->rebuilds == builds && sys->have_list) {
+        launch_adjoint_prepare(u, lv.p, lx.p, dt, sys->img, sys->id, sys->n, sys->g.offset, sys->L, sys->g.qk, sys->x,
+                               sys->xq, sys->pos64, sys->adj_w, sys->adj_wf, st);
+        sys->launches += 1;
+        sys->forces_current = false;
+        sys->pe_step = -1;
+        sys->energy_step = -1;
+      } else {
+        launch_axpy(lv.p, dt, lx.p, (int64_t)n3, st);
+        TRY(load_keeping_list(sys, u));
+        if (!sys->have_list) TRY(rebuild(sys));
+        launch_to_sorted(lv.p, sys->id, sys->n, sys->adj_w, sys->adj_wf, st);
+        sys->launches += 2;
+      }
+      CKL();
       const double c = t == 0 ? h : dt;  // both half-kicks touching state t (one at t = 0)
       const bool in_pe = t > nsteps - n_pe;
-      // H lv (and F where the PE term needs it) in the sorted order, then lx -= c H lv + wpe F
-      TRY(adjoint_pass(sys, lv.p, nullptr, nullptr, nullptr, in_pe));
-      launch_adjoint_update(sys->adj_hw, in_pe ? sys->adj_f : nullptr, sys->id, sys->n, c, in_pe ? wpe : 0.0, lx.p,
-                            st);
-      launch_accum_q(sys->d_adj, c / eps, c, in_pe ? wpe : 0.0, in_pe ? wpe / eps : 0.0, gthd.p, st);
+      // lx -= c H lv + wpe F (F where the PE term needs it), the parameter gradient's terms
+      AdjointOut out{};
+      out.lx = lx.p;
+      out.id = sys->id;
+      out.c = c;
+      out.a = in_pe ? wpe : 0.0;
+      out.gth = gthd.p;
+      out.g0 = c / eps;
+      out.g1 = c;
+      out.g3 = in_pe ? wpe : 0.0;
+      out.g4 = in_pe ? wpe / eps : 0.0;
+      adjoint_launch(sys, out);
       if (t == 0) {
         // MSD term at t = 0: -2 (x_n - x_0) / N
         launch_scaled_diff(b.p, -2.0 / (double)n, xNu.p, x0u.p, (int64_t)n3, st);
         launch_axpy(lx.p, 1.0, b.p, (int64_t)n3, st);
       }
-      sys->launches += 3 + (t == 0 ? 2 : 0);
+      sys->launches += t == 0 ? 2 : 0;
       CKL();
     }
   }

@@ -180,14 +180,26 @@ int launch_force_fp64(int half, ForceLaunch& a);  // returns the grid launched
 size_t dp_force_smem_bytes(const TileArgs& ta, int half);
 bool dp_fits(const TileArgs& ta);
 size_t adjoint_smem_bytes(const TileArgs& ta, int precision);
-// Adjoint pass (HVP, forces, parameter derivatives) over the list; w, hw, fo are dvec4 [N] in sorted
-// order (fo may be null), wf the FP32 copy of w (read by the mixed form).  Writes 5 partials per
-// block [w.dF/deps, w.dF/dsigma, dPE/deps, dPE/dsigma, PE]; the last block to finish (ticket: zero
-// between launches) writes their sums, in block order, to sums[0..4].  Returns the number of blocks.
+// Where an adjoint pass puts its results.  hw, fo: dvec4 [N] in sorted order (fo may be null); or, with
+// lx non-null, the position adjoint in id order is updated instead, lx[3 id + k] -= c (H w).k + a F.k.
+// gth non-null: the parameter gradient takes gth[0] += g0 q[0] + g4 q[4], gth[1] += g1 q[1] + g3 q[3].
+struct AdjointOut {
+  void *hw, *fo;
+  double* lx;
+  const int32_t* id;
+  double c, a;
+  double* gth;
+  double g0, g1, g3, g4;
+};
+// Adjoint pass (HVP, forces, parameter derivatives) over the list; w is dvec4 [N] in sorted order, wf its
+// FP32 copy (read by the mixed form).  Writes 5 partials per block [w.dF/deps, w.dF/dsigma, dPE/deps,
+// dPE/dsigma, PE]; the last block to finish (ticket: zero between launches) writes their sums, in block
+// order, to sums[0..4].  Returns the number of blocks.
 int launch_adjoint_tile(int precision, const void* pos, const uint32_t* cs, int64_t N, Geom g, TileArgs ta, LJConst c,
                         const uint2* rows, const uint2* tile_list, const uint16_t* ent, const void* w,
-                        const float4* wf, void* hw, void* fo, double* part, unsigned int* ticket, double* sums,
+                        const float4* wf, const AdjointOut& out, double* part, unsigned int* ticket, double* sums,
                         int32_t* status, cudaStream_t s);
+int set_wait_budget_adjoint(long long cycles);
 void launch_list_decode(const uint32_t* cs, int64_t N, TileArgs ta, const uint2* rows, const uint16_t* ent,
                         uint64_t E, uint32_t* out, int32_t* status, cudaStream_t s);
 
@@ -310,9 +322,12 @@ void launch_unwrapped(const double* x, const int32_t* img, const int32_t* id, in
 void launch_load_unwrapped(const double* u, const int32_t* img, const int32_t* id, int64_t N, double offset, double L,
                            double* x, cudaStream_t s);
 void launch_axpy(double* y, double a, const double* x, int64_t n, cudaStream_t s);
-// lx[3 id[s] + k] -= c hw[s].k + a f[s].k over the sorted order (f null: a ignored).
-void launch_adjoint_update(const dvec4* hw, const dvec4* f, const int32_t* id, int64_t N, double c, double a,
-                           double* lx, cudaStream_t s);
+// The state before an adjoint pass of the reverse recurrences, in one launch: lv += dt lx (id order); w and
+// its FP32 copy = lv in the sorted order; x (sorted) = offset + u - img L from the unwrapped positions u (id
+// order) and the force kernels' position copies of it (xq at u = 2^-qk, or pos64).
+void launch_adjoint_prepare(const double* u, double* lv, const double* lx, double dt, const int32_t* img,
+                            const int32_t* id, int64_t N, double offset, double L, int qk, double* x, uint4* xq,
+                            dvec4* pos64, dvec4* w, float4* wf, cudaStream_t s);
 // gth[0] += a0 q[0] + a4 q[4], gth[1] += a1 q[1] + a3 q[3] (device scalars)
 void launch_accum_q(const double* q, double a0, double a1, double a3, double a4, double* gth, cudaStream_t s);
 void launch_scaled_diff(double* y, double a, const double* u, const double* w, int64_t n, cudaStream_t s);

@@ -868,27 +868,28 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 }
 
 // ---------------------------------------------------------------------------------------------
-// FP64 pair work on staged tiles.  The FP64 pipe takes 2 lanes per clock per SM on this part (1/64 of
-// the FP32 rate), whatever the number of active lanes, so it is given the pairs inside r_c alone and
-// full warps of them.  A warp takes a run of consecutive keys.  It first filters their rows in FP32
+// Pair work by queues.  A warp takes a run of consecutive keys.  It first filters their rows in FP32
 // (differences of fixed-point copies, r_c^2 widened by a relative 4e-6 against the 3e-7 that the
 // quantisation and FP32 rounding can err) and queues the kept (key, partner) pairs in shared memory;
 // then each lane evaluates a contiguous share of the queue, so that at most the last pair of a lane
 // idles and a key's sum needs no shuffles.  A lane stores the partial sum of a key that began in an earlier
 // lane in its head slot, every other one in the key's slot; the key's own lane adds slot and heads in
-// lane order, so the sums do not depend on timing.  The exact r^2 < r_c^2 test is still the FP64 one.
+// lane order, so the sums do not depend on timing.  The exact r^2 < r_c^2 test is still the pair's own.
+// This pays where a pair inside r_c is dear against the filter: in the FP64 form (the FP64 pipe takes 2
+// lanes per clock per SM, 1/64 of the FP32 rate, whatever the number of active lanes) and in the adjoint
+// pass (about 75 instructions a pair).
 constexpr int kDpThreads = 128;
 constexpr int kDpWarps = kDpThreads / 32;
-constexpr int kDpQueue = 288;  // queued pairs per warp: nine a lane (the smallest that keeps four CTAs per SM)
+constexpr int kDpQueue = 288;  // queued pairs per warp: nine a lane (the smallest that keeps four FP64 CTAs per SM)
 
-template <int NACC, bool DIRECT>
+template <class T, int NACC, bool DIRECT>
 struct DpWarp {
-  double seg[32][NACC];   // per key: the partial sum of the lane in which its run begins
-  double head[32][NACC];  // per lane: the partial sum of a run begun in an earlier lane
-  uint32_t q[kDpQueue];   // key of the warp's run << 16 | staged partner
+  T seg[32][NACC];       // per key: the partial sum of the lane in which its run begins
+  T head[32][NACC];      // per lane: the partial sum of a run begun in an earlier lane
+  uint32_t q[kDpQueue];  // key of the warp's run << 16 | staged partner
 };
-template <int NACC>
-struct DpWarp<NACC, true> {
+template <class T, int NACC>
+struct DpWarp<T, NACC, true> {
   uint32_t q[kDpQueue];
 };
 
@@ -911,7 +912,7 @@ __host__ __device__ __forceinline__ DpLayout dp_layout(const TileArgs& ta) {
   D.L.ent = D.L.cnt = o;
   o += align16(2 * (size_t)ta.list_cap);
   D.warp = o;
-  o += sizeof(DpWarp<NACC, DIRECT>) * kDpWarps;
+  o += sizeof(DpWarp<double, NACC, DIRECT>) * kDpWarps;
   D.total = D.L.total = align16(o);
   return D;
 }
@@ -968,59 +969,66 @@ __device__ __forceinline__ bool dp_stage_finish(const TileInfo& ti, const TileAr
   return true;
 }
 
-// The listed pairs of a staged tile's keys inside r_c (or within the filter's margin of it).
-// pair(key slot, qi, partner slot, acc) adds one pair to the key's NACC sums; done(o, acc) receives
-// the sums of own key o.
-// ent_s: the staged part of the tile's segment, its first cap entries; rows beyond it are read from ent_g.
+// The listed pairs of a staged tile's keys inside r_c (or within the filter's margin of it), NW warps.
+// sq: the staged records; W: the warp's queue.  key(o) loads what a pair needs of own key o, partner(slot)
+// what it needs of the partner (a pair ahead of its use), pair(key, partner, acc) adds one pair to the key's
+// NACC sums, done(o, acc) receives the sums of own key o, batch() is called by every lane after its share
+// of a queue.  ent_s: the staged part of the tile's segment, its first
+// cap entries; rows beyond it are read from ent_g.
 // DIRECT: done(o, acc) is called by the lanes themselves with each partial sum (it must add atomically).
-template <int NACC, bool DIRECT, class Pair, class Done>
-__device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigned char* smem, const DpLayout& D,
-                                              const uint16_t* ent_s, const uint16_t* ent_g, unsigned cap, float cut2,
-                                              int32_t* status, Pair&& pair, Done&& done) {
+template <class T, int NACC, bool DIRECT, int NW, class Key, class Partner, class Pair, class Done, class Batch>
+__device__ __forceinline__ void queue_tile_pairs(const TileShared& S, const uint4* sq, const uint2* s_rows,
+                                                 DpWarp<T, NACC, DIRECT>& W, const uint16_t* ent_s,
+                                                 const uint16_t* ent_g, unsigned cap, float cut2, int32_t* status,
+                                                 Key&& key, Partner&& partner, Pair&& pair, Done&& done,
+                                                 Batch&& batch) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const uint4* sq = (const uint4*)(smem + D.xq);
-  const dvec4* sp = (const dvec4*)(smem + D.L.pos);
-  const uint2* s_rows = (const uint2*)(smem + D.L.rows) + S.row_off;
-  auto& W = ((DpWarp<NACC, DIRECT>*)(smem + D.warp))[warp];
+  s_rows += S.row_off;
   const int n_own = S.own1 - S.own0;
-  const int per = min(32, (n_own + kDpWarps - 1) / kDpWarps);  // keys per warp and turn
-  for (int b0 = warp * per; b0 < n_own; b0 += kDpWarps * per) {
+  const int per = min(32, (n_own + NW - 1) / NW);  // keys per warp and turn
+  for (int b0 = warp * per; b0 < n_own; b0 += NW * per) {
     const int nk = min(per, n_own - b0);
-    double tot[NACC];  // lane k: the sums of key b0 + k
+    T tot[NACC];  // lane k: the sums of key b0 + k
 #pragma unroll
-    for (int q = 0; q < NACC; ++q) tot[q] = 0.0;
+    for (int q = 0; q < NACC; ++q) tot[q] = T(0);
     int ka = 0, kb = 0, cnt = 0;  // lane k: the key's range of the queue; queued pairs
     auto drain = [&]() {
       __syncwarp();
       const int c = (cnt + 31) >> 5, lo = lane * c, hi = min(lo + c, cnt);
-      double acc[NACC];
+      T acc[NACC];
       int kc = -1;
       bool head = lo > 0 && lo < cnt && (W.q[lo - 1] >> 16) == (W.q[lo] >> 16);
-      dvec4 qi = make_dvec4(0.0, 0.0, 0.0, 0.0);
+      auto ki = key(b0);
       auto put = [&]() {
         if constexpr (DIRECT) {
           done(b0 + kc, acc);
         } else {
-          double* dst = head ? W.head[lane] : W.seg[kc];
+          T* dst = head ? W.head[lane] : W.seg[kc];
 #pragma unroll
           for (int q = 0; q < NACC; ++q) dst[q] = acc[q];
           head = false;
         }
       };
+      uint32_t w = lo < hi ? W.q[lo] : 0u;
+      auto pj = partner((int)(w & 0xffffu));
       for (int t = lo; t < hi; ++t) {
-        const uint32_t w = W.q[t];
+        const uint32_t wn = t + 1 < hi ? W.q[t + 1] : w;
+        const auto pn = partner((int)(wn & 0xffffu));
         const int k = (int)(w >> 16);
         if (k != kc) {
           if (kc >= 0) put();
           kc = k;
-          qi = sp[S.own0 + b0 + k];
+          ki = key(b0 + k);
 #pragma unroll
-          for (int q = 0; q < NACC; ++q) acc[q] = 0.0;
+          for (int q = 0; q < NACC; ++q) acc[q] = T(0);
         }
-        pair(b0 + k, qi, (int)(w & 0xffffu), acc);
+        pair(ki, pj, acc);
+        w = wn;
+        pj = pn;
       }
       if (kc >= 0) put();
+      batch();
       __syncwarp();
       if constexpr (!DIRECT) {
         if (kb > ka) {
@@ -1075,6 +1083,18 @@ __device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigne
       if (lane < nk) done(b0 + lane, tot);
     }
   }
+}
+
+// The same on a staged FP64 tile: pair(FP64 position of the key, partner slot, acc).
+template <int NACC, bool DIRECT, class Pair, class Done>
+__device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigned char* smem, const DpLayout& D,
+                                              const uint16_t* ent_g, unsigned cap, float cut2, int32_t* status,
+                                              Pair&& pair, Done&& done) {
+  const dvec4* sp = (const dvec4*)(smem + D.L.pos) + S.own0;
+  queue_tile_pairs<double, NACC, DIRECT, kDpWarps>(
+      S, (const uint4*)(smem + D.xq), (const uint2*)(smem + D.L.rows),
+      ((DpWarp<double, NACC, DIRECT>*)(smem + D.warp))[threadIdx.x >> 5], (const uint16_t*)(smem + D.L.ent), ent_g, cap,
+      cut2, status, [&](int o) { return sp[o]; }, [](int j) { return j; }, pair, done, [] {});
 }
 
 // The FP64 comparison r^2 < r_c^2 of two non-negative values by their bit patterns (the order is the

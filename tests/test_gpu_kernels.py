@@ -32,6 +32,30 @@ def test_fp64_tiles(M, rho, rc, margin, list_form):
     assert gpe == pytest.approx(pe, rel=1e-12) and gvir == pytest.approx(vir, rel=1e-12)
 
 
+@pytest.mark.parametrize("precision,tol", [(ljmd.LJ_MIXED, 2e-4), (ljmd.LJ_FP64, 1e-10)])
+@pytest.mark.parametrize("M,rho,rc,margin", [
+    (5, 1.0, 2.5, 0.6),    # fewer than three cells per side: no tiles
+    (6, 0.5, 2.5, 0.5),    # 3 cells per side: fewer keys than a warp's turn
+    (10, 0.9, 3.5, 1.0),   # long rows, segments beyond shared memory
+    (11, 0.9, 4.5, 1.0),   # beyond the FP64 queue kernel's tile
+])
+def test_adjoint_tiles(M, rho, rc, margin, precision, tol):
+    """Tolerances of the other tests of the Hessian-vector product and the parameter derivatives."""
+    p = O.LJParams(rc_over_sigma=rc)
+    x, L = O.fcc_lattice(M, rho)
+    x = synth.dyadic(O.wrap(x + synth.displacements(len(x), 0.06, 3), L))
+    w = synth.gaussian((len(x), 3), 11)
+    ref = O.hvp(x, L, w, p)
+    dpe, vjp = O.param_derivs(x, L, p, lam=w)
+    with ljmd.System(cutoff=rc, margin=margin, precision=precision) as s:
+        s.set_state(x, None, L)
+        hw, dth = s.hvp(w)
+    rms = np.sqrt((ref ** 2).sum(1).mean())
+    assert np.sqrt(((hw - ref) ** 2).sum(1)).max() / rms <= tol
+    for got, want in zip(dth, (vjp[0], vjp[1], dpe[0], dpe[1])):
+        assert got == pytest.approx(want, rel=max(tol, 1e-12), abs=tol * 1e-3 * abs(dpe[0]))
+
+
 @pytest.mark.parametrize("precision,list_form", [(ljmd.LJ_MIXED, ljmd.LJ_LIST_FULL), (ljmd.LJ_MIXED, ljmd.LJ_LIST_HALF),
                                                  (ljmd.LJ_FP64, ljmd.LJ_LIST_FULL), (ljmd.LJ_FP64, ljmd.LJ_LIST_HALF)])
 @pytest.mark.parametrize("M,rho,every,mode,steps", [
