@@ -132,6 +132,9 @@ __device__ __forceinline__ bool finite_d(double v) {
   return (__double_as_longlong(v) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
 }
 
+// v == 0 by its bits (a comparison of doubles takes a slot of the FP64 pipe).
+__device__ __forceinline__ bool is_zero_d(double v) { return (__double_as_longlong(v) << 1) == 0; }
+
 __device__ __forceinline__ bool finite_f(float v) {
   return (__float_as_int(v) & 0x7f800000) != 0x7f800000;
 }
@@ -206,6 +209,56 @@ __device__ __forceinline__ uint32_t fixq(double xs, int qk) {
 // Difference of two fixed-point coordinates as an FP32 number of units u (one rounding, to 24
 // significant bits; the integer difference itself is exact modulo 2^32).
 __device__ __forceinline__ float qdiff(uint32_t a, uint32_t b) { return __int2float_rn((int)(a - b)); }
+
+// The list-validity decision of a device-decided run (the host rule of ljmd_step, taken on the
+// device so that steps follow each other without a host round trip): the largest squared
+// displacement and drift speed of the step are taken (and reset for the next one); with the
+// margin/2 rule the list expired when the displacement exceeds the limit, with DUTC when the
+// remaining buffer, less the closing 2 v_max dt of the step, is used up.  An expired list stops
+// the run at step s.  One thread.
+__device__ __forceinline__ void step_check_one(uint32_t* dmax_bits, StepCtl* ctl, int s, double disp_limit, int dutc,
+                                               double two_dt) {
+  if (ctl->stop) return;
+  const float d2 = __uint_as_float(atomicExch(dmax_bits, 0u)), v2 = __uint_as_float(atomicExch(dmax_bits + 1, 0u));
+  ctl->last[0] = d2;
+  ctl->last[1] = v2;
+  bool expired;
+  if (dutc) {
+    const double b = ctl->dutc - two_dt * sqrt((double)v2) * (1.0 + 1e-6);
+    ctl->dutc = b;
+    expired = !(b > 0.0);
+  } else {
+    expired = sqrt((double)d2) > disp_limit;
+  }
+  if (expired) {
+    ctl->stop = 1;
+    ctl->stop_at = s;
+  }
+}
+
+// The end of an integrating kernel whose CTAs have written their kinetic energies (thread 0) and raised the
+// maxima: the last CTA to finish takes the energy record and the validity check.  The whole block.
+__device__ __forceinline__ void step_finish(const StepFinish& fin, double* ke_part, uint32_t* dmax_bits) {
+  // thread 0 wrote the CTA's partials (the maxima went by device-wide atomics): it alone orders
+  // those writes before its ticket
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(fin.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    if (fin.rec)
+      energy_record_block(fin.pv, fin.nbf, ke_part, gridDim.x, fin.pe_scale, fin.energies, fin.log, fin.cap, fin.count,
+                          fin.step);
+    if (threadIdx.x == 0) {
+      if (fin.check) step_check_one(dmax_bits, fin.ctl, fin.s, fin.disp_limit, fin.dutc, fin.two_dt);
+      *fin.ticket = 0u;
+    }
+  }
+}
 
 // ---- asynchronous bulk copies into shared memory (cp.async.bulk + mbarrier, sm_90 and later) ----
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

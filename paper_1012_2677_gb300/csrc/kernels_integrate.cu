@@ -13,69 +13,9 @@
 // In the mixed form every FP32 <-> FP64 conversion is done with integer operations (exact for
 // FP32 -> FP64, rounded to nearest for FP64 -> FP32), which keeps the FP64 pipe for the seven
 // operations per particle that need it.
-#include "common.cuh"
+#include "integrate.cuh"
 
 namespace ljmd {
-
-// The list-validity decision of a device-decided run (the host rule of ljmd_step, taken on the
-// device so that steps follow each other without a host round trip): the largest squared
-// displacement and drift speed of the step are taken (and reset for the next one); with the
-// margin/2 rule the list expired when the displacement exceeds the limit, with DUTC when the
-// remaining buffer, less the closing 2 v_max dt of the step, is used up.  An expired list stops
-// the run at step s.  One thread.
-__device__ __forceinline__ void step_check_one(uint32_t* dmax_bits, StepCtl* ctl, int s, double disp_limit, int dutc,
-                                               double two_dt) {
-  if (ctl->stop) return;
-  const float d2 = __uint_as_float(atomicExch(dmax_bits, 0u)), v2 = __uint_as_float(atomicExch(dmax_bits + 1, 0u));
-  ctl->last[0] = d2;
-  ctl->last[1] = v2;
-  bool expired;
-  if (dutc) {
-    const double b = ctl->dutc - two_dt * sqrt((double)v2) * (1.0 + 1e-6);
-    ctl->dutc = b;
-    expired = !(b > 0.0);
-  } else {
-    expired = sqrt((double)d2) > disp_limit;
-  }
-  if (expired) {
-    ctl->stop = 1;
-    ctl->stop_at = s;
-  }
-}
-
-// One particle's inputs to the integrator: force, velocity, position and (when the position copy is
-// rewritten) the displacement reference.
-template <bool MIXED>
-struct IntegrateIn;
-template <>
-struct IntegrateIn<true> {
-  float4 f;
-  uint4 r;
-  double v[3], x[3];
-};
-template <>
-struct IntegrateIn<false> {
-  dvec4 f, r;
-  double v[3], x[3];
-};
-
-template <bool MIXED>
-__device__ __forceinline__ void integrate_load(IntegrateIn<MIXED>& in, const double* __restrict__ x,
-                                               const double* __restrict__ v, const void* __restrict__ fptr,
-                                               const void* __restrict__ refp, int64_t N, int64_t i, int shadow) {
-  if constexpr (MIXED) {
-    in.f = ((const float4*)fptr)[i];
-    if (shadow) in.r = ((const uint4*)refp)[i];
-  } else {
-    in.f = ((const dvec4*)fptr)[i];
-    if (shadow) in.r = ((const dvec4*)refp)[i];
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    in.v[k] = v[k * N + i];
-    in.x[k] = x[k * N + i];
-  }
-}
 
 // Hint that the lines holding particle j's inputs be brought into L2 (one prefetch per stream; no
 // registers are held for the data).
@@ -110,12 +50,7 @@ __global__ void __launch_bounds__(256) k_integrate(double* __restrict__ x, doubl
                                                    int32_t* __restrict__ status, StepFinish fin,
                                                    const int* __restrict__ skip) {
   if (skip && *skip) return;  // a device-decided run stopped before this step
-  const float qu = __int_as_float((127 - a.qk) << 23);  // u = 2^-qk
-  const double kk = a.kpre + a.kpost;
-  const float kpre_f = (float)a.kpre;
-  double ke_acc = 0.0;
-  float d2max = 0.0f, v2max = 0.0f;
-  bool bad = false;
+  IntegrateAcc acc;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   IntegrateIn<MIXED> cur = {};
@@ -125,78 +60,18 @@ __global__ void __launch_bounds__(256) k_integrate(double* __restrict__ x, doubl
     if (i + stride < N) integrate_load<MIXED>(nxt, x, v, fptr, refp, N, i + stride, a.shadow);
     if (i + kPrefetchAhead * stride < N)
       integrate_prefetch_l2<MIXED>(x, v, fptr, refp, N, i + kPrefetchAhead * stride, a.shadow);
-    double F[3];
-    float Ff[3] = {0.0f, 0.0f, 0.0f};
-    if constexpr (MIXED) {
-      const float4 f = cur.f;
-      Ff[0] = f.x;
-      Ff[1] = f.y;
-      Ff[2] = f.z;
-      F[0] = f32_to_f64(f.x);
-      F[1] = f32_to_f64(f.y);
-      F[2] = f32_to_f64(f.z);
-    } else {
-      const dvec4 f = cur.f;
-      F[0] = f.x;
-      F[1] = f.y;
-      F[2] = f.z;
-    }
-    double xs[3];
-    float ke_i = 0.0f, vd2 = 0.0f;
-    double ke_d = 0.0;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      double vk = cur.v[k];
-      if (a.ke) {
-        if (MIXED) {
-          const float vf = fmaf(kpre_f, Ff[k], f64_to_f32(vk));
-          ke_i = fmaf(vf, vf, ke_i);
-        } else {
-          const double vf = fma(a.kpre, F[k], vk);
-          ke_d = fma(vf, vf, ke_d);
-        }
-      }
-      if (kk != 0.0) vk = fma(kk, F[k], vk);
-      if (a.speed) {
-        const float vs = MIXED ? f64_to_f32(vk) : (float)vk;
-        vd2 = fmaf(vs, vs, vd2);
-      }
-      double xk = cur.x[k];
-      if (a.dt != 0.0) xk = fma(a.dt, vk, xk);
-      v[k * N + i] = vk;
-      x[k * N + i] = xk;
-      xs[k] = xk;
-      bad |= !finite_d(xk) || !finite_d(vk);
-    }
-    if (MIXED) ke_acc += f32_to_f64(0.5f * ke_i);  // exact halving and conversion, one FP64 add
-    else ke_acc += 0.5 * ke_d;
-    if (a.shadow) {
-      // speed of the drift (the velocity that moved the particle this step), for the DUTC rule
-      v2max = fmaxf(v2max, vd2);
-      if constexpr (MIXED) {
-        const uint4 q = make_uint4(fixq(xs[0], a.qk), fixq(xs[1], a.qk), fixq(xs[2], a.qk), (uint32_t)i);
-        ((uint4*)pos)[i] = q;
-        // displacement since the list was built, from the records: exact integer differences
-        // (within u of the FP64 ones), converted once and scaled by u
-        const uint4 r = cur.r;
-        const float dx = qdiff(q.x, r.x) * qu, dy = qdiff(q.y, r.y) * qu, dz = qdiff(q.z, r.z) * qu;
-        d2max = fmaxf(d2max, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-      } else {
-        ((dvec4*)pos)[i] = make_dvec4(xs[0], xs[1], xs[2], 0.0);
-        const dvec4 r = cur.r;
-        const double dx = xs[0] - r.x, dy = xs[1] - r.y, dz = xs[2] - r.z;
-        // rounded up to FP32, so the measured maximum never falls short of the FP64 value and the
-        // margin/2 rule keeps its guarantee at the FP64 form's tight limit
-        d2max = fmaxf(d2max, __double2float_ru(fma(dx, dx, fma(dy, dy, dz * dz))));
-      }
-    }
+    integrate_one<MIXED>(cur, a, x, v, pos, N, i, acc);
     cur = nxt;
   }
-  if (bad) atomicOr(status, LJ_ST_NONFINITE);
+  double ke_acc = acc.ke;
+  float d2max = acc.d2max, v2max = acc.v2max;
+  if (acc.bad) atomicOr(status, LJ_ST_NONFINITE);
   __shared__ double sh[32];
   __shared__ float shf[32];
-  const double tk = block_sum(ke_acc, sh);
-  if (threadIdx.x == 0 && a.ke) ke_part[blockIdx.x] = tk;
+  if (a.ke) {
+    const double tk = block_sum(ke_acc, sh);
+    if (threadIdx.x == 0) ke_part[blockIdx.x] = tk;
+  }
   if (a.shadow && !a.speed) {
     const float m = block_max(d2max, shf);
     if (threadIdx.x == 0) atomicMax(dmax_bits, __float_as_uint(m));
@@ -220,27 +95,7 @@ __global__ void __launch_bounds__(256) k_integrate(double* __restrict__ x, doubl
       }
     }
   }
-  if (fin.ticket) {  // the last CTA to finish takes the energy record and the validity check
-    // thread 0 wrote the CTA's partial (the maxima went by device-wide atomics): it alone orders
-    // that write before its ticket
-    __shared__ int s_last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = atomicAdd(fin.ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last) {
-      __threadfence();
-      if (fin.rec)
-        energy_record_block(fin.pv, fin.nbf, ke_part, gridDim.x, fin.pe_scale, fin.energies, fin.log, fin.cap,
-                            fin.count, fin.step);
-      if (threadIdx.x == 0) {
-        if (fin.check) step_check_one(dmax_bits, fin.ctl, fin.s, fin.disp_limit, fin.dutc, fin.two_dt);
-        *fin.ticket = 0u;
-      }
-    }
-  }
+  if (fin.ticket) step_finish(fin, ke_part, dmax_bits);
 }
 
 // Block shape: 256-thread blocks of one resident wave (at most red_blocks(N)), so that the grid-stride
@@ -273,6 +128,7 @@ int launch_integrate(int precision, double* x, double* v, const void* f, void* p
                      IntegrateArgs a, double* ke_part, uint32_t* dmax_bits, int32_t* status, StepFinish fin,
                      cudaStream_t s, const int* skip) {
   int blocks = 1, threads = kRedThreads;
+  a = integrate_prepare(a);
   if (precision == LJ_MIXED) {
     integrate_shape<true>(N, blocks, threads);
     k_integrate<true><<<blocks, threads, 0, s>>>(x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);

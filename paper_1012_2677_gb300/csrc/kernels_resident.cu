@@ -198,13 +198,13 @@ __global__ void __launch_bounds__(MIXED ? kResThreads : kDpThreads, MIXED ? 3 : 
             ked = fma(vf, vf, ked);
           }
         }
-        if (kk != 0.0) vk = fma(kk, F[k], vk);
+        if (!is_zero_d(kk)) vk = fma(kk, F[k], vk);
         if (a.dutc_rule) {
           const float vs = MIXED ? f64_to_f32(vk) : (float)vk;
           vd2 = fmaf(vs, vs, vd2);
         }
         double xk = xv[k * mo + o];
-        if (dt != 0.0) xk = fma(dt, vk, xk);
+        if (!is_zero_d(dt)) xk = fma(dt, vk, xk);
         xv[(3 + k) * mo + o] = vk;
         xv[k * mo + o] = xk;
         xs[k] = xk;

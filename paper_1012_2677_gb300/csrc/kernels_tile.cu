@@ -638,7 +638,8 @@ int set_wait_budget(long long cycles) {
   const long long v = cycles > 0 ? cycles : kWaitBudget;
   if (cudaDeviceSynchronize() != cudaSuccess) return -1;
   if (set_unit_wait_budget(v) || set_wait_budget_force(v) || set_wait_budget_force_half(v) ||
-      set_wait_budget_force_dp(v) || set_wait_budget_resident(v) || set_wait_budget_adjoint(v))
+      set_wait_budget_force_dp(v) || set_wait_budget_resident(v) || set_wait_budget_adjoint(v) ||
+      set_wait_budget_step(v))
     return -1;
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : -1;
 }

@@ -548,15 +548,15 @@ struct EAcc {
   int n = 0;
   float vscale = 1.0f;
   __device__ __forceinline__ void flush() {
-    pe += (double)pe32;
-    vir += (double)(vir32 * vscale);
+    pe += f32_to_f64(pe32);
+    vir += f32_to_f64(vir32 * vscale);
     pe32 = vir32 = 0.0f;
     n = 0;
   }
   __device__ __forceinline__ void add32(float p, float v) {
     pe32 += p;
     vir32 += v;
-    if (++n == 16) flush();
+    if (++n == 16) flush();  // (as a branch: predicated, its FP64 adds would take their slots every time)
   }
 };
 
