@@ -639,7 +639,7 @@ int set_wait_budget(long long cycles) {
   if (cudaDeviceSynchronize() != cudaSuccess) return -1;
   if (set_unit_wait_budget(v) || set_wait_budget_force(v) || set_wait_budget_force_half(v) ||
       set_wait_budget_force_dp(v) || set_wait_budget_resident(v) || set_wait_budget_adjoint(v) ||
-      set_wait_budget_step(v))
+      set_wait_budget_step(v) || set_wait_budget_sort(v))
     return -1;
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : -1;
 }
@@ -647,7 +647,7 @@ int set_wait_budget(long long cycles) {
 void launch_list_tile(int precision, int half, const void* pos, const float4* hi, const double* x, const uint32_t* cs,
                       int64_t N, Geom g, TileArgs ta, ListBand band, uint2* rows, uint2* tile_list, uint16_t* ent,
                       uint64_t cap, unsigned long long* counter, unsigned int* max_list, int32_t* status,
-                      cudaStream_t s) {
+                      cudaStream_t s, const int* pred) {
   const size_t sm = list_smem_bytes(ta, precision);
   int grid = tile_grid(ta, per_sm_for(sm));
   if (!ta.whole) {  // the window kernel: as many CTAs as are resident
@@ -673,12 +673,12 @@ void launch_list_tile(int precision, int half, const void* pos, const float4* hi
     set_smem(k_list_win<true, false, kWinThreads>, sm);
     k_list_win<true, false, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, ta, band, rows, tile_list, ent,
                                                                        cap, counter, max_list, status, nullptr, 0,
-                                                                       nullptr, nullptr);
+                                                                       pred, nullptr);
   } else {
     set_smem(k_list_win<false, false, kWinThreads>, sm);
     k_list_win<false, false, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, ta, band, rows, tile_list, ent,
                                                                         cap, counter, max_list, status, nullptr, 0,
-                                                                        nullptr, nullptr);
+                                                                        pred, nullptr);
   }
 #undef LJ_LIST_LAUNCH
 }

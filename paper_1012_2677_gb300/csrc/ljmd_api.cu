@@ -85,6 +85,11 @@ struct ljmd_sys {
   int res_lanes = 0;
   TileArgs res_ta{};
   ResidentCtl *d_res = nullptr, *h_res = nullptr;
+  GridCtl* d_grid = nullptr;        // d_status, d_total64 and d_sizes are parts of it
+  GridCtl* h_grid = nullptr;        // its pinned copy
+  uint32_t* sort_count = nullptr;   // cell counts of k_sort, behind d_grid: zero between launches
+  void* h_pin = nullptr;            // the pinned block that holds all h_ arrays
+  bool sort_dirty = false;          // a launch may have left counts behind
   void* pos_alt = nullptr;
   int64_t pos_alt_cap = 0;
   double *res_rec = nullptr, *part_force2 = nullptr;
@@ -161,7 +166,7 @@ static void free_all(ljmd_sys* s) {
   void* ptrs[] = {s->x, s->v, s->x_alt, s->v_alt, s->f, s->f_alt, s->hi, s->xq, s->pos64, s->ref, s->id,
                   s->id_alt, s->img, s->img_alt, s->cell_of, s->perm, s->perm_id, s->cell_count, s->cell_start,
                   s->cell_fill, s->rows, s->tile_list, s->ent, s->scan_tmp, s->part_force, s->part_ke,
-                  s->part_misc, s->d_scalars, s->d_energies, s->d_log_count, s->d_status, s->d_dmax, s->d_ctl, s->d_ticket, s->d_total64, s->d_sizes,
+                  s->part_misc, s->d_scalars, s->d_energies, s->d_log_count, s->d_grid, s->d_dmax, s->d_ctl, s->d_ticket,
                   s->adj_w, s->adj_hw, s->adj_f, s->adj_wf, s->adj_ticket, s->part_adj, s->d_adj, s->xref64, s->ldc_list, s->d_ldc,
                   s->d_res, s->pos_alt, s->res_rec, s->part_force2};
   for (void* p : ptrs)
@@ -171,11 +176,7 @@ static void free_all(ljmd_sys* s) {
     cudaEventDestroy(p.second.second);
   }
   for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
-  if (s->h_u32) cudaFreeHost(s->h_u32);
-  if (s->h_f64) cudaFreeHost(s->h_f64);
-  if (s->h_i32) cudaFreeHost(s->h_i32);
-  if (s->h_ctl) cudaFreeHost(s->h_ctl);
-  if (s->h_res) cudaFreeHost(s->h_res);
+  if (s->h_pin) cudaFreeHost(s->h_pin);
 }
 
 enum { PH_FORCE = 0, PH_INTEGRATE = 1, PH_REBUILD = 2, PH_ENERGY = 3, PH_ADJOINT = 4 };
@@ -518,6 +519,17 @@ static int default_lanes(const ljmd_sys* s) {
   return (double)s->ta.T * ppc >= 96.0 ? 2 : 4;
 }
 
+// The tiles' shape at T cells per tile, or as near as the box allows.
+static void tile_shape(TileArgs& ta, int T) {
+  const int n = ta.n;
+  if (T > n - 2) T = n - 2;
+  if (T > kMaxTileT) T = kMaxTileT;
+  if (T < 1) T = 1;
+  ta.ntz = (n + T - 1) / T;
+  ta.T = (n + ta.ntz - 1) / ta.ntz;  // the same number of tiles, of even length
+  ta.ntiles = (int64_t)n * n * ta.ntz;
+}
+
 static int choose_tiles(ljmd_sys* s, int t_cap) {
   ljmd_sys* sys = s;
   TileArgs& ta = s->ta;
@@ -540,13 +552,9 @@ static int choose_tiles(ljmd_sys* s, int t_cap) {
   ta.whole = 0;
   int T = s->tile_T > 0 ? s->tile_T : default_tile_cells(s);
   if (T > t_cap) T = t_cap;
-  if (T > n - 2) T = n - 2;
-  if (T > kMaxTileT) T = kMaxTileT;
-  if (T < 1) T = 1;
   for (;; --T) {
-    ta.ntz = (n + T - 1) / T;
-    ta.T = T = (n + ta.ntz - 1) / ta.ntz;  // the same number of tiles, of even length
-    ta.ntiles = (int64_t)n * n * ta.ntz;
+    tile_shape(ta, T);
+    T = ta.T;
     CK(cudaMemsetAsync(s->d_sizes, 0, 3 * sizeof(unsigned int), s->st));
     launch_tile_sizes(s->cell_start, ta, s->d_sizes, s->st);
     launch_max_count(s->cell_count, s->ncells, s->d_sizes + 2, s->st);
@@ -563,6 +571,77 @@ static int choose_tiles(ljmd_sys* s, int t_cap) {
   }
 }
 
+static void swap_state(ljmd_sys* s) {
+  std::swap(s->x, s->x_alt);
+  std::swap(s->v, s->v_alt);
+  std::swap(s->id, s->id_alt);
+  std::swap(s->img, s->img_alt);
+  std::swap(s->f, s->f_alt);
+}
+
+// The reordering by one launch (kernels_sort.cu) where the box is small enough: up to 6,144 cells (every CTA
+// scans them) and as many particles as the chip holds threads; beyond, the list construction is what counts.
+// The list kernel can then be launched without a look at the tile sizes in between: with capacities
+// guessed from the mean counts (six standard deviations of a Poisson count above them; a liquid's counts vary
+// less), which k_sort compares with the sizes.
+static int sort_small(ljmd_sys* s, bool* sorted, bool* guessed) {
+  ljmd_sys* sys = s;
+  const int64_t N = s->n;
+  const int n = s->g.n;
+  if (n < 3 || s->ncells > kSortCells || N > sort_capacity()) return LJ_OK;
+  if (s->sort_dirty) CK(cudaMemsetAsync(s->sort_count, 0, kSortCells * sizeof(uint32_t), s->st));
+  s->sort_dirty = false;
+  TileArgs& ta = s->ta;
+  ta.n = n;
+  ta.whole = 0;
+  tile_shape(ta, s->tile_T > 0 ? s->tile_T : default_tile_cells(s));
+  const double ppc = (double)N / (double)s->ncells;
+  auto guess = [](double m) { return (int32_t)(m + 6.0 * sqrt(m) + 16.0); };
+  ta.max_staged = guess(9.0 * (ta.T + 2) * ppc);
+  ta.max_own = guess(ta.T * ppc);
+  ta.max_chunks = 9 * ((3 * guess(ppc) + 31) / 32) + 1;
+  int dev = 0, smem_max = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const bool caps = ta.max_staged <= 65535 && list_smem_bytes(ta, s->precision) <= (size_t)smem_max &&
+                    ensure_tile_list(s) == LJ_OK;
+  CK(cudaMemsetAsync(s->d_grid, 0, offsetof(GridCtl, status), s->st));
+  SortArgs a{};
+  a.x = s->x;
+  a.v = s->v;
+  a.img = s->img;
+  a.id = s->id;
+  a.f = s->f;
+  a.x2 = s->x_alt;
+  a.v2 = s->v_alt;
+  a.img2 = s->img_alt;
+  a.id2 = s->id_alt;
+  a.f2 = s->f_alt;
+  a.hi = s->hi;
+  a.pos = force_pos(s);
+  a.ref = s->ref;
+  a.count = s->sort_count;
+  a.cell_count = s->cell_count;
+  a.cell_start = s->cell_start;
+  a.cell_ids = (int32_t*)s->perm;
+  a.ctl = s->d_grid;
+  a.N = N;
+  a.ncells = (int32_t)s->ncells;
+  a.caps = caps ? 1 : 0;
+  a.g = s->g;
+  a.ta = ta;
+  const int r = launch_sort(s->precision, a, s->st);
+  if (r > 0) {
+    cudaGetLastError();
+    return LJ_OK;
+  }
+  CKL();
+  s->launches += 1;
+  *sorted = true;
+  *guessed = caps;
+  return LJ_OK;
+}
+
 // ----------------------------------------------------------------------------------------------
 // Pair-list construction: fold, label, counting sort (Fig. 3), reorder (Sec. 3.3), sorted list.
 static int rebuild(ljmd_sys* s) {
@@ -571,26 +650,28 @@ static int rebuild(ljmd_sys* s) {
   cudaStream_t st = s->st;
   TRY(ensure_cells(s));
   PhaseTimer timer(s, PH_REBUILD);
-  // wrap_label, scatter, cell_order, gather, shadow (+ the scan, tile sizing and list below)
-  s->launches += 5;
-  CK(cudaMemsetAsync(s->cell_count, 0, sizeof(uint32_t) * s->ncells, st));
-  launch_wrap_label(s->x, s->img, N, s->g, s->cell_of, s->cell_count, s->d_status, st);
-  CKL();
-  s->launches += launch_scan_u32(s->cell_count, s->cell_start, s->ncells, s->scan_tmp, st);
-  CKL();
-  CK(cudaMemsetAsync(s->cell_fill, 0, sizeof(uint32_t) * s->ncells, st));
-  launch_scatter(s->cell_of, s->cell_start, s->cell_fill, s->perm, N, st);
-  launch_cell_rank(s->cell_start, s->ncells, s->perm, s->id, s->perm_id, st);
-  launch_gather_state(s->perm_id, N, s->x, s->x_alt, s->v, s->v_alt, s->id, s->id_alt, s->img, s->img_alt, s->f,
-                      s->f_alt, s->precision == LJ_MIXED ? 16 : 32, st, nullptr);
-  CKL();
-  std::swap(s->x, s->x_alt);
-  std::swap(s->v, s->v_alt);
-  std::swap(s->id, s->id_alt);
-  std::swap(s->img, s->img_alt);
-  std::swap(s->f, s->f_alt);
-  launch_shadow_all(s->x, N, s->precision == LJ_MIXED, s->g.qk, s->hi, s->xq, s->pos64, s->ref, st);
-  CKL();
+  bool sorted = false, guessed = false;  // guessed: s->ta holds the capacities that k_sort checks
+  TRY(sort_small(s, &sorted, &guessed));
+  if (!sorted) {
+    // wrap_label, scatter, cell_order, gather, shadow (+ the scan, tile sizing and list below)
+    s->launches += 5;
+    CK(cudaMemsetAsync(s->cell_count, 0, sizeof(uint32_t) * s->ncells, st));
+    launch_wrap_label(s->x, s->img, N, s->g, s->cell_of, s->cell_count, s->d_status, st);
+    CKL();
+    s->launches += launch_scan_u32(s->cell_count, s->cell_start, s->ncells, s->scan_tmp, st);
+    CKL();
+    CK(cudaMemsetAsync(s->cell_fill, 0, sizeof(uint32_t) * s->ncells, st));
+    launch_scatter(s->cell_of, s->cell_start, s->cell_fill, s->perm, N, st);
+    launch_cell_rank(s->cell_start, s->ncells, s->perm, s->id, s->perm_id, st);
+    launch_gather_state(s->perm_id, N, s->x, s->x_alt, s->v, s->v_alt, s->id, s->id_alt, s->img, s->img_alt, s->f,
+                        s->f_alt, s->precision == LJ_MIXED ? 16 : 32, st, nullptr);
+    CKL();
+  }
+  swap_state(s);
+  if (!sorted) {
+    launch_shadow_all(s->x, N, s->precision == LJ_MIXED, s->g.qk, s->hi, s->xq, s->pos64, s->ref, st);
+    CKL();
+  }
   const int half = s->list_half ? 1 : 0;
   uint64_t total = 0;
   int dev = 0, smem_max = 0;
@@ -598,7 +679,7 @@ static int rebuild(ljmd_sys* s) {
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   // the force kernel's two tile buffers must fit: a smaller tile is chosen if they do not
   for (int t_cap = kMaxTileT;;) {
-    TRY(choose_tiles(s, t_cap));
+    if (!guessed) TRY(choose_tiles(s, t_cap));
     bool built = false;
     for (int attempt = 0; attempt < 2; ++attempt) {
       if (s->ent_cap == 0) {
@@ -608,27 +689,43 @@ static int rebuild(ljmd_sys* s) {
         TRY(dalloc_t(s, &s->ent, want));
         s->ent_cap = want;
       }
-      CK(cudaMemsetAsync(s->d_total64, 0, 2 * sizeof(unsigned long long), st));
-      CK(cudaMemsetAsync(s->d_sizes + 3, 0, sizeof(unsigned int), st));
+      if (!guessed || attempt > 0) {
+        CK(cudaMemsetAsync(s->d_total64, 0, 2 * sizeof(unsigned long long), st));
+        CK(cudaMemsetAsync(s->d_sizes + 3, 0, sizeof(unsigned int), st));
+      }
       // the list kernels filter on the FP32 hi copies (mixed) or the FP64 copies (FP64 form, whole box)
       const void* list_pos = s->precision == LJ_MIXED ? (const void*)s->hi : (const void*)s->pos64;
       launch_list_tile(s->precision, half, list_pos, s->hi, s->x, s->cell_start, N, s->g, s->ta, s->band, s->rows,
-                       s->tile_list, s->ent, (uint64_t)s->ent_cap, s->d_total64, s->d_sizes + 3, s->d_status, st);
+                       s->tile_list, s->ent, (uint64_t)s->ent_cap, s->d_total64, s->d_sizes + 3, s->d_status, st,
+                       guessed ? &s->d_grid->ok : nullptr);
       s->launches += 1;
       CKL();
-      CK(cudaMemcpyAsync(s->h_u32 + 4, s->d_total64, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-      CK(cudaMemcpyAsync(s->h_u32 + 12, s->d_sizes + 3, sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-      CK(cudaMemcpyAsync(s->h_u32 + 13, s->d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));  // one round trip: list size, longest segment and status
-      unsigned long long total64, actual64;
-      memcpy(&total64, s->h_u32 + 4, sizeof(total64));
-      memcpy(&actual64, s->h_u32 + 6, sizeof(actual64));
-      s->ta.max_list = (int32_t)s->h_u32[12];
+      const GridCtl* hg = s->h_grid;
+      CK(cudaMemcpyAsync(s->h_grid, s->d_grid, sizeof(GridCtl), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));  // one round trip: sizes, list size, longest segment and status
+      if (sorted && (int64_t)hg->ticket != sort_grid(N)) {  // a wait of k_sort ran out: the state is where it was
+        swap_state(s);
+        s->sort_dirty = true;
+        s->have_list = s->forces_current = false;
+        return LJ_EDEVICE;
+      }
+      if (guessed && !hg->ok) {  // a size beyond its guess: the list kernel has not run
+        guessed = false;
+        TRY(choose_tiles(s, t_cap));
+        attempt = -1;
+        continue;
+      }
+      if (guessed) {
+        s->ta.max_staged = (int32_t)hg->sizes[0];
+        s->ta.max_own = (int32_t)std::max(hg->sizes[1], 1u);
+        s->ta.max_chunks = (int32_t)(9 * ((3 * hg->sizes[2] + 31) / 32) + 1);
+      }
+      const unsigned long long total64 = hg->total[0], actual64 = hg->total[1];
+      s->ta.max_list = (int32_t)hg->sizes[3];
       if (total64 > 4294967295ULL) return LJ_ERANGE;  // row starts are 32-bit
       total = total64;
       if (total <= s->ent_cap) {
-        int32_t w = 0;
-        memcpy(&w, s->h_u32 + 13, sizeof(w));
+        const int32_t w = hg->status;
         if (w) {
           fprintf(stderr, "ljmd: list construction raised status %d (n=%d T=%d tiles=%lld staged<=%d own<=%d)\n", w,
                   s->ta.n, s->ta.T, (long long)s->ta.ntiles, s->ta.max_staged, s->ta.max_own);
@@ -660,6 +757,7 @@ static int rebuild(ljmd_sys* s) {
     }
     if (s->ta.whole || s->ta.T <= 1) return LJ_ERANGE;
     t_cap = s->ta.T - 1;
+    guessed = false;
   }
   s->list_entries = total;
   s->have_list = true;
@@ -960,11 +1058,6 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
 static int ensure_resident(ljmd_sys* s) {
   const size_t psz = s->precision == LJ_MIXED ? 16 : 32;
   if (!s->d_res) TRY(dalloc_t(s, &s->d_res, 1));
-  if (!s->h_res && cudaMallocHost(&s->h_res, sizeof(ResidentCtl)) != cudaSuccess) {
-    s->h_res = nullptr;
-    cudaGetLastError();
-    return LJ_ENOMEM;
-  }
   if (!s->part_force2) TRY(dalloc_t(s, &s->part_force2, 2 * kMaxRedBlocks));
   if (s->pos_alt_cap < s->cap_n) {  // the capacity of the records themselves: the two may change places
     s->pos_alt_cap = 0;
@@ -1110,18 +1203,34 @@ int ljmd_create(ljmd_sys** out, const ljmd_params* p, int32_t precision, void* c
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_scalars, 8);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_energies, 4);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_log_count, 1);
-  if (r == LJ_OK) r = dalloc_t(sys, &sys->d_status, 1);
+  if (r == LJ_OK) r = dalloc(sys, (void**)&sys->d_grid, sizeof(GridCtl) + sizeof(uint32_t) * kSortCells);
+  if (r == LJ_OK) {
+    sys->d_status = &sys->d_grid->status;
+    sys->d_total64 = sys->d_grid->total;
+    sys->d_sizes = sys->d_grid->sizes;
+    sys->sort_count = (uint32_t*)(sys->d_grid + 1);
+  }
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_dmax, 2);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_ctl, 1);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_ticket, 1);
   if (r == LJ_OK && cudaMemsetAsync(sys->d_ticket, 0, sizeof(unsigned int), sys->st) != cudaSuccess) r = LJ_EDEVICE;
-  if (r == LJ_OK && cudaMallocHost(&sys->h_ctl, sizeof(StepCtl)) != cudaSuccess) r = LJ_ENOMEM;
-  if (r == LJ_OK) r = dalloc_t(sys, &sys->d_total64, 2);
-  if (r == LJ_OK) r = dalloc_t(sys, &sys->d_sizes, 4);
-  if (r == LJ_OK && cudaMallocHost(&sys->h_u32, 64) != cudaSuccess) r = LJ_ENOMEM;
-  if (r == LJ_OK && cudaMallocHost(&sys->h_f64, 64) != cudaSuccess) r = LJ_ENOMEM;
-  if (r == LJ_OK && cudaMallocHost(&sys->h_i32, 64) != cudaSuccess) r = LJ_ENOMEM;
-  if (r == LJ_OK && cudaMemsetAsync(sys->d_status, 0, 4, sys->st) != cudaSuccess) r = LJ_EDEVICE;
+  static_assert(sizeof(StepCtl) <= 64 && sizeof(GridCtl) <= 64, "slots of the pinned block");
+  if (r == LJ_OK && cudaMallocHost(&sys->h_pin, 5 * 64 + sizeof(ResidentCtl)) != cudaSuccess) {
+    sys->h_pin = nullptr;
+    r = LJ_ENOMEM;
+  }
+  if (r == LJ_OK) {
+    unsigned char* h = (unsigned char*)sys->h_pin;
+    sys->h_ctl = (StepCtl*)h;
+    sys->h_u32 = (uint32_t*)(h + 64);
+    sys->h_f64 = (double*)(h + 128);
+    sys->h_i32 = (int32_t*)(h + 192);
+    sys->h_grid = (GridCtl*)(h + 256);
+    sys->h_res = (ResidentCtl*)(h + 320);
+  }
+  if (r == LJ_OK &&
+      cudaMemsetAsync(sys->d_grid, 0, sizeof(GridCtl) + sizeof(uint32_t) * kSortCells, sys->st) != cudaSuccess)
+    r = LJ_EDEVICE;
   if (r == LJ_OK && cudaMemsetAsync(sys->d_log_count, 0, 8, sys->st) != cudaSuccess) r = LJ_EDEVICE;
   if (r != LJ_OK) {
     cudaGetLastError();

@@ -130,6 +130,41 @@ struct TileArgs {
   int32_t max_list;    // list entries per tile (padded to 8), at most (known after construction)
   int32_t list_cap;    // entries of a tile's segment the force kernel stages (multiple of 8); the rest stays in HBM
 };
+// Counters of a list construction, and the status word (which lasts), in one block that one copy reads.
+struct GridCtl {
+  unsigned long long total[2];  // list entries, padded and actual
+  unsigned int sizes[4];        // largest: particles staged by a tile, own particles, particles of a cell, list segment
+  int ok;                       // the sizes fit the capacities the list kernel was launched with
+  unsigned int arrived, ticket; // grid barriers and last CTA of k_sort
+  unsigned int pad;
+  int32_t status;
+  unsigned int pad2[3];
+};
+// The reordering of a small box in one cooperative launch (kernels_sort.cu).
+constexpr int kSortCells = 6144;
+struct SortArgs {
+  const double *x, *v;
+  const int32_t *img, *id;
+  const void* f;
+  double *x2, *v2;
+  int32_t *img2, *id2;
+  void* f2;
+  float4* hi;
+  void *pos, *ref;
+  uint32_t *count, *cell_count, *cell_start;  // count: zero between launches
+  int32_t* cell_ids;
+  GridCtl* ctl;
+  int64_t N;
+  int32_t ncells;
+  int32_t caps;  // the tile capacities of ta are meant
+  Geom g;
+  TileArgs ta;
+};
+int64_t sort_capacity();
+int64_t sort_grid(int64_t N);
+int launch_sort(int precision, SortArgs a, cudaStream_t s);
+int set_wait_budget_sort(long long cycles);
+
 // One replica of a batch: its box (offset and p are the batch's), grid, tiles and particles.
 // Global tiles, cells and particles are the replicas' ranges concatenated in replica order.
 struct ReplicaGeo {
@@ -148,7 +183,7 @@ void launch_tile_sizes(const uint32_t* cs, TileArgs ta, unsigned int* out, cudaS
 void launch_list_tile(int precision, int half, const void* pos, const float4* hi, const double* x, const uint32_t* cs,
                       int64_t N, Geom g, TileArgs ta, ListBand band, uint2* rows, uint2* tile_list, uint16_t* ent,
                       uint64_t cap, unsigned long long* counter, unsigned int* max_list, int32_t* status,
-                      cudaStream_t s);
+                      cudaStream_t s, const int* pred = nullptr);
 // pos: the fixed-point records (mixed) or the dvec4 copies (FP64).  Returns the number of blocks
 // (energy partials written to part[2 b], part[2 b + 1]).
 int launch_force_tile(int precision, int half, int lanes, int energy, const void* pos, const uint32_t* cs, int64_t N,

@@ -134,3 +134,32 @@ def test_step_in_force_kernel_matches_separate_launches(lanes, every, mode, T):
     assert (n > 0) == (every > 0)  # (a state between two calls may be recorded by both)
     if n:
         assert np.allclose(la[:n, 1:], lb[:n, 1:], rtol=1e-6, atol=1e-6 * np.abs(lb[:n, 1:]).max())
+
+
+@pytest.mark.parametrize("precision", [ljmd.LJ_MIXED, ljmd.LJ_FP64])
+@pytest.mark.parametrize("n,cells,spread", [
+    (1, 3, 1.0), (255, 4, 1.0), (256, 4, 1.0), (257, 4, 1.0),  # blocks of 256 particles
+    (2500, 6, 0.3),   # most cells empty, counts far beyond what the mean suggests
+    (3000, 18, 1.0), (3000, 19, 1.0),   # the last box that one launch reorders, the first that it does not
+])
+def test_reordering_of_small_boxes(n, cells, spread, precision):
+    """Cell starts, cell order (ids ascending) and pairs are integers: they equal the oracle's."""
+    L = cells * 3.05
+    x = synth.dyadic(np.random.default_rng(n + cells).uniform(0.0, spread * L, (n, 3)))
+    x[::7] += L  # outside the box: folded
+    v = synth.gaussian(x.shape, 9)
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=precision) as s:
+        s.set_state(x, v, L)
+        for _ in range(2):  # the second construction starts from the first one's order
+            s.build_pairlist()
+            assert s.stats()["cells_per_side"] == cells
+            ptr, lst = s.grid()
+            xw = x - np.floor(x / L) * L
+            c = np.minimum((xw * (cells / L)).astype(np.int64), cells - 1)
+            cell = (c[:, 0] * cells + c[:, 1]) * cells + c[:, 2]
+            order = np.lexsort((np.arange(n), cell))
+            assert np.array_equal(ptr[:cells ** 3], np.searchsorted(cell[order], np.arange(cells ** 3)))
+            assert np.array_equal(lst, order)
+            assert np.array_equal(s.pairs(), O.pairs_within(xw, L, 3.0))
+        xs, vs, _, img = s.get_state()
+        assert np.array_equal(xs + img * L, x) and np.array_equal(vs, v)
