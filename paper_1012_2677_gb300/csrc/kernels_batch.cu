@@ -8,11 +8,7 @@
 
 namespace ljmd {
 
-static int grid_of(int64_t n) {
-  int64_t b = (n + 255) / 256;
-  if (b < 1) b = 1;
-  return (int)(b < 1048576 ? b : 1048576);
-}
+static int grid_of(int64_t n, const int* pred = nullptr) { return stride_grid(n, 256, pred); }
 
 // Fold into the replica's box (img counts the folds) and label by the replica's cell grid;
 // global cell = cell_base + (cx n + cy) n + cz.  Same arithmetic as the single-system labelling.
@@ -55,7 +51,7 @@ __global__ void k_wrap_label_batch(double* __restrict__ x, int32_t* __restrict__
 void launch_wrap_label_batch(double* x, int32_t* img, int64_t N, const int32_t* rep_of, const ReplicaGeo* reps,
                              double offset, uint32_t* cell_of, uint32_t* cell_count, int32_t* status,
                              const int* pred, cudaStream_t s) {
-  k_wrap_label_batch<<<grid_of(N), 256, 0, s>>>(x, img, N, rep_of, reps, offset, cell_of, cell_count, status, pred);
+  k_wrap_label_batch<<<grid_of(N, pred), 256, 0, s>>>(x, img, N, rep_of, reps, offset, cell_of, cell_count, status, pred);
 }
 
 // Displacement rule on the device: flag = (largest squared displacement since the build >
@@ -87,7 +83,7 @@ __global__ void k_copy_words(const uint32_t* __restrict__ in, uint32_t* __restri
 }
 void launch_copy_words(const void* in, void* out, int64_t bytes, const int* pred, cudaStream_t s) {
   const int64_t n = bytes / 4;
-  k_copy_words<<<grid_of((n + 3) / 4), 256, 0, s>>>((const uint32_t*)in, (uint32_t*)out, n, pred);
+  k_copy_words<<<grid_of((n + 3) / 4, pred), 256, 0, s>>>((const uint32_t*)in, (uint32_t*)out, n, pred);
 }
 
 // Predicated zero fill of `bytes` (a multiple of 4).
@@ -98,7 +94,7 @@ __global__ void k_zero_words(uint32_t* __restrict__ out, int64_t n, const int* _
 }
 void launch_zero_words(void* out, int64_t bytes, const int* pred, cudaStream_t s) {
   const int64_t n = bytes / 4;
-  k_zero_words<<<grid_of(n), 256, 0, s>>>((uint32_t*)out, n, pred);
+  k_zero_words<<<grid_of(n, pred), 256, 0, s>>>((uint32_t*)out, n, pred);
 }
 
 // Kinetic energy per replica, 1/2 sum v^2 over its particles: blockIdx.y = replica, the blocks

@@ -4,11 +4,7 @@
 
 namespace ljmd {
 
-static int grid_for(int64_t n, int threads) {
-  int64_t b = (n + threads - 1) / threads;
-  if (b < 1) b = 1;
-  return (int)(b < 1048576 ? b : 1048576);
-}
+static int grid_for(int64_t n, int threads, const int* pred = nullptr) { return stride_grid(n, threads, pred); }
 
 // Fold x_state into [offset, offset + L) (one correction per component, counted in img),
 // label c = (cx n + cy) n + cz with cx = floor((x_state - offset) * n / L) clamped to [0, n-1],
@@ -166,7 +162,7 @@ __global__ void k_scatter(const uint32_t* __restrict__ cell_of, const uint32_t* 
 
 void launch_scatter(const uint32_t* cell_of, const uint32_t* cell_start, uint32_t* cell_fill, uint32_t* perm,
                     int64_t N, cudaStream_t s, const int* pred) {
-  k_scatter<<<grid_for(N, 256), 256, 0, s>>>(cell_of, cell_start, cell_fill, perm, N, pred);
+  k_scatter<<<grid_for(N, 256, pred), 256, 0, s>>>(cell_of, cell_start, cell_fill, perm, N, pred);
 }
 
 // Inside each cell order the particles by id (the order of Fig. 3's counting sort, independent of the
@@ -209,10 +205,7 @@ __global__ void k_cell_rank(const uint32_t* __restrict__ start, int64_t ncells, 
 
 void launch_cell_rank(const uint32_t* cell_start, int64_t ncells, const uint32_t* perm_in, const int32_t* id,
                       uint32_t* perm_out, cudaStream_t s, const int* pred) {
-  int64_t b = (ncells + 15) / 16;  // 16 cells per 256-thread block
-  if (b < 1) b = 1;
-  if (b > 1048576) b = 1048576;
-  k_cell_rank<<<(int)b, 256, 0, s>>>(cell_start, ncells, perm_in, id, perm_out, pred);
+  k_cell_rank<<<stride_grid(ncells, 16, pred), 256,  /* 16 cells per 256-thread block */ 0, s>>>(cell_start, ncells, perm_in, id, perm_out, pred);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -249,11 +242,11 @@ void launch_gather_state(const uint32_t* perm, int64_t N, const double* x, doubl
   const uint4* fi = (const uint4*)f;
   uint4* fo = (uint4*)f2;
   if (fbytes == 16)
-    k_gather_state<16><<<grid_for(N, 256), 256, 0, s>>>(perm, N, x, x2, v, v2, id, id2, img, img2, fi, fo, pred);
+    k_gather_state<16><<<grid_for(N, 256, pred), 256, 0, s>>>(perm, N, x, x2, v, v2, id, id2, img, img2, fi, fo, pred);
   else if (fbytes == 32)
-    k_gather_state<32><<<grid_for(N, 256), 256, 0, s>>>(perm, N, x, x2, v, v2, id, id2, img, img2, fi, fo, pred);
+    k_gather_state<32><<<grid_for(N, 256, pred), 256, 0, s>>>(perm, N, x, x2, v, v2, id, id2, img, img2, fi, fo, pred);
   else
-    k_gather_state<0><<<grid_for(N, 256), 256, 0, s>>>(perm, N, x, x2, v, v2, id, id2, img, img2, fi, fo, pred);
+    k_gather_state<0><<<grid_for(N, 256, pred), 256, 0, s>>>(perm, N, x, x2, v, v2, id, id2, img, img2, fi, fo, pred);
 }
 // ---------------------------------------------------------------------------------------------
 // Copies between the sorted SoA state and caller-order AoS (x[3 id + k]).

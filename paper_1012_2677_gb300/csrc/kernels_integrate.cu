@@ -169,9 +169,7 @@ __global__ void k_shadow(const double* __restrict__ x, int64_t N, int mixed, int
 
 void launch_shadow_all(const double* x, int64_t N, int mixed, int qk, float4* hi, uint4* xq, dvec4* pos64, void* ref,
                        cudaStream_t s, const int* pred) {
-  int64_t b = (N + 255) / 256;
-  if (b < 1) b = 1;
-  k_shadow<<<(int)(b < 1048576 ? b : 1048576), 256, 0, s>>>(x, N, mixed, qk, hi, xq, pos64, ref, pred);
+  k_shadow<<<stride_grid(N, 256, pred), 256, 0, s>>>(x, N, mixed, qk, hi, xq, pos64, ref, pred);
 }
 
 }  // namespace ljmd

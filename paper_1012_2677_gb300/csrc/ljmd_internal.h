@@ -116,6 +116,21 @@ void launch_load_state(const double* x_in, const double* v_in, double* x, double
 void launch_shadow_all(const double* x, int64_t N, int mixed, int qk, float4* hi, uint4* xq, dvec4* pos64, void* ref,
                        cudaStream_t s, const int* pred = nullptr);
 
+// Blocks for a grid-stride loop over n items, `per` to a block: one each, but no more than the chip holds at once
+// (2,048 threads per SM, 256-thread blocks) for a launch that a device flag may skip, so that skipping it costs
+// a launch and not the start and end of tens of thousands of blocks (6.6M particles: 15 us, then 2.5 us, for
+// each of the dozen launches of a construction that a batch's step skips).
+inline int stride_grid(int64_t n, int per, const int* pred) {
+  int64_t b = (n + per - 1) / per, most = 1048576;
+  if (pred) {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
+    most = 8 * sms;
+  }
+  return (int)(b < 1 ? 1 : (b < most ? b : most));
+}
+
 // ---- staged cell-column tiles: list and force ---------------------------------------------
 constexpr int kMaxTileT = 14;  // cells per tile along z, at most
 struct TileArgs {
