@@ -128,12 +128,16 @@ __device__ __forceinline__ void energy_record_block(const double* pv, int nbf, c
   }
 }
 
+// By the high word alone: of the whole 64-bit pattern the compiler makes comparisons of doubles, which take
+// slots of the FP64 pipe (six a particle in the integrator).
 __device__ __forceinline__ bool finite_d(double v) {
-  return (__double_as_longlong(v) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
+  return ((unsigned)__double2hiint(v) & 0x7fffffffu) < 0x7ff00000u;
 }
 
 // v == 0 by its bits (a comparison of doubles takes a slot of the FP64 pipe).
-__device__ __forceinline__ bool is_zero_d(double v) { return (__double_as_longlong(v) << 1) == 0; }
+__device__ __forceinline__ bool is_zero_d(double v) {
+  return (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) == 0u;
+}
 
 __device__ __forceinline__ bool finite_f(float v) {
   return (__float_as_int(v) & 0x7f800000) != 0x7f800000;
@@ -161,8 +165,8 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 // infinities and NaNs map to infinities and NaNs.
 __device__ __forceinline__ float f64_to_f32(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sign = (unsigned int)(b >> 63) << 31;
-  const int e = (int)((b >> 52) & 0x7ff);
+  const unsigned int hi = (unsigned int)__double2hiint(x), sign = hi & 0x80000000u;
+  const int e = (int)((hi >> 20) & 0x7ffu);
   if (e == 0x7ff) return __int_as_float((int)(sign | 0x7f800000u | (unsigned int)((b >> 29) & 0x7fffffu) |
                                               ((b & 0xfffffffffffffULL) ? 0x400000u : 0u)));
   if (e < 1023 - 126) return __int_as_float((int)sign);

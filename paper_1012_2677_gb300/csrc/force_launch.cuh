@@ -2,7 +2,6 @@
 // included by the translation unit that builds the form (one each, so that they compile in parallel).
 #pragma once
 
-#include "integrate.cuh"
 #include "tile.cuh"
 
 namespace ljmd {
@@ -97,24 +96,15 @@ __device__ __forceinline__ void pipe_shift(uint4* rec, uint32_t run, uint32_t ax
   __syncwarp();
 }
 
-// Hint that [p, p + bytes) be brought into L2 (whole 16-byte units inside that range).
-__device__ __forceinline__ void bulk_prefetch_l2(const void* p, int64_t bytes) {
-  const uint64_t a = ((uint64_t)p + 15u) & ~(uint64_t)15, e = ((uint64_t)p + (uint64_t)bytes) & ~(uint64_t)15;
-  if (e > a) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
-}
-
-// STEP: the consumers also take the step that follows the force (PipeStep), 32 particles of a tile at a time.
-template <bool HALF, int LANES, bool ENERGY, int NB, bool STEP>
+template <bool HALF, int LANES, bool ENERGY, int NB>
 __global__ void __launch_bounds__(pipe_threads(NB), 1)
     k_force_pipe(const uint4* __restrict__ pos, Geom g, TileArgs ta, LJConst c, const uint2* __restrict__ rows,
                  const uint2* __restrict__ tile_list, const uint16_t* __restrict__ ent, void* __restrict__ fout,
-                 double* __restrict__ part, int32_t* __restrict__ status, const int* __restrict__ skip, PipeStep st) {
-  static_assert(!(HALF && STEP), "a half list's forces are complete only after the launch");
+                 double* __restrict__ part, int32_t* __restrict__ status, const int* __restrict__ skip) {
   constexpr int CW = kPipeConsumers;
   if (skip && *skip) return;  // a device-decided run stopped before this step
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ PipeTile SS[NB];
-  __shared__ int2 own_of[STEP ? 2 * NB : 1];  // the own particles of the last 2 NB tiles
   __shared__ __align__(8) uint64_t full[NB], ready[NB], empty[NB];
   const TileLayout L = tile_layout(ta, true, true, false);
   const size_t buf_bytes = align16(L.total);
@@ -130,7 +120,6 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
   __syncthreads();
   EAcc eacc;
   eacc.vscale = g.qu;
-  IntegrateAcc sacc;
   const int64_t stride = gridDim.x;
   const long long budget = wait_budget();
   if (warp >= CW) {
@@ -179,11 +168,6 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
           mbar_arrive_expect(&full[b], 16u * total + (n_own > 0 ? 8u * (unsigned)(r1 - r0) : 0u) + 2u * n_ent);
         }
         __syncwarp();
-        if (STEP && lane >= 21 && lane < 28) {  // what the step reads of the tile's own particles
-          const int k = lane - 21;
-          if (k == 6) bulk_prefetch_l2(st.ref + gown0, 16 * (int64_t)n_own);
-          else bulk_prefetch_l2((k < 3 ? st.x + k * st.N : st.v + (k - 3) * st.N) + gown0, 8 * (int64_t)n_own);
-        }
         if (lane < 18) {
           const uint32_t n = d.y & 0xffffu;
           if (n > 0) bulk_g2s(buf + L.pos + 16 * (size_t)(d.y >> 16), pos + d.x, 16u * n, &full[b]);
@@ -229,14 +213,13 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
             SS[b].valid = -1;
             mbar_arrive(&ready[b]);
           }
-            break;
+          break;
         }
         if (images) pipe_shift((uint4*)(buf + L.pos), run, ax, ay, az, lane);
       }
       __syncwarp();
       if (lane == 0) {
         SS[b].valid = staged ? 1 : 0;
-        if (STEP) own_of[b + NB * (use & 1u)] = make_int2(gown0, staged ? n_own : 0);
         mbar_arrive(&ready[b]);  // release: bookkeeping and copies visible to the consumers
       }
     }
@@ -249,59 +232,27 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
     int turn = warp;  // chunk of the current tile that is this warp's next
     int b = 0;
     uint32_t use = 0;  // times the buffer was used before
-    // STEP: likewise the step, 32 particles at a time, of the tile kLag before this one.  Its forces are
-    // complete when its buffer is released, which the next tile's staging waits for in any case.
-    constexpr int kLag = NB - 1;
-    int sturn = warp, sb = 0;
-    uint32_t suse = 0;
-    const int64_t nt = (int64_t)blockIdx.x < ta.ntiles ? (ta.ntiles - blockIdx.x + stride - 1) / stride : 0;
-    for (int64_t k = 0; k < nt + (STEP ? kLag : 0); ++k) {
-      if (k < nt) {
-        bool ok = __all_sync(0xffffffffu, mbar_wait(&ready[b], use & 1u, budget)) != 0;
-        if (!ok) {
-          if (lane == 0) atomicOr(status, LJ_ST_TIMEOUT);
-          break;
-        }
-        const PipeTile& S = SS[b];
-        if (S.valid < 0) break;
-        if (S.valid > 0) {
-          const int chunks = (S.own1 - S.own0 + kChunk - 1) / kChunk;
-          if (turn < chunks)
-            force_tile_compute<true, LANES, HALF, ENERGY, false, true, 32 * CW>(
-                S, smem + b * buf_bytes, L, rows, ent, c, g, fout, status, eacc, ta.list_cap,
-                turn * kChunk + lane / LANES);
-          turn = (turn - chunks) % CW;
-          if (turn < 0) turn += CW;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[b]);
-        if (++b == NB) {
-          b = 0;
-          ++use;
-        }
+    for (int64_t t = blockIdx.x; t < ta.ntiles; t += stride) {
+      bool ok = __all_sync(0xffffffffu, mbar_wait(&ready[b], use & 1u, budget)) != 0;
+      if (!ok) {
+        if (lane == 0) atomicOr(status, LJ_ST_TIMEOUT);
+        break;
       }
-      if (STEP && k >= kLag) {
-        // (this warp has not released the buffer's next tile, so the phase waited for is the last or the current one)
-        bool ok = __all_sync(0xffffffffu, mbar_wait(&empty[sb], suse & 1u, budget)) != 0;
-        if (!ok) {
-          if (lane == 0) atomicOr(status, LJ_ST_TIMEOUT);
-          break;
-        }
-        const int2 own = own_of[sb + NB * (suse & 1u)];
-        const int chunks = (own.y + 31) / 32;
-        for (; sturn < chunks; sturn += CW) {
-          const int o = 32 * sturn + lane;
-          if (o < own.y) {
-            IntegrateIn<true> in;
-            integrate_load<true, true>(in, st.x, st.v, fout, st.ref, st.N, own.x + o, 1);
-            integrate_one<true, true>(in, st.a, st.x, st.v, st.pos_out, st.N, own.x + o, sacc);
-          }
-        }
-        sturn -= chunks;
-        if (++sb == NB) {
-          sb = 0;
-          ++suse;
-        }
+      const PipeTile& S = SS[b];
+      if (S.valid < 0) break;
+      if (S.valid > 0) {
+        const int chunks = (S.own1 - S.own0 + kChunk - 1) / kChunk;
+        if (turn < chunks)
+          force_tile_compute<true, LANES, HALF, ENERGY, false, true, 32 * CW>(
+              S, smem + b * buf_bytes, L, rows, ent, c, g, fout, status, eacc, ta.list_cap, turn * kChunk + lane / LANES);
+        turn = (turn - chunks) % CW;
+        if (turn < 0) turn += CW;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[b]);
+      if (++b == NB) {
+        b = 0;
+        ++use;
       }
     }
   }
@@ -317,49 +268,30 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
       part[2 * (size_t)blockIdx.x + 1] = tv;
     }
   }
-  if (STEP) {
-    __shared__ double shk[32];
-    float* shf = (float*)shk;
-    if (sacc.bad) atomicOr(status, LJ_ST_NONFINITE);
-    if (st.a.ke) {
-      const double tk = block_sum(sacc.ke, shk);
-      if (threadIdx.x == 0) st.ke_part[blockIdx.x] = tk;
-      __syncthreads();
-    }
-    const float md = block_max(sacc.d2max, shf);
-    __syncthreads();
-    const float mv = block_max(sacc.v2max, shf);
-    if (threadIdx.x == 0) {
-      atomicMax(st.dmax_bits, __float_as_uint(md));
-      if (st.a.speed) atomicMax(st.dmax_bits + 1, __float_as_uint(mv));
-    }
-    step_finish(st.fin, st.ke_part, st.dmax_bits);
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
 // Its launches; all return the grid launched (the number of energy partials written).
-template <bool HALF, int LANES, bool ENERGY, int NB, bool STEP>
+template <bool HALF, int LANES, bool ENERGY, int NB>
 static int force_pipe_launch(const ForceLaunch& a) {
   const size_t sm = NB * align16(tile_layout(a.ta, true, true, false).total);
-  set_smem(k_force_pipe<HALF, LANES, ENERGY, NB, STEP>, sm);
+  set_smem(k_force_pipe<HALF, LANES, ENERGY, NB>, sm);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count(), a.ta.ntiles));
-  k_force_pipe<HALF, LANES, ENERGY, NB, STEP><<<grid, pipe_threads(NB), sm, a.s>>>(
-      (const uint4*)a.pos, a.g, a.ta, a.c, a.rows, a.tile_list, a.ent, a.f, a.part, a.status, a.skip,
-      a.step ? *a.step : PipeStep{});
+  k_force_pipe<HALF, LANES, ENERGY, NB><<<grid, pipe_threads(NB), sm, a.s>>>((const uint4*)a.pos, a.g, a.ta, a.c, a.rows,
+                                                                       a.tile_list, a.ent, a.f, a.part, a.status, a.skip);
   return grid;
 }
-template <bool HALF, int LANES, bool ENERGY, bool STEP = false>
+template <bool HALF, int LANES, bool ENERGY>
 static int force_pipe(const ForceLaunch& a) {
   switch (a.nbuf) {
-    case 2: return force_pipe_launch<HALF, LANES, ENERGY, 2, STEP>(a);
-    case 3: return force_pipe_launch<HALF, LANES, ENERGY, 3, STEP>(a);
-    default: return force_pipe_launch<HALF, LANES, ENERGY, 4, STEP>(a);
+    case 2: return force_pipe_launch<HALF, LANES, ENERGY, 2>(a);
+    case 3: return force_pipe_launch<HALF, LANES, ENERGY, 3>(a);
+    default: return force_pipe_launch<HALF, LANES, ENERGY, 4>(a);
   }
 }
-template <bool HALF, int LANES, bool STEP = false>
+template <bool HALF, int LANES>
 static int force_pipe_energy(const ForceLaunch& a) {
-  return a.energy ? force_pipe<HALF, LANES, true, STEP>(a) : force_pipe<HALF, LANES, false, STEP>(a);
+  return a.energy ? force_pipe<HALF, LANES, true>(a) : force_pipe<HALF, LANES, false>(a);
 }
 
 }  // namespace ljmd

@@ -79,7 +79,7 @@ int pipe_plan(TileArgs& ta) {
   tz.list_cap = 0;
   const int64_t fixed = (int64_t)align16(tile_layout(tz, true, true, false).total);
   for (int nb = 4; nb >= 2; --nb) {
-    const int64_t per = ((int64_t)smem_max - 2048) / nb & ~(int64_t)15;
+    const int64_t per = ((int64_t)smem_max - 1024) / nb & ~(int64_t)15;
     if (per < fixed) continue;
     const int64_t cap = std::min<int64_t>((per - fixed) / 2, ta.max_list) & ~(int64_t)7;
     if (nb > 2 && 4 * cap < 3 * (int64_t)ta.max_list) continue;

@@ -639,7 +639,7 @@ int set_wait_budget(long long cycles) {
   if (cudaDeviceSynchronize() != cudaSuccess) return -1;
   if (set_unit_wait_budget(v) || set_wait_budget_force(v) || set_wait_budget_force_half(v) ||
       set_wait_budget_force_dp(v) || set_wait_budget_resident(v) || set_wait_budget_adjoint(v) ||
-      set_wait_budget_step(v) || set_wait_budget_sort(v))
+      set_wait_budget_sort(v))
     return -1;
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : -1;
 }

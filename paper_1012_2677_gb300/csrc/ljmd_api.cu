@@ -915,22 +915,6 @@ static int finalize_energies_now(ljmd_sys* s) {
   return LJ_OK;
 }
 
-// Whether the steps of a device-decided run can be taken by the force kernel itself: the mixed form with
-// the full list where the pipelined kernel runs (its forces are complete when a key's row is done; a half
-// list's are not, and in the FP64 form the integrator is 7 % of a step).  The drifted records go to a second
-// buffer, as other tiles still read the old ones; without memory for it the steps stay two launches each.
-static bool step_pipe_ready(ljmd_sys* s) {
-  if (s->precision != LJ_MIXED || s->list_half || s->profiling || s->ta.whole || force_buffers(s) != 2) return false;
-  TileArgs ta = s->ta;
-  if (!step_pipe_lanes(force_lanes(s)) || pipe_plan(ta) == 0) return false;
-  if (s->pos_alt_cap < s->cap_n) {
-    s->pos_alt_cap = 0;
-    if (dalloc(s, &s->pos_alt, 16 * (size_t)s->cap_n) != LJ_OK) return false;
-    s->pos_alt_cap = s->cap_n;
-  }
-  return true;
-}
-
 // Up to `remaining` velocity-Verlet steps with the list-validity rule decided on the device: each
 // step is the kick-drift (with the first half-kick fused into the previous step's second, except
 // for the first step of the call), whose last CTA takes the energy record when due and the validity
@@ -963,20 +947,6 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
   std::vector<size_t> ev_force(K);     // profiling entries before each step's force launch
   std::vector<int64_t> ln_force(K);    // launch count before each step's force launch
   std::vector<char> recorded(K, 0);
-  const bool fused = K > 1 && step_pipe_ready(s);
-  auto swap_records = [&] {
-    void* q = s->xq;
-    s->xq = (uint4*)s->pos_alt;
-    s->pos_alt = q;
-  };
-  PipeStep ps{};
-  ForceLaunch fl{};
-  if (fused) {
-    fl = ForceLaunch{nullptr,    s->cell_start, s->n,          s->g,        s->ta, s->c,           s->rows, s->tile_list,
-                     s->ent,     nullptr,       s->part_force, s->d_status, skip,  force_lanes(s), 0,       0,
-                     0,          0,             0,             st,          &ps};
-    fl.nbuf = pipe_plan(fl.ta);
-  }
   for (int64_t k = 0; k < K; ++k) {
     const int64_t t = s->steps + k;  // state index before the step
     const bool rec = (k == 0 ? s->pe_step == s->steps : true) && want_energy(t);
@@ -999,19 +969,7 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
     fin.disp_limit = s->disp_limit;
     fin.dutc = dutc;
     fin.two_dt = 2.0 * fabs(dt);
-    if (fused && k > 0) {  // the force of state t, then this step's drift
-      a.qk = s->g.qk;
-      ps = PipeStep{s->x, s->v, (const uint4*)s->ref, (uint4*)s->pos_alt, s->n, integrate_prepare(a), s->part_ke, s->d_dmax, fin};
-      fl.pos = s->xq;
-      fl.f = s->f;
-      fl.energy = rec ? 1 : 0;
-      ps.fin.nbf = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count_of(s->device), s->ta.ntiles));
-      s->nb_force = launch_step_pipe(fl);
-      s->launches += 1;
-      swap_records();
-    } else {
-      integrate(s, a, skip, &fin);
-    }
+    integrate(s, a, skip, &fin);
     if (rec) recorded[k] = 1;
     if (s->cap_x) {  // the state after this step's drift (skipped if the run stopped earlier)
       launch_unwrapped(s->x, s->img, s->id, s->n, s->g.offset, s->L, s->cap_x + 3 * s->n * (t + 1 - s->cap_step0),
@@ -1020,14 +978,13 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
     }
     ev_force[k] = s->ev_pending.size();
     ln_force[k] = s->launches;
-    if (!fused || k == K - 1) TRY(run_force(s, want_energy(t + 1), skip));
+    TRY(run_force(s, want_energy(t + 1), skip));
   }
   CKL();
   CK(cudaMemcpyAsync(hc, s->d_ctl, sizeof(StepCtl), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   *stopped = hc->stop != 0;
   const int64_t done = *stopped ? (int64_t)hc->stop_at + 1 : K;
-  if (fused && ((K - done) & 1)) swap_records();  // step done - 1 was the last to write its records
   // skipped launches of the run leave the counters and the profile; the stopping step's force too
   if (*stopped && s->profiling && ev_force[done - 1] >= ev0 && ev_force[done - 1] <= s->ev_pending.size()) {
     for (size_t q = ev_force[done - 1]; q < s->ev_pending.size(); ++q) {
@@ -1059,7 +1016,7 @@ static int ensure_resident(ljmd_sys* s) {
   const size_t psz = s->precision == LJ_MIXED ? 16 : 32;
   if (!s->d_res) TRY(dalloc_t(s, &s->d_res, 1));
   if (!s->part_force2) TRY(dalloc_t(s, &s->part_force2, 2 * kMaxRedBlocks));
-  if (s->pos_alt_cap < s->cap_n) {  // the capacity of the records themselves: the two may change places
+  if (s->pos_alt_cap < s->cap_n) {
     s->pos_alt_cap = 0;
     TRY(dalloc(s, &s->pos_alt, psz * (size_t)s->cap_n));
     s->pos_alt_cap = s->cap_n;

@@ -222,7 +222,6 @@ struct ForceLaunch {
   int lanes, energy, per_sm, nbuf, grid;
   size_t smem;
   cudaStream_t s;
-  const struct PipeStep* step = nullptr;
 };
 void launch_force_mixed_half(const ForceLaunch& a);
 int launch_force_pipe_half(const ForceLaunch& a);
@@ -263,13 +262,11 @@ struct IntegrateArgs {
   int shadow;      // rewrite the force kernel's position copy after the drift
   int speed;       // also reduce the largest drift speed (DUTC rules)
   int qk;          // mixed form: the fixed-point records are at u = 2^-qk
-  double kk;       // kpre + kpost, 1 / u and kpre in FP32: set by the launch (integrate_prepare), as the kernel's
-  double scale;    // threads have few particles each to spread FP64 operations of their own over
-  float kpre_f;
+  double kk;       // kpre + kpost, and kpre in FP32: set by the launch (integrate_prepare), as the kernel's
+  float kpre_f;    // threads have few particles each to spread FP64 operations of their own over
 };
 inline IntegrateArgs integrate_prepare(IntegrateArgs a) {
   a.kk = a.kpre + a.kpost;
-  a.scale = (double)(1ull << (a.qk & 63));
   a.kpre_f = (float)a.kpre;
   return a;
 }
@@ -294,18 +291,6 @@ struct StepFinish {
   double disp_limit;
   int dutc;
   double two_dt;
-};
-// What the force kernel needs to take the step that follows the force as well (mixed form, full list): the
-// arguments of launch_integrate, with the records of the drifted positions going to pos_out.
-struct PipeStep {
-  double *x, *v;
-  const uint4* ref;
-  uint4* pos_out;
-  int64_t N;
-  IntegrateArgs a;
-  double* ke_part;
-  uint32_t* dmax_bits;
-  StepFinish fin;
 };
 // Returns the number of blocks used for KE partials.  With a.shadow, dmax_bits[0] and [1] receive
 // (atomic max) the float bits of the largest squared displacement since the list build and of the
@@ -434,11 +419,6 @@ int set_wait_budget(long long cycles);
 int set_wait_budget_force(long long cycles);
 int set_wait_budget_force_half(long long cycles);
 int set_wait_budget_force_dp(long long cycles);
-int set_wait_budget_step(long long cycles);
-// The pipelined force kernel that takes the following step too: whether it is built for `lanes` threads per key,
-// and its launch (full list; a.step set; a.nbuf and a.ta from pipe_plan).  Returns the grid launched.
-bool step_pipe_lanes(int lanes);
-int launch_step_pipe(const ForceLaunch& a);
 void launch_ldc_collect(const double* x, const double* xref, int64_t N, double th2, int32_t* list, unsigned int cap,
                         unsigned int* count, cudaStream_t s);
 void launch_ldc_pairs(const double* x, const double* xref, int64_t N, Geom g, const int32_t* list, int m, double rs2,

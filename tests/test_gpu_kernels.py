@@ -99,43 +99,6 @@ def test_resident_run_matches_separate_launches(M, rho, every, mode, steps, prec
     assert ea[0] == pytest.approx(eb[0], rel=1e-2 if sum(steps) > 40 else 1e-5)
 
 
-@pytest.mark.parametrize("lanes,every,mode,T", [
-    (2, 3, ljmd.LJ_VALID_HALF_MARGIN, 12), (4, 1, ljmd.LJ_VALID_HALF_MARGIN, 12),
-    (2, 0, ljmd.LJ_VALID_DUTC, 12), (4, 3, ljmd.LJ_VALID_DUTC, 3),
-])
-def test_step_in_force_kernel_matches_separate_launches(lanes, every, mode, T):
-    """Boxes with more than two tiles per SM take a step in the force kernel; with the phase timers on the
-    integrator is a launch of its own.  340,735 particles: rows, records and components at every alignment.
-    Same tolerances as for the resident runs (one rounding of every force for 40 steps); the run is long
-    enough for the list to expire inside it, at an odd and at an even number of steps."""
-    x, L = O.fcc_lattice(44, 0.5)
-    x = x[:-1]
-    v = synth.gaussian(x.shape, 5)
-    out = []
-    for timed in (False, True):
-        log = torch.zeros((64, 4), dtype=torch.float64, device="cuda")
-        with ljmd.System(cutoff=2.5, margin=0.4, list_form=ljmd.LJ_LIST_FULL, energy_every=every, lanes=lanes) as s:
-            s.set_tuning(tile_cells=T)
-            s.set_state(x, v, L)
-            s.set_validity(mode)
-            s.set_energy_log(log)
-            s.set_profiling(timed)
-            for k in (1, 23, 16):
-                s.step(0.004, k)
-            xs, vs, _, img = s.get_state()
-            out.append((xs + img * L, vs, s.stats(), log.cpu().numpy()))
-    (xa, va, sa, la), (xb, vb, sb, lb) = out
-    assert sa["steps"] == sb["steps"] == 40 and sa["status_word"] == sb["status_word"] == 0
-    assert 40 <= sa["kernel_launches"] < sb["kernel_launches"]
-    assert sa["rebuilds"] == sb["rebuilds"] >= 3
-    assert np.abs(xa - xb).max() <= 8e-6
-    assert np.array_equal(la[:, 0], lb[:, 0])
-    n = np.count_nonzero(lb[:, 1])
-    assert (n > 0) == (every > 0)  # (a state between two calls may be recorded by both)
-    if n:
-        assert np.allclose(la[:n, 1:], lb[:n, 1:], rtol=1e-6, atol=1e-6 * np.abs(lb[:n, 1:]).max())
-
-
 @pytest.mark.parametrize("precision", [ljmd.LJ_MIXED, ljmd.LJ_FP64])
 @pytest.mark.parametrize("n,cells,spread", [
     (1, 3, 1.0), (255, 4, 1.0), (256, 4, 1.0), (257, 4, 1.0),  # blocks of 256 particles
