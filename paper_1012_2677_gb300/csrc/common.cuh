@@ -264,6 +264,14 @@ __device__ __forceinline__ void step_finish(const StepFinish& fin, double* ke_pa
   }
 }
 
+// A launch with the programmatic attribute may start before the kernel before it in the stream has ended:
+// nothing of that kernel may be read or overwritten before this returns (at once in any other launch).  The
+// next launch of the stream may start as soon as its blocks find room.
+__device__ __forceinline__ void wait_for_previous_launch() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- asynchronous bulk copies into shared memory (cp.async.bulk + mbarrier, sm_90 and later) ----
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
                  const uint2* __restrict__ tile_list, const uint16_t* __restrict__ ent, void* __restrict__ fout,
                  double* __restrict__ part, int32_t* __restrict__ status, const int* __restrict__ skip) {
   constexpr int CW = kPipeConsumers;
+  wait_for_previous_launch();
   if (skip && *skip) return;  // a device-decided run stopped before this step
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ PipeTile SS[NB];
@@ -277,8 +278,12 @@ static int force_pipe_launch(const ForceLaunch& a) {
   const size_t sm = NB * align16(tile_layout(a.ta, true, true, false).total);
   set_smem(k_force_pipe<HALF, LANES, ENERGY, NB>, sm);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count(), a.ta.ntiles));
-  k_force_pipe<HALF, LANES, ENERGY, NB><<<grid, pipe_threads(NB), sm, a.s>>>((const uint4*)a.pos, a.g, a.ta, a.c, a.rows,
-                                                                       a.tile_list, a.ent, a.f, a.part, a.status, a.skip);
+  if (a.overlap)
+    launch_overlapping(k_force_pipe<HALF, LANES, ENERGY, NB>, grid, pipe_threads(NB), sm, a.s, (const uint4*)a.pos, a.g,
+                       a.ta, a.c, a.rows, a.tile_list, a.ent, a.f, a.part, a.status, a.skip);
+  else
+    k_force_pipe<HALF, LANES, ENERGY, NB><<<grid, pipe_threads(NB), sm, a.s>>>(
+        (const uint4*)a.pos, a.g, a.ta, a.c, a.rows, a.tile_list, a.ent, a.f, a.part, a.status, a.skip);
   return grid;
 }
 template <bool HALF, int LANES, bool ENERGY>

@@ -91,8 +91,10 @@ int pipe_plan(TileArgs& ta) {
 
 int launch_force_tile(int precision, int half, int lanes, int energy, const void* pos, const uint32_t* cs, int64_t N,
                       Geom g, TileArgs ta, LJConst c, const uint2* rows, const uint2* tile_list, const uint16_t* ent,
-                      void* f, double* part, int32_t* status, int per_sm, int nbuf, cudaStream_t s, const int* skip) {
+                      void* f, double* part, int32_t* status, int per_sm, int nbuf, cudaStream_t s, const int* skip,
+                      bool overlap) {
   ForceLaunch a{pos, cs, N, g, ta, c, rows, tile_list, ent, f, part, status, skip, lanes, energy, per_sm, nbuf, 0, 0, s};
+  a.overlap = overlap ? 1 : 0;
   a.smem = force_smem_bytes(ta, precision, nbuf, half);
   a.grid = tile_grid(ta, per_sm > 0 ? per_sm : per_sm_for(a.smem));
   if (precision != LJ_MIXED) {

@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(256) k_integrate(double* __restrict__ x, doubl
                                                    double* __restrict__ ke_part, uint32_t* __restrict__ dmax_bits,
                                                    int32_t* __restrict__ status, StepFinish fin,
                                                    const int* __restrict__ skip) {
+  wait_for_previous_launch();
   if (skip && *skip) return;  // a device-decided run stopped before this step
   IntegrateAcc acc;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -244,15 +245,21 @@ static void integrate_shape(int64_t N, int& blocks, int& threads) {
 
 int launch_integrate(int precision, double* x, double* v, const void* f, void* pos, const void* ref, int64_t N,
                      IntegrateArgs a, double* ke_part, uint32_t* dmax_bits, int32_t* status, StepFinish fin,
-                     cudaStream_t s, const int* skip) {
+                     cudaStream_t s, const int* skip, bool overlap) {
   int blocks = 1, threads = kRedThreads;
   a = integrate_prepare(a);
   if (precision == LJ_MIXED) {
     integrate_shape<true>(N, blocks, threads);
-    k_integrate<true><<<blocks, threads, 0, s>>>(x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);
+    if (overlap)
+      launch_overlapping(k_integrate<true>, blocks, threads, 0, s, x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);
+    else
+      k_integrate<true><<<blocks, threads, 0, s>>>(x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);
   } else {
     integrate_shape<false>(N, blocks, threads);
-    k_integrate<false><<<blocks, threads, 0, s>>>(x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);
+    if (overlap)
+      launch_overlapping(k_integrate<false>, blocks, threads, 0, s, x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);
+    else
+      k_integrate<false><<<blocks, threads, 0, s>>>(x, v, f, pos, ref, N, a, ke_part, dmax_bits, status, fin, skip);
   }
   return blocks;
 }

@@ -782,12 +782,14 @@ static int rebuild(ljmd_sys* s) {
 
 static void* force_pos(ljmd_sys* s) { return s->precision == LJ_MIXED ? (void*)s->xq : (void*)s->pos64; }
 
+// (In a device-decided run the integrator and the pipelined force kernel may each start while the other ends: a
+// step of 500,000 particles takes 81 us instead of 84.  Not while phases are timed.)
 static int integrate(ljmd_sys* s, IntegrateArgs a, const int* skip = nullptr, const StepFinish* fin = nullptr) {
   PhaseTimer timer(s, PH_INTEGRATE);
   s->launches += 1;
   a.qk = s->g.qk;
   return launch_integrate(s->precision, s->x, s->v, s->f, force_pos(s), s->ref, s->n, a, s->part_ke, s->d_dmax,
-                          s->d_status, fin ? *fin : StepFinish{}, s->st, skip);
+                          s->d_status, fin ? *fin : StepFinish{}, s->st, skip, skip && !s->profiling);
 }
 
 // Energy record of state `step` (default: the current one); skipped on the device if *skip is set.
@@ -814,7 +816,7 @@ static int run_force(ljmd_sys* s, bool energy, const int* skip = nullptr) {
     PhaseTimer timer(s, PH_FORCE);
     s->nb_force = launch_force_tile(s->precision, half, lanes, energy ? 1 : 0, force_pos(s), s->cell_start, s->n, s->g,
                                     s->ta, s->c, s->rows, s->tile_list, s->ent, s->f, s->part_force, s->d_status,
-                                    per_sm, force_buffers(s), s->st, skip);
+                                    per_sm, force_buffers(s), s->st, skip, skip && !s->profiling && !half);
   }
   s->launches += 1;
   CKL();

@@ -116,6 +116,23 @@ void launch_load_state(const double* x_in, const double* v_in, double* x, double
 void launch_shadow_all(const double* x, int64_t N, int mixed, int qk, float4* hi, uint4* xq, dvec4* pos64, void* ref,
                        cudaStream_t s, const int* pred = nullptr);
 
+// A launch that may start while the one before it in the stream ends (its kernel calls
+// wait_for_previous_launch first).
+template <class... P, class... A>
+inline void launch_overlapping(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, (P)args...);
+}
+
 // Blocks for a grid-stride loop over n items, `per` to a block: one each, but no more than the chip holds at once
 // (2,048 threads per SM, 256-thread blocks) for a launch that a device flag may skip, so that skipping it costs
 // a launch and not the start and end of tens of thousands of blocks (6.6M particles: 15 us, then 2.5 us, for
@@ -204,7 +221,7 @@ void launch_list_tile(int precision, int half, const void* pos, const float4* hi
 int launch_force_tile(int precision, int half, int lanes, int energy, const void* pos, const uint32_t* cs, int64_t N,
                       Geom g, TileArgs ta, LJConst c, const uint2* rows, const uint2* tile_list, const uint16_t* ent,
                       void* f, double* part, int32_t* status, int per_sm, int nbuf, cudaStream_t s,
-                      const int* skip = nullptr);
+                      const int* skip = nullptr, bool overlap = false);
 // What launch_force_tile hands to the translation unit of a form.
 struct ForceLaunch {
   const void* pos;
@@ -222,6 +239,7 @@ struct ForceLaunch {
   int lanes, energy, per_sm, nbuf, grid;
   size_t smem;
   cudaStream_t s;
+  int overlap = 0;  // the pipelined kernel may start while the launch before it ends
 };
 void launch_force_mixed_half(const ForceLaunch& a);
 int launch_force_pipe_half(const ForceLaunch& a);
@@ -298,7 +316,7 @@ struct StepFinish {
 // pos: the fixed-point records (mixed) or the dvec4 copies (FP64), rewritten when a.shadow is set.
 int launch_integrate(int precision, double* x, double* v, const void* f, void* pos, const void* ref, int64_t N,
                      IntegrateArgs a, double* ke_part, uint32_t* dmax_bits, int32_t* status, StepFinish fin, cudaStream_t s,
-                     const int* skip = nullptr);
+                     const int* skip = nullptr, bool overlap = false);
 // Device-side list-validity decision after the drift of step s of a device-decided run (taken by the
 // integrator's last CTA, StepFinish.check): unless ctl->stop is already set, reads the maxima of the
 // step (squared displacement since the build and squared drift speed, float bits in dmax_bits[0],

@@ -126,3 +126,27 @@ def test_reordering_of_small_boxes(n, cells, spread, precision):
             assert np.array_equal(s.pairs(), O.pairs_within(xw, L, 3.0))
         xs, vs, _, img = s.get_state()
         assert np.array_equal(xs + img * L, x) and np.array_equal(vs, v)
+
+
+@pytest.mark.parametrize("precision,list_form", [(ljmd.LJ_MIXED, ljmd.LJ_LIST_FULL), (ljmd.LJ_FP64, ljmd.LJ_LIST_FULL)])
+def test_overlapping_launches_match_separate_ones(precision, list_form):
+    """The launches of a run of steps may start while the one before them ends; with the phase timers on, none
+    does.  The same kernels: the same bits, also where the list expires inside a run."""
+    x, L = O.fcc_lattice(44, 0.5)
+    x = x[:-1]  # 340,735 particles: more than a resident run takes
+    v = synth.gaussian(x.shape, 5)
+    out = []
+    for timed in (False, True):
+        log = torch.zeros((64, 4), dtype=torch.float64, device="cuda")
+        with ljmd.System(cutoff=2.5, margin=0.4, precision=precision, list_form=list_form, energy_every=3) as s:
+            s.set_state(x, v, L)
+            s.set_energy_log(log)
+            s.set_profiling(timed)
+            for k in (1, 23, 6):
+                s.step(0.004, k)
+            st = s.stats()
+            assert st["status_word"] == 0 and st["rebuilds"] >= 3
+            out.append((*s.get_state(), log.cpu().numpy()[:, 0], st["rebuilds"], st["kernel_launches"]))
+    assert out[0][-1] >= 60 and out[0][-2:] == out[1][-2:]
+    for a, b in zip(out[0][:-2], out[1][:-2]):
+        assert np.array_equal(a, b)
