@@ -140,7 +140,7 @@ def source_sha(path):
 
 
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_force_pipe_fcc1m_rho0.5.md")
-FORCE_SOURCE = os.path.join(ROOT, "paper_1012_2677_gb300", "csrc", "kernels_force.cu")
+FORCE_SOURCE = os.path.join(ROOT, "paper_1012_2677_gb300", "csrc", "force_launch.cuh")
 
 
 def recorded_traffic(kernel_name, N):
@@ -257,8 +257,8 @@ def run_ours(args, wl, world, rank, local):
     pe, ke, vir = s.energies()
     entries = st1["list_entries"]
     half = st1["list_form"] == ljmd.LJ_LIST_HALF  # the automatic list form of this density
-    # the mixed form on tiles: the pipelined kernel with the full list, the single-buffer one with the half
-    kernel_name = "k_force_tile" if half else "k_force_pipe"
+    # the mixed form on tiles: the pipelined kernel, with either list
+    kernel_name = "k_force_pipe (half list)" if half else "k_force_pipe"
     f_ms = prof["force_ms"] / max(prof["force_launches"], 1)
     b, stored, fl = force_kernel_work(N, entries, "mixed")
     roof = roofline(kernel_name, f_ms, b, fl, peaks, FP32_PEAK_TFLOPS, "fp32", peak_kind,
@@ -286,7 +286,7 @@ def run_ours(args, wl, world, rank, local):
                 "ms_per_step": m64["ms"] / args.steps, "steps": args.steps, "warmup": args.warmup, "list": "half",
                 "rebuilds": m64["st1"]["rebuilds"] - m64["st0"]["rebuilds"],
                 "speedup_mixed_over_fp64": (m64["ms"] / args.steps) / (ms / args.steps),
-                "roofline": roofline("k_force_pipe (FP64, half list)", f64_ms, b64, fl64, peaks, FP64_PEAK_TFLOPS,
+                "roofline": roofline("k_force_dp (FP64, half list)", f64_ms, b64, fl64, peaks, FP64_PEAK_TFLOPS,
                                      "fp64", peak_kind),
                 "phases": {k: round(p64[k], 3) for k in ("force_ms", "integrate_ms", "rebuild_ms")}}
         if rank == 0 and not args.no_cpu_baseline and not args.skip_cpu:
@@ -440,7 +440,7 @@ def run_batched(args, stream, world, rank, barrier, peaks, peak_kind):
             "graph_steps": K, "autotuned": {"tile_cells": tile, "lanes": lanes, "cost_ms": round(tune_ms, 4)},
             "rebuilds": st1["rebuilds"] - st0["rebuilds"],
             "gpu_launches": st1["kernel_launches"] - st0["kernel_launches"],
-            "roofline": roofline("k_force_batch", f_ms, bb, fl, peaks, FP32_PEAK_TFLOPS, "fp32", peak_kind),
+            "roofline": roofline("k_force_pipe (all replicas)", f_ms, bb, fl, peaks, FP32_PEAK_TFLOPS, "fp32", peak_kind),
             "timing": "host clock around one ljmd_batch_step call (graph replays, one synchronisation at the end)"}
 
 
@@ -479,7 +479,7 @@ def run_adjoint(stream, peaks, peak_kind):
         bytes_ = 4 * E + n * ((16 if name == "mixed" else 32) + 96)
         res[name] = {"seconds": t, "particle_steps_per_s": n * 50 / t, "loss": loss,
                      "grad_norm_x0": float(np.linalg.norm(gx)), "dloss_deps": gth[0], "dloss_dsigma": gth[1],
-                     "roofline": roofline("k_adjoint_tile", a_ms, bytes_, flops, peaks,
+                     "roofline": roofline("k_adjoint_tile" if name == "mixed" else "k_adjoint_dp", a_ms, bytes_, flops, peaks,
                                           FP32_PEAK_TFLOPS if name == "mixed" else FP64_PEAK_TFLOPS,
                                           "fp32" if name == "mixed" else "fp64", peak_kind,
                                           extra={"launches": prof["adjoint_launches"]})}

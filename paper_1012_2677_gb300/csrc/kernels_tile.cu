@@ -1,5 +1,6 @@
 // Cell-column tiles staged in shared memory: pair-list construction (Alg. 1 over the grid of
-// Sec. 2.2, stored as the sorted list of Sec. 2.4) and the force over that list (Alg. 4-6).
+// Sec. 2.2, stored as the sorted list of Sec. 2.4), tile sizes and list export.  The force over that list
+// (Alg. 4-6) and the adjoint pass, which stage the same tiles, have translation units of their own.
 //
 // A tile is T consecutive cells along z of one (cx, cy) column.  Its CTA stages the particles
 // of the 9 neighbouring columns over the cells z0-1 .. z0+T (9 (T+2) cells, wrapped

@@ -5,7 +5,6 @@
 #include "common.cuh"
 
 #include <algorithm>
-#include <type_traits>
 
 namespace ljmd {
 
