@@ -1288,8 +1288,7 @@ int ljmd_get_state(ljmd_sys* sys, double* x, double* v, double* f, int32_t* img,
     if (!on_device) CK(cudaMemcpyAsync(v, dst, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost, st));
   }
   if (f) {
-    CK(cudaStreamSynchronize(st));  // x_alt may be in use by the x copy above
-    double* dst = on_device ? f : sys->x_alt;
+    double* dst = on_device ? f : sys->x_alt;  // (after the x copy above, in stream order)
     if (sys->precision == LJ_MIXED) launch_scatter_back_f32x4_to_f64x3((const float4*)sys->f, dst, sys->id, N, st);
     else launch_scatter_back_f64x4_to_f64x3((const dvec4*)sys->f, dst, sys->id, N, st);
     CKL();
@@ -1301,8 +1300,7 @@ int ljmd_get_state(ljmd_sys* sys, double* x, double* v, double* f, int32_t* img,
     CKL();
     if (!on_device) CK(cudaMemcpyAsync(img, dst, sizeof(int32_t) * 3 * N, cudaMemcpyDeviceToHost, st));
   }
-  CK(cudaStreamSynchronize(st));
-  return check_status(sys);
+  return check_status(sys);  // waits for the stream: the status copy is the last of its work
 }
 
 int ljmd_build_pairlist(ljmd_sys* sys, double cutoff, double margin) {
@@ -1445,11 +1443,12 @@ int ljmd_energies(ljmd_sys* sys, double* pe, double* ke, double* virial) {
   if (sys->n <= 0) return LJ_ESTATE;
   if (sys->energy_step != sys->steps) TRY(finalize_energies_now(sys));
   CK(cudaMemcpyAsync(sys->h_f64, sys->d_energies, 4 * sizeof(double), cudaMemcpyDeviceToHost, sys->st));
-  CK(cudaStreamSynchronize(sys->st));
+  int32_t w = 0;
+  TRY(device_status(sys, &w));  // waits for the stream
   if (pe) *pe = sys->h_f64[0];
   if (ke) *ke = sys->h_f64[1];
   if (virial) *virial = sys->h_f64[2];
-  return check_status(sys);
+  return w ? LJ_EDEVICE : LJ_OK;
 }
 
 int ljmd_set_energy_log(ljmd_sys* sys, double* device_log, int64_t capacity) {
