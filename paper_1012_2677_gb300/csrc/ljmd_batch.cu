@@ -288,25 +288,20 @@ static int enqueue_rebuild(ljmd_batch* b, const int* pred) {
   const int64_t N = b->N;
   cudaStream_t st = b->st;
   // zero fills are predicated too: the counters of the last construction must survive skipped ones
-  launch_zero_words(b->cell_count, sizeof(uint32_t) * b->ncells, pred, st);
+  launch_zero_words({{b->cell_count, b->cell_fill, (uint32_t*)b->counter, (uint32_t*)b->sizes}, {b->ncells, b->ncells, 4, 4}},
+                    pred, st);
   launch_wrap_label_batch(b->x, b->img, N, b->rep_of, b->reps, b->offset, b->cell_of, b->cell_count, b->status, pred,
                           st);
   b->launches += 1 + launch_scan_u32(b->cell_count, b->cell_start, b->ncells, b->scan_tmp, st, pred);
-  launch_zero_words(b->cell_fill, sizeof(uint32_t) * b->ncells, pred, st);
   launch_scatter(b->cell_of, b->cell_start, b->cell_fill, b->perm, N, st, pred);
   launch_cell_rank(b->cell_start, b->ncells, b->perm, b->id, b->perm_id, st, pred);
   launch_gather_state(b->perm_id, N, b->x, b->x_alt, b->v, b->v_alt, b->id, b->id_alt, b->img, b->img_alt, nullptr,
                       nullptr, 0, st, pred);
-  launch_copy_words(b->x_alt, b->x, 24 * N, pred, st);
-  launch_copy_words(b->v_alt, b->v, 24 * N, pred, st);
-  launch_copy_words(b->id_alt, b->id, 4 * N, pred, st);
-  launch_copy_words(b->img_alt, b->img, 12 * N, pred, st);
-  launch_shadow_all(b->x, N, 1, b->g0.qk, b->hi, b->xq, nullptr, b->ref, st, pred);
-  launch_zero_words(b->counter, 2 * sizeof(unsigned long long), pred, st);
-  launch_zero_words(b->sizes, 4 * sizeof(unsigned int), pred, st);
+  launch_restore_state({b->x_alt, b->v_alt, b->id_alt, b->img_alt, b->x, b->v, b->id, b->img, b->hi, b->xq, (uint4*)b->ref},
+                       N, b->g0.qk, pred, st);
   launch_list_batch(b->hi, b->x, b->cell_start, N, b->g0, b->caps, b->band, b->rows, b->tile_list, b->ent,
                     (uint64_t)b->ent_cap, b->counter, b->sizes + 3, b->status, b->reps, b->R, b->tile_rep, pred, st);
-  b->launches += 14;
+  b->launches += 6;
   BKL();
   return LJ_OK;
 }

@@ -136,7 +136,7 @@ inline void launch_overlapping(void (*kernel)(P...), int grid, int threads, size
 // Blocks for a grid-stride loop over n items, `per` to a block: one each, but no more than the chip holds at once
 // (2,048 threads per SM, 256-thread blocks) for a launch that a device flag may skip, so that skipping it costs
 // a launch and not the start and end of tens of thousands of blocks (6.6M particles: 15 us, then 2.5 us, for
-// each of the dozen launches of a construction that a batch's step skips).
+// each launch of a construction that a batch's step skips).
 inline int stride_grid(int64_t n, int per, const int* pred) {
   int64_t b = (n + per - 1) / per, most = 1048576;
   if (pred) {
@@ -426,7 +426,20 @@ void launch_wrap_label_batch(double* x, int32_t* img, int64_t N, const int32_t* 
                              const int* pred, cudaStream_t s);
 void launch_rebuild_flag(const uint32_t* dmax_bits, float limit2, int* flag, long long* rebuilds, cudaStream_t s);
 void launch_copy_words(const void* in, void* out, int64_t bytes, const int* pred, cudaStream_t s);
-void launch_zero_words(void* out, int64_t bytes, const int* pred, cudaStream_t s);
+struct ZeroArgs {
+  uint32_t* out[4];
+  int64_t words[4];
+};
+void launch_zero_words(ZeroArgs z, const int* pred, cudaStream_t s);
+struct RestoreArgs {
+  const double *x_in, *v_in;
+  const int32_t *id_in, *img_in;
+  double *x, *v;
+  int32_t *id, *img;
+  float4* hi;
+  uint4 *xq, *ref;
+};
+void launch_restore_state(const RestoreArgs& a, int64_t N, int qk, const int* pred, cudaStream_t s);
 void launch_replica_ke(const double* v, int64_t N, const ReplicaGeo* reps, int R, double* ke_rep, cudaStream_t s);
 void launch_load_batch(const double* xin, const double* vin, double* x, double* v, int32_t* id, int32_t* img,
                        int64_t N, const int32_t* rep_of, const ReplicaGeo* reps, double offset, cudaStream_t s);
