@@ -48,6 +48,9 @@ static void force_tile_mixed(const ForceLaunch& a) {
 //             (loaded one tile earlier) -> wait full[b] -> (boundary tiles: image shifts) -> arrive ready[b];
 //   consumers: wait ready[b] -> forces of the warp's share of the tile's own particles -> arrive
 //             empty[b].
+// A tile beyond the capacities (a batch's device-side construction can make one) is recorded in the status
+// word and skipped: it goes through ready and empty as any other, but nothing is copied and full[b]
+// completes no phase, so the producer counts the buffer's fills apart from its uses.
 // Every wait is bounded; a producer that gives up marks the slot aborted and releases the
 // consumers, which then leave.  No copy is in flight when a warp leaves.
 //
@@ -134,6 +137,7 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
     int64_t t = blockIdx.x + b * stride;
     uint2 d = make_uint2(0u, 0u);
     if (t < ta.ntiles) d = load(t);
+    uint32_t fills = 0;  // fills of the buffer so far: a phase of full[b] each (a skipped tile has none)
     for (uint32_t use = 0; t < ta.ntiles; t += NB * stride, ++use) {
       const uint32_t total = __shfl_sync(0xffffffffu, d.x, 18), own = __shfl_sync(0xffffffffu, d.y, 18);
       const int gown0 = (int)__shfl_sync(0xffffffffu, d.x, 19), n_own = (int)(own >> 16);
@@ -205,17 +209,18 @@ __global__ void __launch_bounds__(pipe_threads(NB), 1)
       if (tn < ta.ntiles) d = load(tn);
       if (staged) {
         bool landed = true;
-        if (lane == 0) landed = mbar_wait(&full[b], use & 1u, budget);
+        if (lane == 0) landed = mbar_wait(&full[b], fills & 1u, budget);
         landed = __shfl_sync(0xffffffffu, landed ? 1 : 0, 0) != 0;
         if (!landed) {
           if (lane == 0) {
             atomicOr(status, LJ_ST_TIMEOUT);
-            mbar_wait(&full[b], use & 1u, kWaitBudget);  // let copies in flight land before leaving
+            mbar_wait(&full[b], fills & 1u, kWaitBudget);  // let copies in flight land before leaving
             SS[b].valid = -1;
             mbar_arrive(&ready[b]);
           }
           break;
         }
+        ++fills;
         if (images) pipe_shift((uint4*)(buf + L.pos), run, ax, ay, az, lane);
       }
       __syncwarp();

@@ -1,0 +1,47 @@
+"""Calls at the limits of the kernels' capacities, units and waits: what was built for an ordinary liquid
+must stay right, be refused cleanly or give up cleanly outside it."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1012_2677_gb300 import ljmd, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _min_image(d, L):
+    return d - L * np.round(d / L)
+
+
+def test_batch_tile_beyond_the_capacities_is_skipped_alone():
+    """The capacities of a batch are fixed at the host construction.  Replica 0 contracts (v = -1.6 (x - centre), an
+    FCC gas of rho 0.2: its density triples in 60 steps and no pair comes close), so a later device-side
+    construction makes tiles beyond 1.4 times the largest there was: the call must end with LJ_EDEVICE and the
+    status bit, and every other replica, whose tiles go through the same buffers after the skipped ones (98 tiles
+    a replica, 608 buffers on the chip), must be where a single system takes it: 60 steps accumulate at most
+    dt^2 60^2 / 2 times the force difference of the two summation orders (1e-5 of |F| < 10), 3e-6, and less than
+    ten times that with the growth of a difference over 0.24 time units."""
+    R, N, rho, dt, steps = 20, 2000, 0.2, 0.004, 60
+    xs, vs = [], []
+    for r in range(R):
+        x, L = synth.fcc_thinned(N, rho, 40 + r)
+        xs.append(synth.dyadic(x))
+        vs.append(synth.dyadic(-1.6 * (xs[0] - 0.5 * L) if r == 0 else synth.thermal_velocities(N, 1.0, 60 + r)))
+    x, v = np.concatenate(xs), np.concatenate(vs)
+    bx, bv, bf = (np.empty_like(x) for _ in range(3))
+    with ljmd.Batch([N] * R, [L] * R, cutoff=2.5, margin=0.3) as b:
+        assert b.stats()["tiles"] > 152 * 4 + 98
+        b.set_state(x, v)
+        with pytest.raises(ljmd.LjmdError) as e:
+            b.step(dt, steps)
+        assert e.value.code == ljmd.LJ_EDEVICE
+        assert b.stats()["status_word"] & (ljmd.LJ_ST_CELL_RANGE | ljmd.LJ_ST_LIST_OVERFLOW)
+        assert not b.stats()["status_word"] & (ljmd.LJ_ST_TIMEOUT | ljmd.LJ_ST_NONFINITE)
+        with pytest.raises(ljmd.LjmdError):  # the arrays are filled; the status is still raised
+            ljmd._chk(ljmd.load().ljmd_batch_get_state(b.h, *(a.ctypes.data for a in (bx, bv, bf)), 0), "get_state")
+    for r in range(1, R):
+        with ljmd.System(cutoff=2.5, margin=0.3, precision=ljmd.LJ_MIXED) as s:
+            s.set_state(xs[r], vs[r], L)
+            s.step(dt, steps)
+            sx, _, _, _ = s.get_state()
+        assert np.abs(_min_image(bx[r * N:(r + 1) * N] - sx, L)).max() < 3e-5, r
