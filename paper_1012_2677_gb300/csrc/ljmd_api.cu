@@ -642,6 +642,19 @@ static int sort_small(ljmd_sys* s, bool* sorted, bool* guessed) {
   return LJ_OK;
 }
 
+// Reads the counters of a construction back and sees whether k_sort, if it ran, got to its end.  If a wait
+// of it ran out, its outputs are not to be used: the state stays where it was.
+static int read_grid(ljmd_sys* s, bool sorted) {
+  ljmd_sys* sys = s;
+  CK(cudaMemcpyAsync(s->h_grid, s->d_grid, sizeof(GridCtl), cudaMemcpyDeviceToHost, s->st));
+  CK(cudaStreamSynchronize(s->st));
+  if (!sorted || (int64_t)s->h_grid->ticket == sort_grid(s->n)) return LJ_OK;
+  swap_state(s);
+  s->sort_dirty = true;
+  s->have_list = s->forces_current = false;
+  return LJ_EDEVICE;
+}
+
 // ----------------------------------------------------------------------------------------------
 // Pair-list construction: fold, label, counting sort (Fig. 3), reorder (Sec. 3.3), sorted list.
 static int rebuild(ljmd_sys* s) {
@@ -672,6 +685,8 @@ static int rebuild(ljmd_sys* s) {
     launch_shadow_all(s->x, N, s->precision == LJ_MIXED, s->g.qk, s->hi, s->xq, s->pos64, s->ref, st);
     CKL();
   }
+  // (k_sort's outputs are used without a look at it only by the list kernel that it lets run)
+  if (sorted && !guessed) TRY(read_grid(s, sorted));
   const int half = s->list_half ? 1 : 0;
   uint64_t total = 0;
   int dev = 0, smem_max = 0;
@@ -701,14 +716,7 @@ static int rebuild(ljmd_sys* s) {
       s->launches += 1;
       CKL();
       const GridCtl* hg = s->h_grid;
-      CK(cudaMemcpyAsync(s->h_grid, s->d_grid, sizeof(GridCtl), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));  // one round trip: sizes, list size, longest segment and status
-      if (sorted && (int64_t)hg->ticket != sort_grid(N)) {  // a wait of k_sort ran out: the state is where it was
-        swap_state(s);
-        s->sort_dirty = true;
-        s->have_list = s->forces_current = false;
-        return LJ_EDEVICE;
-      }
+      TRY(read_grid(s, sorted));  // one round trip: sizes, list size, longest segment and status
       if (guessed && !hg->ok) {  // a size beyond its guess: the list kernel has not run
         guessed = false;
         TRY(choose_tiles(s, t_cap));

@@ -45,3 +45,43 @@ def test_batch_tile_beyond_the_capacities_is_skipped_alone():
             s.step(dt, steps)
             sx, _, _, _ = s.get_state()
         assert np.abs(_min_image(bx[r * N:(r + 1) * N] - sx, L)).max() < 3e-5, r
+
+
+TINY = 16  # SM clock cycles: no wait of a kernel is over that fast
+
+
+def _state_whatever_the_status(s, n):
+    x, v, f = (np.empty((n, 3)) for _ in range(3))
+    img = np.empty((n, 3), dtype=np.int32)
+    ljmd.load().ljmd_get_state(s.h, *(a.ctypes.data for a in (x, v, f, img)), 0)
+    return x, v, f, img
+
+
+# 10,700 particles in 27 cells: the tile capacities guessed from the mean counts do not fit in shared memory (237 KB
+# of 227), the ones measured afterwards do (221 KB)
+@pytest.mark.parametrize("N,rho,rc,guess_fits", [(4000, 0.5, 2.5, True), (10700, 0.94, 6.9, False)])
+def test_reordering_of_a_small_box_times_out(N, rho, rc, guess_fits):
+    x, L = synth.fcc_thinned(N, rho, 5)
+    x = synth.dyadic(O.wrap(x + synth.displacements(N, 0.03, 6), L))
+    v = synth.dyadic(synth.thermal_velocities(N, 1.0, 7))
+    with ljmd.System(cutoff=rc, margin=0.5, precision=ljmd.LJ_MIXED, list_form=ljmd.LJ_LIST_FULL) as s:
+        s.set_state(x, v, L)
+        ljmd.ljmd_set_wait_budget(TINY)
+        try:
+            with pytest.raises(ljmd.LjmdError) as e:
+                s.build_pairlist()
+        finally:
+            ljmd.ljmd_set_wait_budget(0)
+        assert e.value.code == ljmd.LJ_EDEVICE
+        st = s.stats()
+        assert st["status_word"] == ljmd.LJ_ST_TIMEOUT and st["rebuilds"] == 0
+        if not guess_fits:  # given up before the list kernel: the reordering is the only launch
+            assert st["kernel_launches"] == 1
+        gx, gv, _, img = _state_whatever_the_status(s, N)
+        assert np.array_equal(gx, x) and np.array_equal(gv, v) and not img.any()
+    with ljmd.System(cutoff=rc, margin=0.5, precision=ljmd.LJ_MIXED, list_form=ljmd.LJ_LIST_FULL) as s:
+        s.set_state(x, v, L)
+        s.compute_forces()
+        _, _, f, _ = s.get_state()
+    F, _, _ = O.forces(x, L, O.LJParams(rc_over_sigma=rc))
+    assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-5
