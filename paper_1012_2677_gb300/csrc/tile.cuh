@@ -868,8 +868,8 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 
 // ---------------------------------------------------------------------------------------------
 // Pair work by queues.  A warp takes a run of consecutive keys.  It first filters their rows in FP32
-// (differences of fixed-point copies, r_c^2 widened by a relative 4e-6 against the 3e-7 that the
-// quantisation and FP32 rounding can err) and queues the kept (key, partner) pairs in shared memory;
+// (differences of fixed-point copies, r_c^2 widened by what the copies' rounding, an absolute u each, and
+// the FP32 arithmetic can err: LJConst::rc2w) and queues the kept (key, partner) pairs in shared memory;
 // then each lane evaluates a contiguous share of the queue, so that at most the last pair of a lane
 // idles and a key's sum needs no shuffles.  A lane stores the partial sum of a key that began in an earlier
 // lane in its head slot, every other one in the key's slot; the key's own lane adds slot and heads in
@@ -1129,7 +1129,7 @@ struct DpForce {
     f8c2 = 8.0 * c.eps * c.c2s;
     f24s = 24.0 * c.eps * sig6;
     f48s = 48.0 * c.eps * sig6 * sig6;
-    cut2 = c.rc2q * 1.000004f;
+    cut2 = c.rc2w;
     sp = (const dvec4*)(smem + D.L.pos);
     sq = (const uint4*)(smem + D.xq);
     fout = f;

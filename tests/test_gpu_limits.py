@@ -85,3 +85,39 @@ def test_reordering_of_a_small_box_times_out(N, rho, rc, guess_fits):
         _, _, f, _ = s.get_state()
     F, _, _ = O.forces(x, L, O.LJParams(rc_over_sigma=rc))
     assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-5
+
+
+@pytest.mark.parametrize("list_form", [ljmd.LJ_LIST_FULL, ljmd.LJ_LIST_HALF])
+@pytest.mark.parametrize("sigma", [50.0, 1e-3, 1e-5, 3.4e-10])
+def test_fp64_form_in_any_unit_of_length(sigma, list_form):
+    """The FP64 form's results do not depend on the unit of length (argon in metres: sigma = 3.4e-10): forces,
+    energies and the Hessian-vector product with the tolerances of the other FP64 tests, and a few steps of a box
+    that runs resident.  Positions and box are multiples of the storage's last bit q (2^-50 beside the offset 4 of
+    a small box; 2^-42 at least where the box is 715), so that nothing is rounded on the way in.  A step rounds a
+    stored position by q / 2 at most, and the image of a particle outside the box by as much; through the forces
+    (K dt^2 < 0.01) that adds a hundredth: five steps stay within 4 q of the oracle's."""
+    q = 2.0 ** (-50 if sigma < 1.0 else -41)
+    p = O.LJParams(sigma=sigma, rc_over_sigma=2.5)
+    x, L = O.fcc_lattice(8, 0.7)
+    x = O.wrap(x + synth.displacements(len(x), 0.06, 3), L)
+    x, L = np.round(x * sigma / q) * q, np.round(L * sigma / q) * q
+    w = synth.gaussian(x.shape, 11)
+    F, pe, vir = O.forces(x, L, p)
+    with ljmd.System(sigma=sigma, cutoff=2.5 * sigma, margin=0.5 * sigma, precision=ljmd.LJ_FP64,
+                     list_form=list_form) as s:
+        s.set_state(x, w, L)
+        s.compute_forces()
+        _, _, f, _ = s.get_state()
+        gpe, _, gvir = s.energies()
+        assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-11
+        assert gpe == pytest.approx(pe, rel=1e-12) and gvir == pytest.approx(vir, rel=1e-12)
+        s.step(0.002 * sigma, 5)
+        xs, _, _, img = s.get_state()
+        xo, *_ = O.vv_run(x, w, L, 0.002 * sigma, 5, p)
+        assert np.abs(xs + img * L - xo).max() <= 4 * q
+    if list_form == ljmd.LJ_LIST_FULL:
+        ref = O.hvp(x, L, w, p)
+        with ljmd.System(sigma=sigma, cutoff=2.5 * sigma, margin=0.5 * sigma, precision=ljmd.LJ_FP64) as s:
+            s.set_state(x, None, L)
+            hw, _ = s.hvp(w)
+        assert np.sqrt(((hw - ref) ** 2).sum(1)).max() / np.sqrt((ref ** 2).sum(1).mean()) <= 1e-10
