@@ -427,7 +427,11 @@ int ljmd_batch_get_pairs(ljmd_batch* b, int32_t replica, int64_t* ij, int64_t ca
 
 int ljmd_batch_get_stats(ljmd_batch* b, ljmd_batch_stats* out);
 
-/* Kernel shape: tile_cells (1..14, 0 keeps) and force lanes (2, 4, 8; 0 keeps).  Drops the graph. */
+/*
+ * Kernel shape: tile_cells (cells per tile along z at density 0.5, 1..14, 0 keeps; shorter in denser replicas,
+ * where a tile would have more than 150 particles of its own, and where its shared memory would not fit) and
+ * force lanes (2, 4, 8; 0 keeps).  Drops the graph.
+ */
 int ljmd_batch_set_tuning(ljmd_batch* b, int32_t tile_cells, int32_t lanes);
 
 /*

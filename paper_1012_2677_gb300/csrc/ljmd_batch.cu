@@ -35,10 +35,11 @@ struct ljmd_batch {
   int32_t* tile_rep = nullptr;  // replica of every global tile
   TileArgs caps{};
   int64_t ncells = 0;
-  // preferred cells per tile along z: 256 replicas of 500 to 50,000 particles at densities 0.3 to 0.9 take
-  // 1.25, 1.24, 1.06, 0.96, 1.33 ms per force launch at 4, 6, 8, 10, 12 (four threads per key), and
-  // 102, 97, 89, 88, 107 ms for 40 steps
+  // preferred cells per tile along z (replica_tile): 256 replicas of 500 to 50,000 particles at densities 0.3
+  // to 0.9, r_s = 2.8, take 1.25, 1.24, 1.06, 0.96, 1.33 ms per force launch at 4, 6, 8, 10, 12 (four threads
+  // per key), and 102, 97, 89, 88, 107 ms for 40 steps
   int tile_T = 10;
+  int tile_cap = kMaxTileT;  // longest tile whose shared memory fitted (host_build)
   int lanes = 4;   // threads per key in the force kernel
   // device state (sorted by cell within each replica)
   double *x = nullptr, *v = nullptr, *x_alt = nullptr, *v_alt = nullptr;
@@ -128,11 +129,17 @@ static int join_user(ljmd_batch* b) {
 
 // Cells per tile along z for one replica: the preferred T at density 0.5, scaled by 0.5 / rho so that
 // a tile stages about the same number of particles in every replica (the shared-memory capacity is
-// set by the densest replica's tiles).
+// set by the densest replica's tiles), and no more than 150 particles of its own: with a longer search length
+// the cells hold more, and where two tiles do not fit on an SM the steps lose the pipelined kernel (16
+// replicas of 30,000 particles, us a step at 1 cell, 2, ...: r_s 4.5, rho 0.7, 87 a cell: 252, 395, 363, 393,
+// 1284; r_s 3.8, rho 0.8, 59 a cell: 277, 246, 310, 290, 377, 464; r_s 3.3, rho 0.5, 23 a cell: 250, 187, 171,
+// 154, 172, 152, 183, 199, 213).
+constexpr double kTileKeys = 150.0;
 static int replica_tile(int pref, int64_t n_cells, int64_t count, double L) {
-  const double rho = (double)count / (L * L * L);
+  const double rho = (double)count / (L * L * L), ppc = (double)count / (double)(n_cells * n_cells * n_cells);
   int T = (int)lround((double)pref * 0.5 / std::max(rho, 1e-9));
   T = std::max(1, std::min(T, pref));
+  T = std::min(T, std::max(1, (int)std::min(kTileKeys / std::max(ppc, 1e-9), (double)kMaxTileT)));
   T = std::min<int>(T, (int)n_cells - 2);
   return std::max(1, std::min(T, kMaxTileT));
 }
@@ -148,6 +155,22 @@ static int upload_tile_rep(ljmd_batch* b) {
   BTRY(balloc(&b->tile_rep, tr.size()));
   BK(cudaMemcpy(b->tile_rep, tr.data(), sizeof(int32_t) * tr.size(), cudaMemcpyHostToDevice));
   return LJ_OK;
+}
+
+// The replicas' tiles for the preferred length, none longer than tile_cap, and the tables that depend on them.
+static int set_tiles(ljmd_batch* b) {
+  int64_t tiles = 0;
+  for (ReplicaGeo& rg : b->reps_h) {
+    rg.T = std::min(replica_tile(b->tile_T, rg.n, rg.count, rg.g.L), b->tile_cap);
+    rg.ntz = (rg.n + rg.T - 1) / rg.T;
+    rg.tile_base = tiles;
+    tiles += (int64_t)rg.n * rg.n * rg.ntz;
+  }
+  if (tiles > 0x7fffffffLL) return LJ_ERANGE;
+  b->caps.ntiles = tiles;
+  BK(cudaMemcpyAsync(b->reps, b->reps_h.data(), sizeof(ReplicaGeo) * b->R, cudaMemcpyHostToDevice, b->st));
+  BTRY(balloc(&b->tile_list, kTileWords * (size_t)tiles));
+  return upload_tile_rep(b);
 }
 
 // Coefficients of the truncation terms of Eq. 2 (Sec. 2.1), as in the single-system path.
@@ -187,7 +210,7 @@ static int setup_replicas(ljmd_batch* b) {
   int qk = 31 - (int)ceil(log2(W));
   if (qk > 30) qk = 30;
   b->reps_h.assign(b->R, ReplicaGeo{});
-  int64_t tiles = 0, cells = 0;
+  int64_t cells = 0;
   for (int r = 0; r < b->R; ++r) {
     const double L = b->box[r];
     if (!(L >= 2.0 * (rs + p.margin)) || !isfinite(L)) return LJ_EINVAL;
@@ -216,25 +239,19 @@ static int setup_replicas(ljmd_batch* b) {
     g.qu = (float)ldexp(1.0, -qk);
     g.Lq = (uint32_t)fmod(nearbyint(ldexp(L, qk)), 4294967296.0);
     g.q_inv_L = (float)(ldexp(1.0, -qk) / L);
-    const int T = replica_tile(b->tile_T, n, b->count[r], L);
     rg.n = (int32_t)n;
-    rg.T = T;
-    rg.ntz = (int32_t)((n + T - 1) / T);
-    rg.tile_base = tiles;
     rg.cell_base = cells;
     rg.base = b->base[r];
     rg.count = b->count[r];
-    tiles += n * n * rg.ntz;
     cells += n * n * n;
   }
-  if (cells > 0xffffffffLL || tiles > 0x7fffffffLL) return LJ_ERANGE;
+  if (cells > 0xffffffffLL) return LJ_ERANGE;
   b->g0 = b->reps_h[0].g;
   b->ncells = cells;
   b->caps.n = 0;
   b->caps.T = 0;
   b->caps.ntz = 0;
   b->caps.whole = 0;
-  b->caps.ntiles = tiles;
   double c2, c0;
   batch_truncation(p.cutoff / p.sigma, p.truncation, &c2, &c0);
   LJConst& c = b->c;
@@ -272,14 +289,11 @@ static int setup_replicas(ljmd_batch* b) {
   b->band.hi = (float)(rs * rs + band);
   b->disp_limit = 0.5 * p.margin - (2.0 * sqrt(3.0) * ldexp(1.0, -qk) + 1e-6 * (0.5 * p.margin) + 1e-9);
   BTRY(balloc(&b->reps, b->R));
-  BK(cudaMemcpyAsync(b->reps, b->reps_h.data(), sizeof(ReplicaGeo) * b->R, cudaMemcpyHostToDevice, b->st));
-  BTRY(upload_tile_rep(b));
+  BTRY(set_tiles(b));
   BTRY(balloc(&b->cell_count, b->ncells));
   BTRY(balloc(&b->cell_start, b->ncells + 1));
   BTRY(balloc(&b->cell_fill, b->ncells));
-  BTRY(balloc(&b->scan_tmp, scan_tmp_words(b->ncells)));
-  BTRY(balloc(&b->tile_list, kTileWords * (size_t)tiles));
-  return LJ_OK;
+  return balloc(&b->scan_tmp, scan_tmp_words(b->ncells));
 }
 
 // The rebuild of every replica's cell sort and list: fold, label, counting sort, reorder, shadow,
@@ -323,24 +337,36 @@ static int host_build(ljmd_batch* b) {
   launch_wrap_label_batch(b->x, b->img, b->N, b->rep_of, b->reps, b->offset, b->cell_of, b->cell_count, b->status,
                           nullptr, st);
   b->launches += 1 + launch_scan_u32(b->cell_count, b->cell_start, b->ncells, b->scan_tmp, st);
-  BK(cudaMemsetAsync(b->sizes, 0, 4 * sizeof(unsigned int), st));
-  launch_tile_sizes_batch(b->cell_start, b->caps, b->reps, b->R, b->tile_rep, b->sizes, st);
-  b->launches += 1;
-  BKL();
-  BK(cudaMemcpyAsync(b->h_u64, b->sizes, 2 * sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-  BK(cudaStreamSynchronize(st));
-  unsigned int staged, own;
-  memcpy(&staged, (char*)b->h_u64, 4);
-  memcpy(&own, (char*)b->h_u64 + 4, 4);
-  // headroom for the density fluctuations of the steps between host constructions
-  b->caps.max_staged = (int32_t)std::min<double>(65535.0, ceil(staged * 1.3) + 32);
-  b->caps.max_own = (int32_t)(ceil(own * 1.4) + 16);
-  b->caps.max_chunks = 1;
-  if (staged > 65535) return LJ_ERANGE;
   int dev = 0, smem_max = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (batch_list_smem_bytes(b->caps) > (size_t)smem_max) return LJ_ERANGE;
+  for (;;) {
+    BK(cudaMemsetAsync(b->sizes, 0, 4 * sizeof(unsigned int), st));
+    launch_tile_sizes_batch(b->cell_start, b->caps, b->reps, b->R, b->tile_rep, b->sizes, st);
+    b->launches += 1;
+    BKL();
+    BK(cudaMemcpyAsync(b->h_u64, b->sizes, 2 * sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
+    BK(cudaStreamSynchronize(st));
+    unsigned int staged, own;
+    memcpy(&staged, (char*)b->h_u64, 4);
+    memcpy(&own, (char*)b->h_u64 + 4, 4);
+    // headroom for the density fluctuations of the steps between host constructions
+    b->caps.max_staged = (int32_t)std::min<double>(65535.0, ceil(staged * 1.3) + 32);
+    b->caps.max_own = (int32_t)(ceil(own * 1.4) + 16);
+    b->caps.max_chunks = 1;
+    b->caps.max_list = 0;
+    TileArgs tz = b->caps;
+    tz.list_cap = 0;
+    const bool fits = staged <= 65535 && batch_list_smem_bytes(tz) <= (size_t)smem_max &&
+                      batch_force_smem_bytes(tz) <= (size_t)smem_max;
+    // shorter tiles until the list kernel and two buffers of the pipelined force kernel fit
+    int longest = 1;
+    for (const ReplicaGeo& rg : b->reps_h) longest = std::max(longest, rg.T);
+    if (fits && (longest == 1 || pipe_plan(tz) > 0)) break;
+    if (longest == 1) return LJ_ERANGE;
+    b->tile_cap = longest - 1;
+    BTRY(set_tiles(b));
+  }
   if (b->ent_cap == 0) {
     double est = 0.0;
     for (int r = 0; r < b->R; ++r) {
@@ -388,7 +414,6 @@ static int host_build(ljmd_batch* b) {
     TileArgs tz = b->caps;
     tz.list_cap = 0;
     const size_t base_bytes = batch_force_smem_bytes(tz);
-    if (base_bytes > (size_t)smem_max) return LJ_ERANGE;
     // room for the list next to the positions so that 4 CTAs share an SM where possible
     const int64_t target = std::max<int64_t>((int64_t)base_bytes + 4096, 54 * 1024);
     const int64_t room = (std::min<int64_t>(smem_max, target) - (int64_t)base_bytes) / 2 - 16;
@@ -767,21 +792,10 @@ int ljmd_batch_set_tuning(ljmd_batch* b, int32_t tile_cells, int32_t lanes) {
   if (lanes) b->lanes = lanes;
   if (tile_cells && tile_cells != b->tile_T) {
     b->tile_T = tile_cells;
-    for (ReplicaGeo& rg : b->reps_h) {
-      rg.T = replica_tile(tile_cells, rg.n, rg.count, rg.g.L);
-      rg.ntz = (rg.n + rg.T - 1) / rg.T;
-    }
-    int64_t tiles = 0;
-    for (ReplicaGeo& rg : b->reps_h) {
-      rg.tile_base = tiles;
-      tiles += (int64_t)rg.n * rg.n * rg.ntz;
-    }
-    b->caps.ntiles = tiles;
-    BK(cudaMemcpyAsync(b->reps, b->reps_h.data(), sizeof(ReplicaGeo) * b->R, cudaMemcpyHostToDevice, b->st));
-    BTRY(balloc(&b->tile_list, kTileWords * (size_t)tiles));
-    BTRY(upload_tile_rep(b));
+    b->tile_cap = kMaxTileT;
     b->have_list = false;
     b->forces_current = false;
+    BTRY(set_tiles(b));
   }
   drop_graph(b);
   return LJ_OK;

@@ -47,6 +47,52 @@ def test_batch_tile_beyond_the_capacities_is_skipped_alone():
         assert np.abs(_min_image(bx[r * N:(r + 1) * N] - sx, L)).max() < 3e-5, r
 
 
+def _liquid(N, rho, seed):
+    x, L = synth.fcc_thinned(N, rho, seed)
+    return O.wrap(x + synth.displacements(N, 0.05, seed + 1), L), L
+
+
+def _droplet(N, L, seed):
+    """A ball of N particles at density 0.95 in a box that is otherwise empty."""
+    x, l = _liquid(8 * N // 4, 0.95, seed)
+    r = np.sqrt(((x - 0.5 * l) ** 2).sum(1))
+    return x[np.argsort(r)[:N]] - 0.5 * l + 0.5 * L, L
+
+
+@pytest.mark.parametrize("rc,make", [
+    (3.5, lambda: [_liquid(6000, 0.8, 3), _liquid(900, 0.5, 4)]),
+    (4.5, lambda: [_liquid(9000, 0.85, 5), _liquid(2500, 0.4, 6)]),
+    (5.0, lambda: [_droplet(10000, 66.0, 7), _liquid(2500, 0.5, 8)]),  # tiles by the mean count do not fit here
+])
+def test_batch_with_a_long_cutoff(rc, make):
+    """Cells of a long search length hold many particles: the default tiles must still fit."""
+    boxes = make()
+    xs = [synth.dyadic(x) for x, _ in boxes]
+    n, box = [len(x) for x in xs], [L for _, L in boxes]
+    x = np.concatenate(xs)
+    v = synth.dyadic(synth.thermal_velocities(len(x), 0.7, 9))
+    with ljmd.Batch(n, box, cutoff=rc, margin=0.5) as b:
+        b.set_state(x, v)
+        pe, _, _ = b.energies()
+        b.set_state(x, v)
+        _, _, f = b.get_state()
+        b.step(0.002, 11, graph_steps=5)
+        bx, _, _ = b.get_state()
+        assert b.stats()["status_word"] == 0
+    o = 0
+    for r, xr in enumerate(xs):
+        sl = slice(o, o + n[r])
+        F, pe_o, _ = O.forces(xr, box[r], O.LJParams(rc_over_sigma=rc))
+        assert np.sqrt(((f[sl] - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-5
+        assert pe[r] == pytest.approx(pe_o, rel=1e-6)
+        with ljmd.System(cutoff=rc, margin=0.5, precision=ljmd.LJ_MIXED) as s:
+            s.set_state(xr, v[sl], box[r])
+            s.step(0.002, 11)
+            sx, _, _, _ = s.get_state()
+        assert np.abs(_min_image(bx[sl] - sx, box[r])).max() < 1e-5
+        o += n[r]
+
+
 TINY = 16  # SM clock cycles: no wait of a kernel is over that fast
 
 
