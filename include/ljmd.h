@@ -435,7 +435,8 @@ int ljmd_batch_get_stats(ljmd_batch* b, ljmd_batch_stats* out);
 int ljmd_batch_set_tuning(ljmd_batch* b, int32_t tile_cells, int32_t lanes);
 
 /*
- * Autotuner: for tile_cells in {2, 3, 4, 6} and lanes in {2, 4, 8}, construct the lists at the
+ * Autotuner: for tile_cells in {2, 3, 4, 6, 10} (10 is the default; those that give the same tiles are tried
+ * once, as the first of them) and lanes in {2, 4, 8}, construct the lists at the
  * current positions and time `trials` force launches and the construction (CUDA events); keep the
  * shape with the least force + construction / 10.  The state is unchanged.  Outputs may be NULL.
  */

@@ -14,6 +14,8 @@
 
 using namespace ljmd;
 
+constexpr int kBatchTile = 10;  // default of ljmd_batch.tile_T
+
 struct ljmd_batch {
   int device = 0;
   cudaStream_t st = nullptr;       // the batch's own stream (capturable)
@@ -38,7 +40,7 @@ struct ljmd_batch {
   // preferred cells per tile along z (replica_tile): 256 replicas of 500 to 50,000 particles at densities 0.3
   // to 0.9, r_s = 2.8, take 1.25, 1.24, 1.06, 0.96, 1.33 ms per force launch at 4, 6, 8, 10, 12 (four threads
   // per key), and 102, 97, 89, 88, 107 ms for 40 steps
-  int tile_T = 10;
+  int tile_T = kBatchTile;
   int tile_cap = kMaxTileT;  // longest tile whose shared memory fitted (host_build)
   int lanes = 4;   // threads per key in the force kernel
   // device state (sorted by cell within each replica)
@@ -837,12 +839,13 @@ int ljmd_batch_time_force(ljmd_batch* b, int32_t trials, double* ms_per_launch) 
 // Project autotuner: for each (tile_cells, lanes) candidate, construct the list at the current
 // positions and time `trials` force launches plus the construction (CUDA events on the batch's
 // stream); the cost is force + construction / 10 (a typical list lifetime).  The fastest is kept.
+// The default length is among the candidates; lengths that give the same tiles are tried once.
 // Positions and velocities are unchanged (constructions only reorder).
 int ljmd_batch_autotune(ljmd_batch* b, int32_t trials, int32_t* best_tile, int32_t* best_lanes, double* best_ms) {
   if (!b || trials <= 0) return LJ_EINVAL;
   if (b->broken) return LJ_EDEVICE;
   if (!b->have_state) return LJ_ESTATE;
-  const int tiles[] = {2, 3, 4, 6};
+  const int tiles[] = {2, 3, 4, 6, kBatchTile};
   const int lanes_c[] = {2, 4, 8};
   cudaEvent_t e0, e1, e2;
   BK(cudaEventCreate(&e0));
@@ -851,7 +854,12 @@ int ljmd_batch_autotune(ljmd_batch* b, int32_t trials, int32_t* best_tile, int32
   double best = 1e300;
   int bt = b->tile_T, bl = b->lanes;
   int rc = LJ_OK;
+  std::vector<std::vector<int>> tried;
   for (int T : tiles) {
+    std::vector<int> shape;
+    for (const ReplicaGeo& rg : b->reps_h) shape.push_back(replica_tile(T, rg.n, rg.count, rg.g.L));
+    if (std::find(tried.begin(), tried.end(), shape) != tried.end()) continue;
+    tried.push_back(shape);
     if ((rc = ljmd_batch_set_tuning(b, T, 0)) != LJ_OK) break;
     if (cudaEventRecord(e0, b->st) != cudaSuccess) {
       rc = LJ_EDEVICE;

@@ -167,3 +167,16 @@ def test_fp64_form_in_any_unit_of_length(sigma, list_form):
             s.set_state(x, None, L)
             hw, _ = s.hvp(w)
         assert np.sqrt(((hw - ref) ** 2).sum(1)).max() / np.sqrt((ref ** 2).sum(1).mean()) <= 1e-10
+
+
+def test_batch_autotuner_knows_the_default():
+    """A batch whose force launch takes 164 us with the tiles of tile_cells = 6 and 130 us with the default's: the
+    autotuner, which keeps the fastest, must not leave it slower than it found it."""
+    x, L = synth.fcc_thinned(20000, 0.3, 5)
+    x = O.wrap(x + synth.displacements(len(x), 0.05, 6), L)
+    with ljmd.Batch([len(x)] * 40, [L] * 40, cutoff=2.5, margin=0.3) as b:
+        b.set_state(np.tile(x, (40, 1)))
+        default = b.time_force(20)
+        tile, lanes, _ = b.autotune(trials=10)
+        assert tile == b.stats()["tile_cells"] == 10
+        assert b.time_force(20) <= 1.1 * default
