@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(NT, kWinCtas)
                uint2* __restrict__ tile_list, uint16_t* __restrict__ ent, uint64_t cap,
                unsigned long long* __restrict__ counter, unsigned int* __restrict__ max_list,
                int32_t* __restrict__ status, const ReplicaGeo* __restrict__ reps, int R,
-               const int* __restrict__ pred, const int32_t* __restrict__ tile_rep) {
+               const int* __restrict__ pred, const int32_t* __restrict__ tile_rep, uint2* __restrict__ desc) {
   static_assert(NT >= 64, "warp 0 prepares the next tile while the others count");
   if (pred && !*pred) return;  // predicated (batched rebuild inside a graph)
   extern __shared__ __align__(16) unsigned char smem[];
@@ -375,8 +375,8 @@ __global__ void __launch_bounds__(NT, kWinCtas)
         if (t + 2 * (int64_t)gridDim.x < ta_in.ntiles) prefetch(t + 2 * (int64_t)gridDim.x);
       }
     };
-    if (warp == kNW - 1)  // the pipelined force kernel's staging descriptor
-      tile_desc_write(ti, ta.n, g.Lq, S, s_ready[buf] != 0, tile_list + ta_in.ntiles + kTileDesc * t, lane);
+    if (desc && warp == kNW - 1)  // the pipelined force kernel's staging descriptor
+      tile_desc_write(ti, ta.n, g.Lq, S, s_ready[buf] != 0, desc + kTileDesc * t, lane);
     if (!s_ready[buf]) {  // sizing inconsistency: record and skip the tile
       if (threadIdx.x == 0) atomicOr(status, LJ_ST_CELL_RANGE);
       if (warp == 0) prepare_next();
@@ -648,8 +648,9 @@ int set_wait_budget(long long cycles) {
 void launch_list_tile(int precision, int half, const void* pos, const float4* hi, const double* x, const uint32_t* cs,
                       int64_t N, Geom g, TileArgs ta, ListBand band, uint2* rows, uint2* tile_list, uint16_t* ent,
                       uint64_t cap, unsigned long long* counter, unsigned int* max_list, int32_t* status,
-                      cudaStream_t s, const int* pred) {
+                      cudaStream_t s, const int* pred, bool descriptors) {
   const size_t sm = list_smem_bytes(ta, precision);
+  uint2* desc = descriptors ? tile_list + ta.ntiles : nullptr;
   int grid = tile_grid(ta, per_sm_for(sm));
   if (!ta.whole) {  // the window kernel: as many CTAs as are resident
     set_smem(k_list_win<false, false, kWinThreads>, sm);
@@ -674,12 +675,12 @@ void launch_list_tile(int precision, int half, const void* pos, const float4* hi
     set_smem(k_list_win<true, false, kWinThreads>, sm);
     k_list_win<true, false, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, ta, band, rows, tile_list, ent,
                                                                        cap, counter, max_list, status, nullptr, 0,
-                                                                       pred, nullptr);
+                                                                       pred, nullptr, desc);
   } else {
     set_smem(k_list_win<false, false, kWinThreads>, sm);
     k_list_win<false, false, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, ta, band, rows, tile_list, ent,
                                                                         cap, counter, max_list, status, nullptr, 0,
-                                                                        pred, nullptr);
+                                                                        pred, nullptr, desc);
   }
 #undef LJ_LIST_LAUNCH
 }
@@ -769,7 +770,7 @@ void launch_list_batch(const float4* hi, const double* x, const uint32_t* cs, in
   const int grid = tile_grid(caps, resident_per_sm(k_list_win<false, true, kWinThreads>, kWinThreads, sm));
   k_list_win<false, true, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, caps, band, rows, tile_list, ent,
                                                                      cap, counter, max_list, status, reps, R, pred,
-                                                                     tile_rep);
+                                                                     tile_rep, tile_list + caps.ntiles);
 }
 
 // ---- list validity: the large displacement check (LDC) of Alg. 2 -----------------------------

@@ -55,8 +55,8 @@ struct ljmd_sys {
   uint32_t *cell_of = nullptr, *perm = nullptr, *perm_id = nullptr;  // perm_id: perm ordered by id in each cell
   uint32_t *cell_count = nullptr, *cell_start = nullptr, *cell_fill = nullptr;
   uint2* rows = nullptr;        // per particle: (start, length) of its row in ent
-  uint2* tile_list = nullptr;   // per tile: (start, length) of its segment of ent; then the staging descriptors
-  int64_t tile_list_cap = 0;
+  uint2* tile_list = nullptr;   // per tile: (start, length) of its segment of ent; then, for the pipelined
+  int64_t tile_list_cap = 0;    // force kernel, the staging descriptors (capacity in 8-byte words)
   uint16_t* ent = nullptr;       // SortedList: partner indices into the key's staged tile
   size_t ent_cap = 0;
   TileArgs ta{};
@@ -464,10 +464,19 @@ static int check_status(ljmd_sys* s) {
 
 static void* force_pos(ljmd_sys* s);
 
+static int force_buffers(const ljmd_sys* s);
+
+// Whether the force over the tiles of s->ta is the pipelined kernel's, which reads staging descriptors.
+static bool wants_descriptors(const ljmd_sys* s) {
+  return s->precision == LJ_MIXED && !s->ta.whole && force_buffers(s) == 2;
+}
+
 static int ensure_tile_list(ljmd_sys* s) {
-  if (s->ta.ntiles > s->tile_list_cap) {
-    TRY(dalloc_t(s, &s->tile_list, kTileWords * (size_t)s->ta.ntiles));
-    s->tile_list_cap = s->ta.ntiles;
+  const int64_t words = (wants_descriptors(s) ? kTileWords : 1) * s->ta.ntiles;
+  if (words > s->tile_list_cap) {
+    s->tile_list_cap = 0;
+    TRY(dalloc_t(s, &s->tile_list, (size_t)words));
+    s->tile_list_cap = words;
   }
   return LJ_OK;
 }
@@ -719,7 +728,7 @@ static int rebuild(ljmd_sys* s) {
       const void* list_pos = s->precision == LJ_MIXED ? (const void*)s->hi : (const void*)s->pos64;
       launch_list_tile(s->precision, half, list_pos, s->hi, s->x, s->cell_start, N, s->g, s->ta, s->band, s->rows,
                        s->tile_list, s->ent, (uint64_t)s->ent_cap, s->d_total64, s->d_sizes + 3, s->d_status, st,
-                       guessed ? &s->d_grid->ok : nullptr);
+                       guessed ? &s->d_grid->ok : nullptr, wants_descriptors(s));
       s->launches += 1;
       CKL();
       const GridCtl* hg = s->h_grid;

@@ -207,7 +207,8 @@ struct ReplicaGeo {
   int64_t cell_base;       // first global cell
   int64_t base, count;     // first global particle, particles
 };
-constexpr int kTileWords = 25;  // 8-byte words of tile_list per tile: its list segment and its staging descriptor
+constexpr int kTileWords = 25;  // 8-byte words of tile_list per tile: its list segment and its staging descriptor,
+                                // which only the pipelined force kernel reads (200 B: 54 GB at 1,024 cells per side)
 size_t list_smem_bytes(const TileArgs& ta, int precision);
 size_t force_smem_bytes(const TileArgs& ta, int precision, int nbuf, int half);
 void launch_max_count(const uint32_t* cnt, int64_t n, unsigned int* out, cudaStream_t s);
@@ -216,7 +217,7 @@ void launch_tile_sizes(const uint32_t* cs, TileArgs ta, unsigned int* out, cudaS
 void launch_list_tile(int precision, int half, const void* pos, const float4* hi, const double* x, const uint32_t* cs,
                       int64_t N, Geom g, TileArgs ta, ListBand band, uint2* rows, uint2* tile_list, uint16_t* ent,
                       uint64_t cap, unsigned long long* counter, unsigned int* max_list, int32_t* status,
-                      cudaStream_t s, const int* pred = nullptr);
+                      cudaStream_t s, const int* pred, bool descriptors);
 // pos: the fixed-point records (mixed) or the dvec4 copies (FP64).  Returns the number of blocks
 // (energy partials written to part[2 b], part[2 b + 1]).
 int launch_force_tile(int precision, int half, int lanes, int energy, const void* pos, const uint32_t* cs, int64_t N,

@@ -180,3 +180,19 @@ def test_batch_autotuner_knows_the_default():
         tile, lanes, _ = b.autotune(trials=10)
         assert tile == b.stats()["tile_cells"] == 10
         assert b.time_force(20) <= 1.1 * default
+
+
+def test_dilute_fp64_box_holds_no_staging_descriptors():
+    """256 cells per side, 4.2 million tiles: 8 bytes a tile for its list segment (34 MB) beside three words a cell
+    (201 MB).  The 192 bytes a tile that only the mixed form's pipelined kernel reads would add 805 MB."""
+    torch = pytest.importorskip("torch")
+    x = synth.uniform_positions(1000, 769.0, 3)
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_FP64) as s:
+        s.set_state(x, None, 769.0)
+        torch.cuda.synchronize()
+        free0, _ = torch.cuda.mem_get_info()
+        s.build_pairlist()
+        free1, _ = torch.cuda.mem_get_info()
+        assert s.stats()["cells_per_side"] == 256
+        assert free0 - free1 < 300e6
+        assert np.array_equal(s.pairs(), O.pairs_within(x, 769.0, 3.0))
