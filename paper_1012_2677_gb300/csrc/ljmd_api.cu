@@ -667,7 +667,6 @@ static int read_grid(ljmd_sys* s, bool sorted) {
   if (!sorted || (int64_t)s->h_grid->ticket == sort_grid(s->n)) return LJ_OK;
   swap_state(s);
   s->sort_dirty = true;
-  s->have_list = s->forces_current = false;
   return LJ_EDEVICE;
 }
 
@@ -677,6 +676,7 @@ static int rebuild(ljmd_sys* s) {
   ljmd_sys* sys = s;
   const int64_t N = s->n;
   cudaStream_t st = s->st;
+  s->have_list = s->forces_current = false;  // whatever happens on the way: the order and the tiles change
   TRY(ensure_cells(s));
   PhaseTimer timer(s, PH_REBUILD);
   bool sorted = false, guessed = false;  // guessed: s->ta holds the capacities that k_sort checks

@@ -196,3 +196,24 @@ def test_dilute_fp64_box_holds_no_staging_descriptors():
         assert s.stats()["cells_per_side"] == 256
         assert free0 - free1 < 300e6
         assert np.array_equal(s.pairs(), O.pairs_within(x, 769.0, 3.0))
+
+
+def test_a_refused_list_leaves_no_list_behind():
+    """A cutoff whose cells are beyond what a tile can stage (16,384 particles in 27 cells) is refused; the
+    particles are in the new cells' order by then, so the former list is gone: forces are refused too until a
+    list can be built again."""
+    x, L = O.fcc_lattice(16, 1.0)
+    x = synth.dyadic(O.wrap(x + synth.displacements(len(x), 0.03, 6), L))
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_MIXED) as s:
+        s.set_state(x, None, L)
+        s.compute_forces()
+        for call in (lambda: s.build_pairlist(7.5, 0.5), s.compute_forces, lambda: s.step(0.001, 1)):
+            with pytest.raises(ljmd.LjmdError) as e:
+                call()
+            assert e.value.code == ljmd.LJ_ERANGE
+        s.build_pairlist(2.5, 0.5)
+        s.compute_forces()
+        gx, _, f, _ = s.get_state()
+        assert np.array_equal(gx, x) and s.stats()["status_word"] == 0
+    F, _, _ = O.forces(x, L)
+    assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-5
