@@ -71,7 +71,7 @@ bool dp_fits(const TileArgs& ta) {
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   TileArgs tz = ta;
   tz.list_cap = 0;
-  return dp_layout<3, false>(tz).total + 2048 <= (size_t)smem_max;  // 2 KB: static shared memory
+  return dp_layout<3, false>(tz).total + kStaticSmem <= (size_t)smem_max;
 }
 
 // The FP64 form on tiles; returns the grid launched.

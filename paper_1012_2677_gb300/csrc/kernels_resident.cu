@@ -522,7 +522,7 @@ static bool resident_fits(const TileArgs& ta) {
   int dev = 0, smem_max = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (sm + 2816 > (size_t)smem_max) return false;
+  if (sm + kStaticSmem > (size_t)smem_max) return false;
   set_smem(k_resident<MIXED, HALF, LANES>, sm);
   return ta.ntiles <=
          (int64_t)sm_count() * resident_per_sm(k_resident<MIXED, HALF, LANES>, MIXED ? kResThreads : kDpThreads, sm);

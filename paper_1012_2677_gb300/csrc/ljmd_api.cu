@@ -468,7 +468,7 @@ static int force_buffers(const ljmd_sys* s);
 
 // Whether the force over the tiles of s->ta is the pipelined kernel's, which reads staging descriptors.
 static bool wants_descriptors(const ljmd_sys* s) {
-  return s->precision == LJ_MIXED && !s->ta.whole && force_buffers(s) == 2;
+  return !s->ta.whole && force_buffers(s) == 2;
 }
 
 static int ensure_tile_list(ljmd_sys* s) {
@@ -497,11 +497,12 @@ static int sm_count_of(int dev) {
 }
 
 static int force_buffers(const ljmd_sys* s) {
+  if (s->precision != LJ_MIXED) return 1;
   if (s->force_nbuf) return s->force_nbuf;
   // fewer tiles than two per SM: the single-buffer kernel (the pipelined one holds one CTA per SM
   // with two producer warps)
   if (s->ta.ntiles > 0 && s->ta.ntiles < 2 * (int64_t)sm_count_of(s->device)) return 1;
-  return s->precision == LJ_MIXED ? 2 : 1;
+  return 2;
 }
 
 // Default cells per tile along z.  The mixed form with the full list (the pipelined force kernel):
@@ -773,7 +774,7 @@ static int rebuild(ljmd_sys* s) {
     const int nbuf = s->ta.whole ? 1 : force_buffers(s);
     // static shared memory (bookkeeping of two staged tiles, 1.2 KB each, or of four in the pipelined
     // kernel) comes out of the same limit
-    const int64_t smem_dyn = (int64_t)smem_max - (nbuf == 2 ? 5376 : 2816);
+    const int64_t smem_dyn = (int64_t)smem_max - (nbuf == 2 ? 5376 : kStaticSmem);
     if ((int64_t)base_bytes <= smem_dyn) {
       const int64_t room = (smem_dyn - (int64_t)base_bytes) / (2 * nbuf) - 16;
       s->ta.list_cap = (int32_t)std::max<int64_t>(0, std::min<int64_t>(s->ta.max_list, room) & ~(int64_t)7);

@@ -209,6 +209,9 @@ struct ReplicaGeo {
 };
 constexpr int kTileWords = 25;  // 8-byte words of tile_list per tile: its list segment and its staging descriptor,
                                 // which only the pipelined force kernel reads (200 B: 54 GB at 1,024 cells per side)
+// Static shared memory of the kernels that stage one tile, at most (their bookkeeping and final sums), out of
+// the same limit as the tile.
+constexpr int kStaticSmem = 2816;
 size_t list_smem_bytes(const TileArgs& ta, int precision);
 size_t force_smem_bytes(const TileArgs& ta, int precision, int nbuf, int half);
 void launch_max_count(const uint32_t* cnt, int64_t n, unsigned int* out, cudaStream_t s);

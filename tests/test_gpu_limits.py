@@ -217,3 +217,17 @@ def test_a_refused_list_leaves_no_list_behind():
         assert np.array_equal(gx, x) and s.stats()["status_word"] == 0
     F, _, _ = O.forces(x, L)
     assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-5
+
+
+def test_fp64_tiles_around_the_queue_kernels_capacity():
+    """27 cells, each tile stages the whole box: from about 4,520 particles on the queue kernel's tile does not fit
+    beside its static shared memory, and the general kernel takes over without a gap."""
+    for N in range(4492, 4557, 4):
+        x, L = _liquid(N, 0.9, 11)
+        with ljmd.System(cutoff=5.0, margin=0.5, precision=ljmd.LJ_FP64, list_form=ljmd.LJ_LIST_FULL) as s:
+            s.set_state(synth.dyadic(x), None, L)
+            s.compute_forces()
+            assert s.stats()["cells_per_side"] == 3
+            _, _, f, _ = s.get_state()
+        F, _, _ = O.forces(synth.dyadic(x), L, O.LJParams(rc_over_sigma=5.0))
+        assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-11, N
