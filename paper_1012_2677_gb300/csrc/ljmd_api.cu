@@ -14,6 +14,9 @@
 
 using namespace ljmd;
 
+// The block that d_grid points to: counters, cell counts of k_sort, control block of a resident run.
+constexpr size_t kGridBytes = sizeof(GridCtl) + sizeof(uint32_t) * kSortCells;
+
 struct ljmd_sys {
   int device = 0;
   cudaStream_t st = nullptr;
@@ -68,6 +71,7 @@ struct ljmd_sys {
   size_t scan_tmp_cap = 0;
   int64_t cap_n = 0;       // particle capacity of the per-particle buffers
   int64_t cap_cells = 0;   // capacity of the per-cell buffers
+  double *part_mem = nullptr;  // holds part_force and part_force2, which a resident run exchanges
   double *part_force = nullptr, *part_ke = nullptr, *part_misc = nullptr, *d_scalars = nullptr;
   double* d_energies = nullptr;
   int64_t* d_log_count = nullptr;
@@ -80,8 +84,8 @@ struct ljmd_sys {
   double* cap_x = nullptr;
   int64_t cap_step0 = 0;
   StepCtl* h_ctl = nullptr;     // pinned mirror
-  // resident runs (allocated on first use): threads per key (0: the tiles do not fit at once), control
-  // block and its pinned mirror, second position buffer, energy partials of a run's states
+  // resident runs: threads per key (0: the tiles do not fit at once), control block and its pinned mirror,
+  // energy partials of the last state and of a run's states (only these are allocated on first use)
   int res_lanes = 0;
   TileArgs res_ta{};
   ResidentCtl *d_res = nullptr, *h_res = nullptr;
@@ -90,8 +94,6 @@ struct ljmd_sys {
   uint32_t* sort_count = nullptr;   // cell counts of k_sort, behind d_grid: zero between launches
   void* h_pin = nullptr;            // the pinned block that holds all h_ arrays
   bool sort_dirty = false;          // a launch may have left counts behind
-  void* pos_alt = nullptr;
-  int64_t pos_alt_cap = 0;
   double *res_rec = nullptr, *part_force2 = nullptr;
   int64_t res_rec_cap = 0;
   int64_t last_build_step = 0;  // sys->steps at the last list construction
@@ -165,10 +167,10 @@ static int dalloc_t(ljmd_sys* sys, T** p, size_t count) {
 static void free_all(ljmd_sys* s) {
   void* ptrs[] = {s->x, s->v, s->x_alt, s->v_alt, s->f, s->f_alt, s->hi, s->xq, s->pos64, s->ref, s->id,
                   s->id_alt, s->img, s->img_alt, s->cell_of, s->perm, s->perm_id, s->cell_count, s->cell_start,
-                  s->cell_fill, s->rows, s->tile_list, s->ent, s->scan_tmp, s->part_force, s->part_ke,
+                  s->cell_fill, s->rows, s->tile_list, s->ent, s->scan_tmp, s->part_mem, s->part_ke,
                   s->part_misc, s->d_scalars, s->d_energies, s->d_log_count, s->d_grid, s->d_dmax, s->d_ctl, s->d_ticket,
                   s->adj_w, s->adj_hw, s->adj_f, s->adj_wf, s->adj_ticket, s->part_adj, s->d_adj, s->xref64, s->ldc_list, s->d_ldc,
-                  s->d_res, s->pos_alt, s->res_rec, s->part_force2};
+                  s->res_rec};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto& p : s->ev_pending) {
@@ -1039,34 +1041,33 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
   return LJ_OK;
 }
 
-static int ensure_resident(ljmd_sys* s) {
-  const size_t psz = s->precision == LJ_MIXED ? 16 : 32;
-  if (!s->d_res) TRY(dalloc_t(s, &s->d_res, 1));
-  if (!s->part_force2) TRY(dalloc_t(s, &s->part_force2, 2 * kMaxRedBlocks));
-  if (s->pos_alt_cap < s->cap_n) {
-    s->pos_alt_cap = 0;
-    TRY(dalloc(s, &s->pos_alt, psz * (size_t)s->cap_n));
-    s->pos_alt_cap = s->cap_n;
-  }
-  const int64_t want = 3 * (int64_t)(kResidentSteps + 1) * s->ta.ntiles;
+// Energy partials for a run of K steps, no more: allocating a megabyte takes 30 us, and the first step of 4,000
+// particles on a new handle, list construction included, 100.  False: no memory.
+static bool ensure_records(ljmd_sys* s, int K) {
+  if (s->prm.energy_every <= 0) return true;
+  int64_t slots = 2;
+  while (slots < K + 1) slots *= 2;
+  const int64_t want = 3 * slots * s->ta.ntiles;
   if (s->res_rec_cap < want) {
-    TRY(dalloc_t(s, &s->res_rec, (size_t)want));
+    s->res_rec_cap = 0;
+    if (dalloc_t(s, &s->res_rec, (size_t)want) != LJ_OK) return false;
     s->res_rec_cap = want;
   }
-  return LJ_OK;
+  return true;
 }
 
 // Up to `remaining` steps as one resident run (kernels_resident.cu), with the final half kick of the
 // call if it gets to its end (*finished).  *advanced and *stopped as device_run; *launched = false: the
-// device cannot hold the grid now and nothing was done.
+// device cannot hold the grid now, or has no room for the energy partials, and nothing was done.
 static int resident_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remaining, int64_t* advanced,
                         bool* stopped, bool* finished, bool* launched) {
   ljmd_sys* sys = s;
   cudaStream_t st = s->st;
-  TRY(ensure_resident(s));
   const int ee = s->prm.energy_every;
   auto want_energy = [&](int64_t t) { return ee > 0 && (t % ee) == 0; };
   const int K = (int)std::min<int64_t>(remaining, kResidentSteps);
+  *launched = false;
+  if (!ensure_records(s, K)) return LJ_OK;
   ResidentCtl* hc = s->h_res;
   const size_t head = offsetof(ResidentCtl, dmax);
   memset(hc, 0, head + sizeof(hc->dmax[0]) * (size_t)K);
@@ -1085,7 +1086,7 @@ static int resident_run(ljmd_sys* s, double dt, bool first_of_call, int64_t rema
   a.v = s->v;
   a.f = s->f;
   a.pos = force_pos(s);
-  a.pos_alt = s->pos_alt;
+  a.pos_alt = s->f_alt;  // of the same size, and free between list constructions
   a.ref = s->ref;
   a.id = s->id;
   a.img = s->img;
@@ -1181,18 +1182,21 @@ int ljmd_create(ljmd_sys** out, const ljmd_params* p, int32_t precision, void* c
     return LJ_EDEVICE;
   }
   int r = LJ_OK;
-  if (r == LJ_OK) r = dalloc_t(sys, &sys->part_force, 2 * kMaxRedBlocks);
+  if (r == LJ_OK) r = dalloc_t(sys, &sys->part_mem, 4 * kMaxRedBlocks);
+  sys->part_force = sys->part_mem;
+  sys->part_force2 = sys->part_mem ? sys->part_mem + 2 * kMaxRedBlocks : nullptr;
   if (r == LJ_OK) r = dalloc_t(sys, &sys->part_ke, kMaxRedBlocks);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->part_misc, 4 * kMaxRedBlocks);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_scalars, 8);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_energies, 4);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_log_count, 1);
-  if (r == LJ_OK) r = dalloc(sys, (void**)&sys->d_grid, sizeof(GridCtl) + sizeof(uint32_t) * kSortCells);
+  if (r == LJ_OK) r = dalloc(sys, (void**)&sys->d_grid, kGridBytes + sizeof(ResidentCtl));
   if (r == LJ_OK) {
     sys->d_status = &sys->d_grid->status;
     sys->d_total64 = sys->d_grid->total;
     sys->d_sizes = sys->d_grid->sizes;
     sys->sort_count = (uint32_t*)(sys->d_grid + 1);
+    sys->d_res = (ResidentCtl*)((unsigned char*)sys->d_grid + kGridBytes);
   }
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_dmax, 2);
   if (r == LJ_OK) r = dalloc_t(sys, &sys->d_ctl, 1);
@@ -1213,7 +1217,7 @@ int ljmd_create(ljmd_sys** out, const ljmd_params* p, int32_t precision, void* c
     sys->h_res = (ResidentCtl*)(h + 320);
   }
   if (r == LJ_OK &&
-      cudaMemsetAsync(sys->d_grid, 0, sizeof(GridCtl) + sizeof(uint32_t) * kSortCells, sys->st) != cudaSuccess)
+      cudaMemsetAsync(sys->d_grid, 0, kGridBytes, sys->st) != cudaSuccess)
     r = LJ_EDEVICE;
   if (r == LJ_OK && cudaMemsetAsync(sys->d_log_count, 0, 8, sys->st) != cudaSuccess) r = LJ_EDEVICE;
   if (r != LJ_OK) {

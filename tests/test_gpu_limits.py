@@ -231,3 +231,18 @@ def test_fp64_tiles_around_the_queue_kernels_capacity():
             _, _, f, _ = s.get_state()
         F, _, _ = O.forces(synth.dyadic(x), L, O.LJParams(rc_over_sigma=5.0))
         assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-11, N
+
+
+def test_first_step_of_a_resident_box_allocates_nothing():
+    """Beyond the list construction, which comes before: 32,000 particles, no energies asked for."""
+    torch = pytest.importorskip("torch")
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_MIXED, list_form=ljmd.LJ_LIST_FULL, energy_every=0) as s:
+        s.init_lattice(20, 0.5, 1.0, 1)
+        s.build_pairlist()
+        torch.cuda.synchronize()
+        free0, _ = torch.cuda.mem_get_info()
+        n0 = s.stats()["kernel_launches"]
+        s.step(0.001, 3)
+        free1, _ = torch.cuda.mem_get_info()
+        assert s.stats()["kernel_launches"] - n0 == 1  # one resident run
+        assert free1 == free0
