@@ -246,3 +246,64 @@ def test_first_step_of_a_resident_box_allocates_nothing():
         free1, _ = torch.cuda.mem_get_info()
         assert s.stats()["kernel_launches"] - n0 == 1  # one resident run
         assert free1 == free0
+
+
+def _gives_up(s, call):
+    """call with the short budget ends with LJ_EDEVICE or, where it does not look at the status itself, leaves it."""
+    ljmd.ljmd_set_wait_budget(TINY)
+    try:
+        try:
+            call()
+        except ljmd.LjmdError as e:
+            assert e.code == ljmd.LJ_EDEVICE
+    finally:
+        ljmd.ljmd_set_wait_budget(0)
+    assert s.stats()["status_word"] == ljmd.LJ_ST_TIMEOUT
+
+
+def _device_still_usable():
+    x, L = _liquid(2000, 0.6, 5)
+    x = synth.dyadic(x)
+    F, _, _ = O.forces(x, L)
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_FP64) as s:
+        s.set_state(x, None, L)
+        s.step(0.0, 1)
+        _, _, f, _ = s.get_state()
+        assert s.stats()["status_word"] == 0
+    assert np.sqrt(((f - F) ** 2).sum(1)).max() / np.sqrt((F ** 2).sum(1).mean()) <= 1e-11
+
+
+@pytest.mark.parametrize("list_form", [ljmd.LJ_LIST_FULL, ljmd.LJ_LIST_HALF])
+def test_list_kernel_wait_times_out(list_form):
+    """8,000 cells: more than the one-launch reordering takes, so nothing gives up before the list kernel."""
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_MIXED, list_form=list_form) as s:
+        s.init_lattice(30, 0.5, 1.0, 1)
+        _gives_up(s, s.build_pairlist)
+        assert s.stats()["cells_per_side"] == 20 and s.stats()["kernel_launches"] > 2
+    _device_still_usable()
+
+
+@pytest.mark.parametrize("list_form", [ljmd.LJ_LIST_FULL, ljmd.LJ_LIST_HALF])
+@pytest.mark.parametrize("precision", [ljmd.LJ_MIXED, ljmd.LJ_FP64])
+def test_grid_barrier_of_a_resident_run_times_out(precision, list_form):
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=precision, list_form=list_form, energy_every=1) as s:
+        s.init_lattice(10, 0.5, 1.0, 1)
+        s.build_pairlist()
+        n0 = s.stats()["kernel_launches"]
+        _gives_up(s, lambda: s.step(0.005, 5))
+        assert s.stats()["kernel_launches"] - n0 == 1
+        with pytest.raises(ljmd.LjmdError):  # the run's state is not to be had
+            s.step(0.005, 1)
+    _device_still_usable()
+
+
+def test_waits_of_the_fp64_queue_kernels_time_out():
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_FP64) as s:
+        s.init_lattice(20, 0.5, 1.0, 1)
+        s.build_pairlist()
+        _gives_up(s, s.compute_forces)
+    with ljmd.System(cutoff=2.5, margin=0.5, precision=ljmd.LJ_FP64, list_form=ljmd.LJ_LIST_FULL) as s:
+        s.init_lattice(10, 0.5, 1.0, 1)
+        s.build_pairlist()
+        _gives_up(s, lambda: s.hvp(np.ones((4000, 3))))
+    _device_still_usable()
