@@ -10,7 +10,7 @@ template <bool MIXED, bool HALF, bool WHOLE, bool LONGLIST, int LANES, bool ENER
 static void force_tile_launch(const ForceLaunch& a) {
   set_smem(k_force_tile<MIXED, LANES, HALF, ENERGY, WHOLE, LONGLIST>, a.smem);
   k_force_tile<MIXED, LANES, HALF, ENERGY, WHOLE, LONGLIST><<<a.grid, kTileThreads, a.smem, a.s>>>(
-      a.pos, a.cs, a.N, a.g, a.ta, a.c, a.rows, a.tile_list, a.ent, a.f, a.part, a.status, a.nbuf, a.skip);
+      a.pos, a.cs, a.N, a.g, a.ta, a.c, a.rows, a.tile_list, a.ent, a.f, a.part, a.status, a.skip);
 }
 
 template <bool MIXED, bool HALF, bool WHOLE, bool LONGLIST, int LANES>

@@ -326,8 +326,8 @@ __global__ void __launch_bounds__(kDpThreads, 3)
     if (force_tile_prepare(ti, t, ta, cs, tile_list, S, status)) {
       stage_issue<false, true>(ti, ta, pos, rows, ent, S, smem, D.L, &bar);
       if (!dp_stage_finish(ti, ta, g, S, smem, D, &bar, ph, status)) return;
-      queue_tile_pairs<double, NACC, false, kDpWarps>(
-          S, sq, (const uint2*)(smem + D.L.rows), ((DpWarp<double, NACC, false>*)(smem + D.warp))[threadIdx.x >> 5],
+      queue_tile_pairs<NACC, false>(
+          S, sq, (const uint2*)(smem + D.L.rows), ((DpWarp<NACC, false>*)(smem + D.warp))[threadIdx.x >> 5],
           (const uint16_t*)(smem + D.L.ent), ent + S.list_base, (unsigned)ta.list_cap, c.rc2w, status,
           [&](int o) { return Key{sp[S.own0 + o], w[S.gown0 + o]}; }, [&](int j) { return Key{sp[j], w[sq[j].w]}; },
           [&](const Key& k, const Key& j, double* acc) {
@@ -360,8 +360,7 @@ __global__ void __launch_bounds__(kDpThreads, 3)
           [&](int o, const double* a) {
             adjoint_row(out, S.gown0 + o, a[0], a[1], a[2], FO ? a[NACC - 3] : 0.0, FO ? a[NACC - 2] : 0.0,
                         FO ? a[NACC - 1] : 0.0);
-          },
-          [] {});
+          });
       npairs += (double)np;
       np = 0;
     }

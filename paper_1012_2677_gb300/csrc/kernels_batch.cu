@@ -66,11 +66,9 @@ void launch_rebuild_flag(const uint32_t* dmax_bits, float limit2, int* flag, lon
   k_rebuild_flag<<<1, 1, 0, s>>>(dmax_bits, limit2, flag, rebuilds);
 }
 
-// Predicated copy of `bytes` (a multiple of 4) from in to out: 16-byte words while both
+// Copy of `bytes` (a multiple of 4) from in to out: 16-byte words while both
 // addresses are 16-byte aligned (the device allocations are), then the 4-byte tail.
-__global__ void k_copy_words(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n,
-                             const int* __restrict__ pred) {
-  if (pred && !*pred) return;
+__global__ void k_copy_words(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, int64_t n) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t n16 = 0;
   if ((((uintptr_t)in | (uintptr_t)out) & 15u) == 0) {
@@ -81,9 +79,9 @@ __global__ void k_copy_words(const uint32_t* __restrict__ in, uint32_t* __restri
   }
   for (int64_t i = 4 * n16 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) out[i] = in[i];
 }
-void launch_copy_words(const void* in, void* out, int64_t bytes, const int* pred, cudaStream_t s) {
+void launch_copy_words(const void* in, void* out, int64_t bytes, cudaStream_t s) {
   const int64_t n = bytes / 4;
-  k_copy_words<<<grid_of((n + 3) / 4, pred), 256, 0, s>>>((const uint32_t*)in, (uint32_t*)out, n, pred);
+  k_copy_words<<<grid_of((n + 3) / 4), 256, 0, s>>>((const uint32_t*)in, (uint32_t*)out, n);
 }
 
 // Predicated zero fill of up to four arrays of 4-byte words, in one launch.

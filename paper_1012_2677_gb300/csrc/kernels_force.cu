@@ -4,8 +4,8 @@
 
 namespace ljmd {
 
-// Shared memory of the force kernel: `nbuf` tile buffers (with two, the next tile's copies are in
-// flight while the current one is computed); one for the whole-box case.
+// Shared memory of the force kernel: `nbuf` tile buffers (two: the least that the pipelined kernel takes); one
+// for the whole-box case.
 size_t force_buffer_bytes(const TileArgs& ta, int precision, int half) {
   const bool mixed = precision == LJ_MIXED;
   return align16(tile_layout(ta, mixed, true, !mixed && (half || ta.whole)).total);
@@ -93,14 +93,11 @@ int launch_force_tile(int precision, int half, int lanes, int energy, const void
                       Geom g, TileArgs ta, LJConst c, const uint2* rows, const uint2* tile_list, const uint16_t* ent,
                       void* f, double* part, int32_t* status, int per_sm, int nbuf, cudaStream_t s, const int* skip,
                       bool overlap) {
-  ForceLaunch a{pos, cs, N, g, ta, c, rows, tile_list, ent, f, part, status, skip, lanes, energy, per_sm, nbuf, 0, 0, s};
+  ForceLaunch a{pos, cs, N, g, ta, c, rows, tile_list, ent, f, part, status, skip, lanes, energy, per_sm, 1, 0, 0, s};
   a.overlap = overlap ? 1 : 0;
-  a.smem = force_smem_bytes(ta, precision, nbuf, half);
+  a.smem = force_smem_bytes(ta, precision, 1, half);
   a.grid = tile_grid(ta, per_sm > 0 ? per_sm : per_sm_for(a.smem));
-  if (precision != LJ_MIXED) {
-    if (!ta.whole) a.nbuf = 1;
-    return launch_force_fp64(half, a);
-  }
+  if (precision != LJ_MIXED) return launch_force_fp64(half, a);
   if (!ta.whole && nbuf == 2 && (a.nbuf = pipe_plan(a.ta)) > 0) {
     if (half) {
       const int grid = launch_force_pipe_half(a);
@@ -117,8 +114,6 @@ int launch_force_tile(int precision, int half, int lanes, int energy, const void
     }
   }
   a.ta = ta;
-  a.nbuf = 1;
-  a.smem = force_smem_bytes(ta, precision, 1, half);
   if (half) launch_force_mixed_half(a);
   else force_tile_mixed<false>(a);
   return a.grid;

@@ -269,9 +269,7 @@ int launch_integrate(int precision, double* x, double* v, const void* f, void* p
 // forms); for the mixed form the fixed-point records, for FP64 the dvec4 copy; and the
 // displacement reference (the records for mixed, the dvec4 for FP64) if ref != NULL.
 __global__ void k_shadow(const double* __restrict__ x, int64_t N, int mixed, int qk, float4* __restrict__ hi,
-                         uint4* __restrict__ xq, dvec4* __restrict__ pos64, void* __restrict__ ref,
-                         const int* __restrict__ pred) {
-  if (pred && !*pred) return;
+                         uint4* __restrict__ xq, dvec4* __restrict__ pos64, void* __restrict__ ref) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
     const double a = x[i], b = x[N + i], c = x[2 * N + i];
     float4 h;
@@ -293,8 +291,8 @@ __global__ void k_shadow(const double* __restrict__ x, int64_t N, int mixed, int
 }
 
 void launch_shadow_all(const double* x, int64_t N, int mixed, int qk, float4* hi, uint4* xq, dvec4* pos64, void* ref,
-                       cudaStream_t s, const int* pred) {
-  k_shadow<<<stride_grid(N, 256, pred), 256, 0, s>>>(x, N, mixed, qk, hi, xq, pos64, ref, pred);
+                       cudaStream_t s) {
+  k_shadow<<<stride_grid(N, 256, nullptr), 256, 0, s>>>(x, N, mixed, qk, hi, xq, pos64, ref);
 }
 
 }  // namespace ljmd

@@ -800,7 +800,7 @@ static int rebuild(ljmd_sys* s) {
       TRY(dalloc_t(s, &s->xref64, 3 * (size_t)s->n));
       s->xref_cap = s->n;
     }
-    launch_copy_words(s->x, s->xref64, 24 * s->n, nullptr, s->st);
+    launch_copy_words(s->x, s->xref64, 24 * s->n, s->st);
     s->launches += 1;
   }
   s->pe_step = -1;

@@ -115,7 +115,7 @@ void launch_load_state(const double* x_in, const double* v_in, double* x, double
 // records xq (X, Y, Z at u = 2^-qk, w = sorted index); fp64: the dvec4 copy.  ref (optional)
 // receives xq (mixed) or the dvec4 (fp64) as the displacement reference.
 void launch_shadow_all(const double* x, int64_t N, int mixed, int qk, float4* hi, uint4* xq, dvec4* pos64, void* ref,
-                       cudaStream_t s, const int* pred = nullptr);
+                       cudaStream_t s);
 
 // A launch that may start while the one before it in the stream ends (its kernel calls
 // wait_for_previous_launch first).
@@ -430,7 +430,7 @@ void launch_wrap_label_batch(double* x, int32_t* img, int64_t N, const int32_t* 
                              double offset, uint32_t* cell_of, uint32_t* cell_count, int32_t* status,
                              const int* pred, cudaStream_t s);
 void launch_rebuild_flag(const uint32_t* dmax_bits, float limit2, int* flag, long long* rebuilds, cudaStream_t s);
-void launch_copy_words(const void* in, void* out, int64_t bytes, const int* pred, cudaStream_t s);
+void launch_copy_words(const void* in, void* out, int64_t bytes, cudaStream_t s);
 struct ZeroArgs {
   uint32_t* out[4];
   int64_t words[4];

@@ -271,17 +271,16 @@ __host__ __device__ __forceinline__ TileLayout tile_layout(const TileArgs& ta, b
   return L;
 }
 
-// Issue the bulk copies of one tile (warp `issuer`; lane k < 9 handles column k, lane 9 the rows
+// Issue the bulk copies of one tile (warp 0; lane k < 9 handles column k, lane 9 the rows
 // and list segment), all completing on `bar`.  Copies: positions (fixed-point records, hi or FP64), and for the
 // force kernel the own rows and the list segment.  No barrier inside: the other warps go on.
 template <bool MIXED, bool FORCE>
 __device__ __forceinline__ void stage_issue(const TileInfo& ti, const TileArgs& ta, const void* __restrict__ pos,
                                             const uint2* __restrict__ rows, const uint16_t* __restrict__ ent,
-                                            TileShared& S, unsigned char* smem, const TileLayout& L, uint64_t* bar,
-                                            int issuer = 0) {
+                                            TileShared& S, unsigned char* smem, const TileLayout& L, uint64_t* bar) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned bpp = MIXED ? 16u : 32u;
-  if (warp != issuer) return;
+  if (warp != 0) return;
   unsigned bytes = (unsigned)S.total * bpp;
   int r0 = 0, r1 = 0;
   const int n_own = S.own1 - S.own0;
@@ -780,77 +779,44 @@ __device__ __forceinline__ bool force_tile_prepare(const TileInfo& ti, int64_t t
   return true;
 }
 
-// Force over the list, tile by tile.  With nbuf = 2 each CTA walks its tiles with two
-// shared-memory buffers: the copies of tile t + gridDim.x are issued before tile t is computed,
-// so the copy latency overlaps the pair arithmetic; with nbuf = 1 the tiles are staged one after
-// the other and the overlap comes from the other CTAs of the SM.  Energies: per-thread FP64
-// sums -> one partial per block.
+// Force over the list, tile by tile: a tile's copies overlap the arithmetic of the SM's other CTAs.
+// Energies: per-thread FP64 sums -> one partial per block.
 template <bool MIXED, int LANES, bool HALF, bool ENERGY, bool WHOLE, bool LONGLIST>
 __global__ void __launch_bounds__(kTileThreads, 4)
     k_force_tile(const void* __restrict__ pos, const uint32_t* __restrict__ cs, int64_t N, Geom g, TileArgs ta,
                  LJConst c, const uint2* __restrict__ rows, const uint2* __restrict__ tile_list,
                  const uint16_t* __restrict__ ent, void* __restrict__ fout, double* __restrict__ part,
-                 int32_t* __restrict__ status, int nbuf, const int* __restrict__ skip) {
+                 int32_t* __restrict__ status, const int* __restrict__ skip) {
   if (skip && *skip) return;  // a device-decided run stopped before this step
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ TileShared SS[2];
-  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ TileShared S;
+  __shared__ __align__(8) uint64_t bar;
   const TileLayout L = tile_layout(ta, MIXED, true, !MIXED && (HALF || WHOLE));
-  const size_t buf_bytes = align16(L.total);
   EAcc eacc;
   eacc.vscale = g.qu;
   if (WHOLE) {
     if (blockIdx.x == 0) {
-      stage_whole<MIXED, !MIXED>(N, pos, SS[0], smem, L);
+      stage_whole<MIXED, !MIXED>(N, pos, S, smem, L);
       __syncthreads();
-      force_tile_compute<MIXED, LANES, HALF, ENERGY, true, false>(SS[0], smem, L, rows, ent, c, g, fout, status, eacc,
+      force_tile_compute<MIXED, LANES, HALF, ENERGY, true, false>(S, smem, L, rows, ent, c, g, fout, status, eacc,
                                                                   ta.list_cap);
     }
   } else {
-    const bool pipelined = nbuf == 2;
     if (threadIdx.x == 0) {
-      mbar_init(&bars[0], 1);
-      mbar_init(&bars[1], 1);
+      mbar_init(&bar, 1);
       fence_proxy_async_smem();
     }
     __syncthreads();
-    uint32_t ph0 = 0, ph1 = 0;
-    int64_t t = blockIdx.x;
-    int b = 0;
-    bool v_cur = false, v_next = false;
-    if (pipelined && t < ta.ntiles) {
-      v_cur = force_tile_prepare(tile_info(t, ta), t, ta, cs, tile_list, SS[0], status);
-      if (v_cur) stage_issue<MIXED, true>(tile_info(t, ta), ta, pos, rows, ent, SS[0], smem, L, &bars[0]);
-    }
-    for (; t < ta.ntiles; t += gridDim.x) {
-      if (!pipelined) {
-        v_cur = force_tile_prepare(tile_info(t, ta), t, ta, cs, tile_list, SS[0], status);
-        if (v_cur) stage_issue<MIXED, true>(tile_info(t, ta), ta, pos, rows, ent, SS[0], smem, L, &bars[0]);
-      } else {
-        const int64_t tn = t + gridDim.x;
-        v_next = false;
-        if (tn < ta.ntiles) {
-          v_next = force_tile_prepare(tile_info(tn, ta), tn, ta, cs, tile_list, SS[b ^ 1], status);
-          if (v_next)
-            stage_issue<MIXED, true>(tile_info(tn, ta), ta, pos, rows, ent, SS[b ^ 1], smem + (b ^ 1) * buf_bytes, L,
-                                     &bars[b ^ 1]);
-        }
-      }
-      if (v_cur) {
-        uint32_t& ph = b ? ph1 : ph0;
-        if (!stage_finish<MIXED, true>(tile_info(t, ta), ta, g, SS[b], smem + b * buf_bytes, L, &bars[b], ph,
-                                       !MIXED && HALF, status)) {
-          if (v_next) mbar_wait(&bars[b ^ 1], b ? ph0 : ph1, kWaitBudget);  // drain the other buffer's copies
-          return;
-        }
-        force_tile_compute<MIXED, LANES, HALF, ENERGY, false, LONGLIST>(SS[b], smem + b * buf_bytes, L, rows, ent, c, g,
-                                                                        fout, status, eacc, ta.list_cap);
+    uint32_t ph = 0;
+    for (int64_t t = blockIdx.x; t < ta.ntiles; t += gridDim.x) {
+      const TileInfo ti = tile_info(t, ta);
+      if (force_tile_prepare(ti, t, ta, cs, tile_list, S, status)) {
+        stage_issue<MIXED, true>(ti, ta, pos, rows, ent, S, smem, L, &bar);
+        if (!stage_finish<MIXED, true>(ti, ta, g, S, smem, L, &bar, ph, !MIXED && HALF, status)) return;
+        force_tile_compute<MIXED, LANES, HALF, ENERGY, false, LONGLIST>(S, smem, L, rows, ent, c, g, fout, status, eacc,
+                                                                        ta.list_cap);
       }
       __syncthreads();
-      if (pipelined) {
-        v_cur = v_next;
-        b ^= 1;
-      }
     }
   }
   if (ENERGY) {
@@ -881,14 +847,14 @@ constexpr int kDpThreads = 128;
 constexpr int kDpWarps = kDpThreads / 32;
 constexpr int kDpQueue = 288;  // queued pairs per warp: nine a lane (the smallest that keeps four FP64 CTAs per SM)
 
-template <class T, int NACC, bool DIRECT>
+template <int NACC, bool DIRECT>
 struct DpWarp {
-  T seg[32][NACC];       // per key: the partial sum of the lane in which its run begins
-  T head[32][NACC];      // per lane: the partial sum of a run begun in an earlier lane
+  double seg[32][NACC];       // per key: the partial sum of the lane in which its run begins
+  double head[32][NACC]; // per lane: the partial sum of a run begun in an earlier lane
   uint32_t q[kDpQueue];  // key of the warp's run << 16 | staged partner
 };
-template <class T, int NACC>
-struct DpWarp<T, NACC, true> {
+template <int NACC>
+struct DpWarp<NACC, true> {
   uint32_t q[kDpQueue];
 };
 
@@ -911,7 +877,7 @@ __host__ __device__ __forceinline__ DpLayout dp_layout(const TileArgs& ta) {
   D.L.ent = D.L.cnt = o;
   o += align16(2 * (size_t)ta.list_cap);
   D.warp = o;
-  o += sizeof(DpWarp<double, NACC, DIRECT>) * kDpWarps;
+  o += sizeof(DpWarp<NACC, DIRECT>) * kDpWarps;
   D.total = D.L.total = align16(o);
   return D;
 }
@@ -968,34 +934,32 @@ __device__ __forceinline__ bool dp_stage_finish(const TileInfo& ti, const TileAr
   return true;
 }
 
-// The listed pairs of a staged tile's keys inside r_c (or within the filter's margin of it), NW warps.
+// The listed pairs of a staged tile's keys inside r_c (or within the filter's margin of it).
 // sq: the staged records; W: the warp's queue.  key(o) loads what a pair needs of own key o, partner(slot)
 // what it needs of the partner (a pair ahead of its use), pair(key, partner, acc) adds one pair to the key's
-// NACC sums, done(o, acc) receives the sums of own key o, batch() is called by every lane after its share
-// of a queue.  ent_s: the staged part of the tile's segment, its first
-// cap entries; rows beyond it are read from ent_g.
+// NACC sums, done(o, acc) receives the sums of own key o.  ent_s: the staged part of the tile's segment, its
+// first cap entries; rows beyond it are read from ent_g.
 // DIRECT: done(o, acc) is called by the lanes themselves with each partial sum (it must add atomically).
-template <class T, int NACC, bool DIRECT, int NW, class Key, class Partner, class Pair, class Done, class Batch>
+template <int NACC, bool DIRECT, class Key, class Partner, class Pair, class Done>
 __device__ __forceinline__ void queue_tile_pairs(const TileShared& S, const uint4* sq, const uint2* s_rows,
-                                                 DpWarp<T, NACC, DIRECT>& W, const uint16_t* ent_s,
+                                                 DpWarp<NACC, DIRECT>& W, const uint16_t* ent_s,
                                                  const uint16_t* ent_g, unsigned cap, float cut2, int32_t* status,
-                                                 Key&& key, Partner&& partner, Pair&& pair, Done&& done,
-                                                 Batch&& batch) {
+                                                 Key&& key, Partner&& partner, Pair&& pair, Done&& done) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   s_rows += S.row_off;
   const int n_own = S.own1 - S.own0;
-  const int per = min(32, (n_own + NW - 1) / NW);  // keys per warp and turn
-  for (int b0 = warp * per; b0 < n_own; b0 += NW * per) {
+  const int per = min(32, (n_own + kDpWarps - 1) / kDpWarps);  // keys per warp and turn
+  for (int b0 = warp * per; b0 < n_own; b0 += kDpWarps * per) {
     const int nk = min(per, n_own - b0);
-    T tot[NACC];  // lane k: the sums of key b0 + k
+    double tot[NACC];  // lane k: the sums of key b0 + k
 #pragma unroll
-    for (int q = 0; q < NACC; ++q) tot[q] = T(0);
+    for (int q = 0; q < NACC; ++q) tot[q] = 0.0;
     int ka = 0, kb = 0, cnt = 0;  // lane k: the key's range of the queue; queued pairs
     auto drain = [&]() {
       __syncwarp();
       const int c = (cnt + 31) >> 5, lo = lane * c, hi = min(lo + c, cnt);
-      T acc[NACC];
+      double acc[NACC];
       int kc = -1;
       bool head = lo > 0 && lo < cnt && (W.q[lo - 1] >> 16) == (W.q[lo] >> 16);
       auto ki = key(b0);
@@ -1003,7 +967,7 @@ __device__ __forceinline__ void queue_tile_pairs(const TileShared& S, const uint
         if constexpr (DIRECT) {
           done(b0 + kc, acc);
         } else {
-          T* dst = head ? W.head[lane] : W.seg[kc];
+          double* dst = head ? W.head[lane] : W.seg[kc];
 #pragma unroll
           for (int q = 0; q < NACC; ++q) dst[q] = acc[q];
           head = false;
@@ -1020,14 +984,13 @@ __device__ __forceinline__ void queue_tile_pairs(const TileShared& S, const uint
           kc = k;
           ki = key(b0 + k);
 #pragma unroll
-          for (int q = 0; q < NACC; ++q) acc[q] = T(0);
+          for (int q = 0; q < NACC; ++q) acc[q] = 0.0;
         }
         pair(ki, pj, acc);
         w = wn;
         pj = pn;
       }
       if (kc >= 0) put();
-      batch();
       __syncwarp();
       if constexpr (!DIRECT) {
         if (kb > ka) {
@@ -1090,10 +1053,10 @@ __device__ __forceinline__ void dp_tile_pairs(const TileShared& S, const unsigne
                                               const uint16_t* ent_g, unsigned cap, float cut2, int32_t* status,
                                               Pair&& pair, Done&& done) {
   const dvec4* sp = (const dvec4*)(smem + D.L.pos) + S.own0;
-  queue_tile_pairs<double, NACC, DIRECT, kDpWarps>(
+  queue_tile_pairs<NACC, DIRECT>(
       S, (const uint4*)(smem + D.xq), (const uint2*)(smem + D.L.rows),
-      ((DpWarp<double, NACC, DIRECT>*)(smem + D.warp))[threadIdx.x >> 5], (const uint16_t*)(smem + D.L.ent), ent_g, cap,
-      cut2, status, [&](int o) { return sp[o]; }, [](int j) { return j; }, pair, done, [] {});
+      ((DpWarp<NACC, DIRECT>*)(smem + D.warp))[threadIdx.x >> 5], (const uint16_t*)(smem + D.L.ent), ent_g, cap,
+      cut2, status, [&](int o) { return sp[o]; }, [](int j) { return j; }, pair, done);
 }
 
 // The FP64 comparison r^2 < r_c^2 of two non-negative values by their bit patterns (the order is the
