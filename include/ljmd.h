@@ -345,8 +345,10 @@ int ljmd_get_profile(ljmd_sys* sys, ljmd_profile* out);
  * arithmetic; for the mixed form this is the pipelined kernel, in which producer
  * warps stage tiles into two to four buffers and consumer warps compute, and it is the default there;
  * 1 is the default otherwise, and the FP64 form always uses one).  A new tile_cells or force_buffers
- * takes effect at the next list construction (forced at the next force evaluation).  Results
- * do not depend on these knobs beyond FP32 summation order.
+ * takes effect at the next list construction (forced at the next force evaluation).  lanes,
+ * force_ctas_per_sm and force_buffers have no effect on the steps of a box whose tiles all fit on the chip
+ * (ljmd_step takes them in one launch, with threads per key by the tile's size), only on its single force
+ * evaluations.  Results do not depend on these knobs beyond FP32 summation order.
  */
 int ljmd_set_tuning(ljmd_sys* sys, int32_t tile_cells, int32_t lanes, int32_t force_ctas_per_sm,
                     int32_t force_buffers);

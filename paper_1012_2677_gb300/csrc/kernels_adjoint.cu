@@ -1,7 +1,7 @@
 // Element-wise kernels of the reverse-time (adjoint) pass through velocity-Verlet: moving adjoint
 // vectors between the caller's id order and the library's cell-sorted order, the unwrapped
 // trajectory state, and the vector updates of the recurrences.  The pair work (Hessian-vector
-// product, forces and parameter derivatives) is the adjoint tile kernel of kernels_tile.cu.
+// product, forces and parameter derivatives) is in the kernels of kernels_adjoint_tile.cu.
 #include "common.cuh"
 
 namespace ljmd {

@@ -483,11 +483,6 @@ static int ensure_tile_list(ljmd_sys* s) {
   return LJ_OK;
 }
 
-// Tile geometry for the staged list/force kernels: T cells along z per tile, shared-memory
-// capacities from the actual largest tile of the current cell occupancy.
-// Tile buffers per force CTA: the requested number, else two for the form with a pipelined
-// kernel (producer warps stage the next tiles while consumer warps compute): the mixed form; one
-// otherwise.
 // Multiprocessors of a device (152 if the attribute cannot be read).
 static int sm_count_of(int dev) {
   int sms = 0;
@@ -498,11 +493,13 @@ static int sm_count_of(int dev) {
   return sms;
 }
 
+// Tile buffers per force CTA, 1 or 2 (as many as fit): one in the FP64 form; in the mixed form the requested
+// number, else two (the pipelined kernel: producer warps stage the next tiles while consumer warps compute).
 static int force_buffers(const ljmd_sys* s) {
   if (s->precision != LJ_MIXED) return 1;
   if (s->force_nbuf) return s->force_nbuf;
-  // fewer tiles than two per SM: the single-buffer kernel (the pipelined one holds one CTA per SM
-  // with two producer warps)
+  // fewer tiles than two per SM: the single-buffer kernel (the pipelined one runs one CTA per SM, whose
+  // producers and consumers would each have a tile or two)
   if (s->ta.ntiles > 0 && s->ta.ntiles < 2 * (int64_t)sm_count_of(s->device)) return 1;
   return 2;
 }
@@ -549,6 +546,8 @@ static void tile_shape(TileArgs& ta, int T) {
   ta.ntiles = (int64_t)n * n * ta.ntz;
 }
 
+// Tile geometry for the staged list/force kernels: T cells along z per tile (t_cap at most), shared-memory
+// capacities from the actual largest tile of the current cell occupancy.
 static int choose_tiles(ljmd_sys* s, int t_cap) {
   ljmd_sys* sys = s;
   TileArgs& ta = s->ta;

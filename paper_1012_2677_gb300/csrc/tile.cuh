@@ -114,8 +114,8 @@ __device__ __forceinline__ bool stage_offsets(const TileInfo& ti, const TileArgs
   return S.total <= ta.max_staged;
 }
 
-// Staging descriptor of a tile, kTileDesc words of 8 bytes written by the list kernel (behind the tiles'
-// list segments: tile_list + ntiles) and read by the pipelined force kernel, one word per lane, so that
+// Staging descriptor of a tile, kTileDesc words of 8 bytes written by the list kernel where the pipelined force
+// kernel follows (behind the tiles' list segments: tile_list + ntiles), which reads one word per lane, so that
 // staging a tile takes no bookkeeping at all in the ten or so steps of a list's life:
 //   0..17  run 2 k + r of column k: first sorted index; staged slot << 16 | particles (a column is one
 //          run, or two where z wraps)
