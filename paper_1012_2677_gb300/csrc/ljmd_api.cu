@@ -1040,19 +1040,21 @@ static int device_run(ljmd_sys* s, double dt, bool first_of_call, int64_t remain
   return LJ_OK;
 }
 
-// Energy partials for a run of K steps, no more: allocating a megabyte takes 30 us, and the first step of 4,000
-// particles on a new handle, list construction included, 100.  False: no memory.
-static bool ensure_records(ljmd_sys* s, int K) {
-  if (s->prm.energy_every <= 0) return true;
-  int64_t slots = 2;
-  while (slots < K + 1) slots *= 2;
-  const int64_t want = 3 * slots * s->ta.ntiles;
-  if (s->res_rec_cap < want) {
+// Energy records (a state each) that a resident run of K steps may take, 0 if there is no memory.  They are made
+// for the life of a list as last seen, and more as this one lives longer (a run that has fewer ends early and
+// another follows), not for the longest run at once: a few hundred kilobytes more start a new block of the allocator, which took the first step of
+// 4,000 particles on a new handle, list construction included, from 100 to 195 us.
+static int64_t resident_records(ljmd_sys* s, int K) {
+  if (s->prm.energy_every <= 0) return K + 1;
+  const int64_t age = s->steps - s->last_build_step;
+  const int64_t life =
+      std::min<int64_t>(std::max(s->lifetime_est + s->lifetime_est / 4, 2 * age), kResidentSteps - 1) + 2;
+  if (s->res_rec_cap < 3 * std::min<int64_t>(K + 1, life) * s->ta.ntiles) {
     s->res_rec_cap = 0;
-    if (dalloc_t(s, &s->res_rec, (size_t)want) != LJ_OK) return false;
-    s->res_rec_cap = want;
+    if (dalloc_t(s, &s->res_rec, (size_t)(3 * life * s->ta.ntiles)) != LJ_OK) return 0;
+    s->res_rec_cap = 3 * life * s->ta.ntiles;
   }
-  return true;
+  return s->res_rec_cap / (3 * s->ta.ntiles);
 }
 
 // Up to `remaining` steps as one resident run (kernels_resident.cu), with the final half kick of the
@@ -1064,9 +1066,11 @@ static int resident_run(ljmd_sys* s, double dt, bool first_of_call, int64_t rema
   cudaStream_t st = s->st;
   const int ee = s->prm.energy_every;
   auto want_energy = [&](int64_t t) { return ee > 0 && (t % ee) == 0; };
-  const int K = (int)std::min<int64_t>(remaining, kResidentSteps);
+  int K = (int)std::min<int64_t>(remaining, kResidentSteps);
   *launched = false;
-  if (!ensure_records(s, K)) return LJ_OK;
+  const int64_t records = resident_records(s, K);
+  if (records == 0) return LJ_OK;
+  K = (int)std::min<int64_t>(K, records - 1);
   ResidentCtl* hc = s->h_res;
   const size_t head = offsetof(ResidentCtl, dmax);
   memset(hc, 0, head + sizeof(hc->dmax[0]) * (size_t)K);
