@@ -134,18 +134,23 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-def source_sha(path):
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+def source_sha(paths):
+    h = hashlib.sha256()
+    for path in paths:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_force_pipe_fcc1m_rho0.5.md")
-FORCE_SOURCE = os.path.join(ROOT, "paper_1012_2677_gb300", "csrc", "force_launch.cuh")
+# the kernel and its launch, the tile layout and pair arithmetic, the buffers and staged share of the list
+FORCE_SOURCES = [os.path.join(ROOT, "paper_1012_2677_gb300", "csrc", f)
+                 for f in ("force_launch.cuh", "tile.cuh", "kernels_force.cu")]
 
 
 def recorded_traffic(kernel_name, N):
     """DRAM bytes of one force launch at N particles, scaled by N from the per-particle traffic in
-    the committed ncu summary of a smaller case of the same kernel, if the kernel source is
+    the committed ncu summary of a smaller case of the same kernel, if the kernel's sources are
     unchanged since the counters were taken (else None).  The summary's lines 'key: value'
     give kernel, source_sha and dram_bytes_per_particle."""
     rec = {}
@@ -157,7 +162,7 @@ def recorded_traffic(kernel_name, N):
                     rec[k.strip().strip("`")] = v.strip().strip("`")
     except OSError:
         return None
-    if rec.get("source_sha") != source_sha(FORCE_SOURCE) or rec.get("kernel") != kernel_name:
+    if rec.get("source_sha") != source_sha(FORCE_SOURCES) or rec.get("kernel") != kernel_name:
         return None
     try:
         return round(float(rec["dram_bytes_per_particle"]) * N)
