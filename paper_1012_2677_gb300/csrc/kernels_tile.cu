@@ -293,14 +293,15 @@ size_t list_smem_bytes(const TileArgs& ta, int precision) {
   return tile_layout(ta, precision == LJ_MIXED, false).total;
 }
 
-template <bool HALF, bool BATCHED, int NT>
+// DESC: the pipelined force kernel follows, so its staging descriptors are written.
+template <bool HALF, bool BATCHED, bool DESC, int NT>
 __global__ void __launch_bounds__(NT, kWinCtas)
     k_list_win(const float4* __restrict__ pos, const double* __restrict__ x, const uint32_t* __restrict__ cs_in,
                int64_t N, Geom g_in, TileArgs ta_in, ListBand band, uint2* __restrict__ rows,
                uint2* __restrict__ tile_list, uint16_t* __restrict__ ent, uint64_t cap,
                unsigned long long* __restrict__ counter, unsigned int* __restrict__ max_list,
                int32_t* __restrict__ status, const ReplicaGeo* __restrict__ reps, int R,
-               const int* __restrict__ pred, const int32_t* __restrict__ tile_rep, uint2* __restrict__ desc) {
+               const int* __restrict__ pred, const int32_t* __restrict__ tile_rep) {
   static_assert(NT >= 64, "warp 0 prepares the next tile while the others count");
   if (pred && !*pred) return;  // predicated (batched rebuild inside a graph)
   extern __shared__ __align__(16) unsigned char smem[];
@@ -375,8 +376,8 @@ __global__ void __launch_bounds__(NT, kWinCtas)
         if (t + 2 * (int64_t)gridDim.x < ta_in.ntiles) prefetch(t + 2 * (int64_t)gridDim.x);
       }
     };
-    if (desc && warp == kNW - 1)  // the pipelined force kernel's staging descriptor
-      tile_desc_write(ti, ta.n, g.Lq, S, s_ready[buf] != 0, desc + kTileDesc * t, lane);
+    if (DESC && warp == kNW - 1)  // the pipelined force kernel's staging descriptor
+      tile_desc_write(ti, ta.n, g.Lq, S, s_ready[buf] != 0, tile_list + ta_in.ntiles + kTileDesc * t, lane);
     if (!s_ready[buf]) {  // sizing inconsistency: record and skip the tile
       if (threadIdx.x == 0) atomicOr(status, LJ_ST_CELL_RANGE);
       if (warp == 0) prepare_next();
@@ -650,17 +651,21 @@ void launch_list_tile(int precision, int half, const void* pos, const float4* hi
                       uint64_t cap, unsigned long long* counter, unsigned int* max_list, int32_t* status,
                       cudaStream_t s, const int* pred, bool descriptors) {
   const size_t sm = list_smem_bytes(ta, precision);
-  uint2* desc = descriptors ? tile_list + ta.ntiles : nullptr;
-  int grid = tile_grid(ta, per_sm_for(sm));
-  if (!ta.whole) {  // the window kernel: as many CTAs as are resident
-    set_smem(k_list_win<false, false, kWinThreads>, sm);
-    grid = tile_grid(ta, resident_per_sm(k_list_win<false, false, kWinThreads>, kWinThreads, sm));
-  }
+  const int grid = tile_grid(ta, per_sm_for(sm));
 #define LJ_LIST_LAUNCH(M, H, W)                                                                                 \
   do {                                                                                                          \
     set_smem(k_list_tile<M, H, W>, sm);                                                                         \
     k_list_tile<M, H, W><<<grid, kTileThreads, sm, s>>>(pos, x, cs, N, g, ta, band, rows, tile_list, ent, cap, \
                                                         counter, max_list, status);                             \
+  } while (0)
+// tiles, either form: one thread per key on the hi copies (the list is the same), as many CTAs as are resident
+#define LJ_WIN_LAUNCH(H, D)                                                                                     \
+  do {                                                                                                          \
+    set_smem(k_list_win<H, false, D, kWinThreads>, sm);                                                         \
+    const int wgrid = tile_grid(ta, resident_per_sm(k_list_win<H, false, D, kWinThreads>, kWinThreads, sm));    \
+    k_list_win<H, false, D, kWinThreads><<<wgrid, kWinThreads, sm, s>>>(                                        \
+        hi, x, cs, N, g, ta, band, rows, tile_list, ent, cap, counter, max_list, status, nullptr, 0, pred,      \
+        nullptr);                                                                                               \
   } while (0)
   const bool mixed = precision == LJ_MIXED;
   if (ta.whole) {
@@ -671,18 +676,15 @@ void launch_list_tile(int precision, int half, const void* pos, const float4* hi
       if (half) LJ_LIST_LAUNCH(false, true, true);
       else LJ_LIST_LAUNCH(false, false, true);
     }
-  } else if (half) {  // tiles, either form: one thread per key on the hi copies (the list is the same)
-    set_smem(k_list_win<true, false, kWinThreads>, sm);
-    k_list_win<true, false, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, ta, band, rows, tile_list, ent,
-                                                                       cap, counter, max_list, status, nullptr, 0,
-                                                                       pred, nullptr, desc);
+  } else if (half) {
+    if (descriptors) LJ_WIN_LAUNCH(true, true);
+    else LJ_WIN_LAUNCH(true, false);
   } else {
-    set_smem(k_list_win<false, false, kWinThreads>, sm);
-    k_list_win<false, false, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, ta, band, rows, tile_list, ent,
-                                                                        cap, counter, max_list, status, nullptr, 0,
-                                                                        pred, nullptr, desc);
+    if (descriptors) LJ_WIN_LAUNCH(false, true);
+    else LJ_WIN_LAUNCH(false, false);
   }
 #undef LJ_LIST_LAUNCH
+#undef LJ_WIN_LAUNCH
 }
 
 void launch_list_decode(const uint32_t* cs, int64_t N, TileArgs ta, const uint2* rows, const uint16_t* ent,
@@ -766,11 +768,11 @@ void launch_list_batch(const float4* hi, const double* x, const uint32_t* cs, in
                        unsigned long long* counter, unsigned int* max_list, int32_t* status, const ReplicaGeo* reps,
                        int R, const int32_t* tile_rep, const int* pred, cudaStream_t s) {
   const size_t sm = win_layout(caps).total;
-  set_smem(k_list_win<false, true, kWinThreads>, sm);
-  const int grid = tile_grid(caps, resident_per_sm(k_list_win<false, true, kWinThreads>, kWinThreads, sm));
-  k_list_win<false, true, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, caps, band, rows, tile_list, ent,
+  set_smem(k_list_win<false, true, true, kWinThreads>, sm);
+  const int grid = tile_grid(caps, resident_per_sm(k_list_win<false, true, true, kWinThreads>, kWinThreads, sm));
+  k_list_win<false, true, true, kWinThreads><<<grid, kWinThreads, sm, s>>>(hi, x, cs, N, g, caps, band, rows, tile_list, ent,
                                                                      cap, counter, max_list, status, reps, R, pred,
-                                                                     tile_rep, tile_list + caps.ntiles);
+                                                                     tile_rep);
 }
 
 // ---- list validity: the large displacement check (LDC) of Alg. 2 -----------------------------
