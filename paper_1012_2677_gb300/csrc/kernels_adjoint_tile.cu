@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kDpThreads, 3)
       if (!dp_stage_finish(ti, ta, g, S, smem, D, &bar, ph, status)) return;
       queue_tile_pairs<NACC, false>(
           S, sq, (const uint2*)(smem + D.L.rows), ((DpWarp<NACC, false>*)(smem + D.warp))[threadIdx.x >> 5],
-          (const uint16_t*)(smem + D.L.ent), ent + S.list_base, (unsigned)ta.list_cap, c.rc2w, status,
+          (const uint16_t*)(smem + D.L.ent), ent + S.list_base, (unsigned)ta.list_cap, filter_cut2(c), status,
           [&](int o) { return Key{sp[S.own0 + o], w[S.gown0 + o]}; }, [&](int j) { return Key{sp[j], w[sq[j].w]}; },
           [&](const Key& k, const Key& j, double* acc) {
             const dvec4 &qj = j.x, &wj = j.w;

@@ -329,13 +329,6 @@ static int setup_geometry(ljmd_sys* s, double L) {
   c.f8c2q = ldexpf(c.f8c2, -g.qk);
   c.sig2q = ldexpf(c.sig2f, 2 * g.qk);
   c.rc2q = ldexpf(c.rc2f, 2 * g.qk);
-  // A distance between fixed-point copies is within sqrt(3) u of the true one (each coordinate is rounded by
-  // at most u / 2), and its FP32 square within a relative 4e-7.  The absolute term counts where u is not small
-  // against r_c: lengths far below one unit (u is 2^-30 at least) and cells far longer than r_c.
-  {
-    const double rq = ldexp(p.cutoff, g.qk) + 2.0;
-    c.rc2w = (float)(rq * rq * (1.0 + 4e-6));
-  }
   c.c2q = ldexpf(c.c2f, -2 * g.qk);
 
   // FP32 list filter on hi parts: each hi difference is exact and differs from the exact

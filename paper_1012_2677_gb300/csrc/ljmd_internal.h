@@ -56,7 +56,6 @@ struct LJConst {
   // FP32 constants above with their exponents shifted (no extra rounding); the virial comes out
   // in units of 1/u and is multiplied by u (exactly) when it is summed.
   float f24q, f48q, f8c2q, sig2q, rc2q, c2q;
-  float rc2w;  // r_c^2 in units of u^2, widened by what the filter of the FP64 form's queues can err
   // the adjoint kernel's constants: 1 / sigma and c2 / sigma^2, FP64 and FP32
   double inv_sigma, c2s;
   float inv_sigmaf, c2sf;

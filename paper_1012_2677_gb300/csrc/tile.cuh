@@ -835,7 +835,7 @@ __global__ void __launch_bounds__(kTileThreads, 4)
 // ---------------------------------------------------------------------------------------------
 // Pair work by queues.  A warp takes a run of consecutive keys.  It first filters their rows in FP32
 // (differences of fixed-point copies, r_c^2 widened by what the copies' rounding, an absolute u each, and
-// the FP32 arithmetic can err: LJConst::rc2w) and queues the kept (key, partner) pairs in shared memory;
+// the FP32 arithmetic can err: filter_cut2) and queues the kept (key, partner) pairs in shared memory;
 // then each lane evaluates a contiguous share of the queue, so that at most the last pair of a lane
 // idles and a key's sum needs no shuffles.  A lane stores the partial sum of a key that began in an earlier
 // lane in its head slot, every other one in the key's slot; the key's own lane adds slot and heads in
@@ -1075,6 +1075,15 @@ __device__ __forceinline__ double rcp_cubic64(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
+// r_c^2 for the queues' filter, in units of u^2: a distance between fixed-point copies is within sqrt(3) u of the
+// true one (each coordinate is rounded by at most u / 2), and its FP32 square and this figure within a relative
+// 1e-6.  The absolute term counts where u is not small against r_c: lengths far below one unit (u is 2^-30 at
+// least) and cells far longer than r_c.
+__device__ __forceinline__ float filter_cut2(const LJConst& c) {
+  const float r = sqrtf(c.rc2q) + 2.0f;
+  return r * r * 1.000004f;
+}
+
 // One pair of the FP64 form's force, its sums over pairs (r^-6, r^-12, r^2 and their number, from which
 // the energies come) and the scattered sums of the half list.
 template <bool HALF, bool ENERGY>
@@ -1092,7 +1101,7 @@ struct DpForce {
     f8c2 = 8.0 * c.eps * c.c2s;
     f24s = 24.0 * c.eps * sig6;
     f48s = 48.0 * c.eps * sig6 * sig6;
-    cut2 = c.rc2w;
+    cut2 = filter_cut2(c);
     sp = (const dvec4*)(smem + D.L.pos);
     sq = (const uint4*)(smem + D.xq);
     fout = f;
